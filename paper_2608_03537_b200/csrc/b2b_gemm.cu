@@ -142,7 +142,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       RingPos<RING> ring;
       bool ok = true;
       // one box into the current slot (a pair operand: signals the even CTA's full barrier)
@@ -202,7 +202,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // implies the slot's PREVIOUS fill has landed and been consumed (else the parity test passes on the older phase):
     // here the scores of sub-tile k+1 wait for pfree(k) first, which lies behind S.V of sub-tile k-2 (the previous tenant
     // of their first slot); the other three slots' previous tenants are this lane's own.
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       constexpr uint32_t idesc_ml1 = make_idesc_bf16(256, 128, false, !KM);
       RingPos<RING> ring;
       bool ok = true;
@@ -269,7 +269,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else if (warp == kMl2Warp) {
     // ------------------------------------------------------------------------------------------ S.V UMMAs (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       constexpr uint32_t idesc_ml2 = make_idesc_bf16(256, 128, false, true);
       RingPos<RING> ring;
       bool ok = true;

@@ -221,7 +221,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
   // the barrier's latest one: the next phase belongs to the UMMAs that need the very load being issued.)
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       int xi = 0;  // next X tile of this cluster to fetch
       // X of the cluster's xi-th tile into buffer xi & 1 (this CTA's 128 rows, two K blocks); false = buffer still in use
@@ -277,7 +277,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ ML1 lane (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       constexpr uint32_t idesc = make_idesc_bf16(256, 128, false, true);
       int j1 = 0, t1 = 0;  // chunk-in-tile, tile
       for (int c = 0; c < total; ++c) {
@@ -307,7 +307,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
     }
   } else if (warp == kMl2Warp) {
     // ------------------------------------------------------------------------------------------ ML2 lane (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       constexpr uint32_t idesc = make_idesc_bf16(256, 128, false, true);
       int j2 = 0, t2 = 0;
       for (int c = 0; c < total; ++c) {

@@ -140,7 +140,7 @@ b2b_stream_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       RingPos<kStages> ring;
       bool ok = true;
       auto next_stage = [&](uint32_t& sa, uint32_t& full, uint32_t bytes) {
@@ -190,7 +190,7 @@ b2b_stream_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ UMMA issuer (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       constexpr uint32_t idesc_ml1 = make_idesc_bf16(256, 256, false, true);
       constexpr uint32_t idesc_ml2 = make_idesc_bf16(256, 128, false, true);
       RingPos<kStages> ring;

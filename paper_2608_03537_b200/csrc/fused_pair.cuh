@@ -236,7 +236,7 @@ fused_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       RingPos<NSTAGES> ring;
       bool ok = true;
       // A stage is handed back by the UMMA commit (K-block use) or by the eight epilogue warps (residual use); the two
@@ -281,8 +281,7 @@ fused_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             auto load_b_half = [&](uint32_t dst, int first_group, int width) {
               for (int j = 0; j < width / 128; ++j) {
                 const int col = group_col(ncta0, first_group + static_cast<int>(pm) * (width / 128) + j);
-                if (p.b_nk) tma_load_3d_pair(dst + j * 8192, &tmB, full, kb * 64, col, b);
-                else tma_load_3d_pair(dst + j * 8192, &tmB, full, col, kb * 64, b);
+                tma_load_3d_pair(dst + j * 8192, &tmB, full, p.b_nk ? kb * 64 : col, p.b_nk ? col : kb * 64, b);
               }
             };
             if (LOCK) {
@@ -313,7 +312,7 @@ fused_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ UMMA issuer (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       RingPos<NSTAGES> ring;
       uint32_t full_bits = 0;     // per-stage phase of bar_full (a stage is not a K-block stage on every lap)
       uint32_t slot_uses[2] = {0, 0};

@@ -39,6 +39,17 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   return r;
 }
 
+// One lane of a converged warp.  TMA copies, UMMAs and commits take uniform registers: behind `lane == 0` the compiler does
+// not know that one thread is left and issues them as for a divergent warp, behind elect.sync it does.  Measured (every
+// producer and UMMA issuer of the library, before / after): self-attention 256 x 512 x 512 46.3 / 44.1 us, 32 x 4096 queries
+// of 256 keys 25.2 / 24.9, 8192 x 4096 x 4096 with GELU + RMSNorm 243.9 / 238.0.  A loop over boxes that does not unroll, or a
+// branch per box, costs more than that: a producer of two 8 KB boxes per stage went from 392 to 206 clocks a stage without.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

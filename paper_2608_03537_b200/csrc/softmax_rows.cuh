@@ -143,7 +143,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -178,7 +178,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ UMMA issuer (even CTA)
-    if (lane == 0 && pm == 0) {
+    if (pm == 0 && elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       uint32_t slot_uses[2] = {0, 0};
