@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "b2b_params.h"
+#include "few_rows.h"
 #include "host_common.h"
 #include "row_params.h"
 
@@ -75,12 +76,18 @@ bool programmatic_launch_enabled() {
   return on;
 }
 
-int split_row_block(int epi, int N, int K, long long row_pairs) {
-  // COMFUSE_SPLIT_BLOCK=<width> forces the two-kernel form with that block width where N is a multiple of it (0 = never)
+// COMFUSE_SPLIT_BLOCK=<width> forces the tile kernel, in the two-kernel form with that block width where N is a multiple of
+// it (0 = never)
+static int forced_split_block() {
   static const int forced = [] {
     const char* e = std::getenv("COMFUSE_SPLIT_BLOCK");
     return e ? std::atoi(e) : -1;
   }();
+  return forced;
+}
+
+int split_row_block(int epi, int N, int K, long long row_pairs) {
+  const int forced = forced_split_block();
   if (forced >= 0) return (forced > 0 && N > forced && N % forced == 0) ? forced : 0;
   // Measured (8192 rows; on-chip / two kernels with 256-column blocks, us): N = 4096: K = 4096 242 / 212, K = 1024 101 / 87,
   // K = 256 64 / 62 (LayerNorm 57 / 66); N = 2048: K = 4096 147 / 118, K = 1024 59 / 55; N = 1024, K = 4096: 55 / 69.
@@ -218,14 +225,17 @@ comfuse_status_t validate_gemm_desc(const comfuse_gemm_desc_t* d) {
   return COMFUSE_OK;
 }
 
+// Pairs of 128-row blocks that a call's form is chosen for (see gemm_epilogue_rows: `form_rows`).
+long long form_row_pairs(const comfuse_gemm_desc_t* d, int form_rows) { return static_cast<long long>(d->batch) * ((static_cast<long long>(form_rows) + 255) / 256); }
+
 // Does a fused instantiation exist for this description?  `on_chip_only`: without the two-kernel form.
-comfuse_status_t fused_supported(const comfuse_gemm_desc_t* d, bool on_chip_only = false) {
+comfuse_status_t fused_supported(const comfuse_gemm_desc_t* d, int form_rows, bool on_chip_only = false) {
   FusedParams p = {};
   p.b_nk = (d->flags & COMFUSE_FLAG_B_ROW_MAJOR_NK) ? 1 : 0;
   p.M = d->M;
   p.N = d->N;
   p.K = d->K;
-  p.wide_block = on_chip_only ? 0 : wide_row_block(kind_to_epi(d->kind), d->N, d->K, static_cast<long long>(d->batch) * ((d->M + 255) / 256));
+  p.wide_block = on_chip_only ? 0 : wide_row_block(kind_to_epi(d->kind), d->N, d->K, form_row_pairs(d, form_rows));
   p.wide = p.wide_block > 0;
   GemmMaps dummy;
   std::memset(&dummy, 0, sizeof(dummy));
@@ -237,6 +247,48 @@ comfuse_status_t fused_supported(const comfuse_gemm_desc_t* d, bool on_chip_only
     default: break;
   }
   return e == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_UNSUPPORTED;
+}
+
+// The few-rows form (few_rows.cu), with the finishing kernel behind its two-kernel variant.
+comfuse_status_t run_few_rows(const FewRowsPlan& plan, int epi, const comfuse_gemm_desc_t& d, const comfuse_epilogue_args_t& a, const void* A,
+                              const void* B, void* Y, float2* partials, const DeviceInfo& dev, cudaStream_t st, int form_rows) {
+  const bool b_nk = (d.flags & COMFUSE_FLAG_B_ROW_MAJOR_NK) != 0;
+  auto bs = [&](long long given, long long rows, long long ld) { return static_cast<uint64_t>(d.batch > 1 ? given : rows * ld) * 2; };
+  CUtensorMap tmW, tmX;
+  if (!encode_tmap_bf16_3d(&tmX, A, d.K, d.M, d.batch, static_cast<uint64_t>(d.lda) * 2, bs(d.batch_stride_a, d.M, d.lda), plan.mt) ||
+      !encode_tmap_bf16_3d(&tmW, B, b_nk ? d.K : d.N, b_nk ? d.N : d.K, d.batch, static_cast<uint64_t>(d.ldb) * 2,
+                           bs(d.batch_stride_b, b_nk ? d.N : d.K, d.ldb), 64))
+    return COMFUSE_ERR_CUDA;
+  FewRowsParams p = {};
+  p.M = d.M; p.N = d.N; p.K = d.K; p.batch = d.batch;
+  p.alpha = d.alpha; p.eps = d.eps;
+  p.b_nk = b_nk ? 1 : 0;
+  p.wide = plan.wide ? 1 : 0;
+  p.post_relu = (d.flags & COMFUSE_FLAG_POST_RELU) ? 1 : 0;
+  p.no_activation = (d.flags & COMFUSE_FLAG_NO_ACTIVATION) ? 1 : 0;
+  p.bias = static_cast<const uint16_t*>(a.bias);
+  p.gamma = static_cast<const uint16_t*>(a.gamma);
+  p.beta = static_cast<const uint16_t*>(a.beta);
+  p.residual = static_cast<const uint16_t*>(a.residual);
+  p.ldr = d.ldr; p.batch_stride_r = d.batch > 1 ? d.batch_stride_r : 0;
+  p.Y = static_cast<uint16_t*>(Y);
+  p.ldy = d.ldy; p.batch_stride_y = d.batch > 1 ? d.batch_stride_y : 0;
+  p.row_max = a.row_max; p.row_argmax = a.row_argmax;
+  p.wide_partials = plan.wide ? partials : nullptr;
+  p.status = dev.status_word;
+  p.timeout_ns = timeout_ns();
+  cudaError_t e = launch_few_rows(epi, plan, tmW, tmX, p, st);
+  if (e == cudaSuccess && plan.wide) {
+    RowParams r = {};
+    r.batch = d.batch; r.M = d.M; r.N = d.N;
+    r.gamma = p.gamma; r.beta = p.beta;
+    r.eps = d.eps;
+    r.post_relu = p.post_relu;
+    r.Y = p.Y; r.ldy = p.ldy; r.batch_stride_y = p.batch_stride_y;
+    r.row_max = a.row_max; r.row_argmax = a.row_argmax;
+    e = launch_wide_row_finish(epi, r, partials, plan.nblocks, 256, static_cast<long long>(d.batch) * form_rows, st);
+  }
+  return e == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
 }
 
 }  // namespace
@@ -344,38 +396,14 @@ comfuse_status_t prepare_compiled_program(int N, const StageProgram& prog) {
   return launch_compiled_program(maps, p, nullptr, false, false) == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_UNSUPPORTED;
 }
 
-}  // namespace comfuse
-
-using namespace comfuse;
-
-extern "C" {
-
-const char* comfuse_status_string(comfuse_status_t s) {
-  switch (s) {
-    case COMFUSE_OK: return "ok";
-    case COMFUSE_ERR_INVALID_ARG: return "invalid argument";
-    case COMFUSE_ERR_UNSUPPORTED: return "unsupported shape or op list for the fused path";
-    case COMFUSE_ERR_ALIGNMENT: return "pointer or leading dimension not aligned";
-    case COMFUSE_ERR_WORKSPACE: return "workspace missing or too small";
-    case COMFUSE_ERR_ARCH: return "device is not compute capability 10.x";
-    case COMFUSE_ERR_CUDA: return "CUDA call failed";
-    case COMFUSE_ERR_TIMEOUT: return "bounded device-side wait expired";
-    case COMFUSE_ERR_BOUNDS: return "a bounds predicate of the checked build failed (access skipped)";
-    default: return "unknown status";
-  }
-}
-
-uint64_t comfuse_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
-
-comfuse_status_t comfuse_workspace_size(const comfuse_gemm_desc_t* desc, size_t* bytes) {
-  if (!bytes) return COMFUSE_ERR_INVALID_ARG;
+static comfuse_status_t workspace_need(const comfuse_gemm_desc_t* desc, int form_rows, size_t* bytes) {
   comfuse_status_t s = validate_gemm_desc(desc);
   if (s != COMFUSE_OK) return s;
   if (desc->fused) {
-    s = fused_supported(desc);
+    s = fused_supported(desc, form_rows);
     if (s != COMFUSE_OK) return s;
     // rows wider than one cluster: one partial statistic (8 bytes) per row and 4096-column block
-    *bytes = static_cast<size_t>(wide_row_blocks(kind_to_epi(desc->kind), desc->N, desc->K, static_cast<long long>(desc->batch) * ((desc->M + 255) / 256))) *
+    *bytes = static_cast<size_t>(wide_row_blocks(kind_to_epi(desc->kind), desc->N, desc->K, form_row_pairs(desc, form_rows))) *
              desc->batch * desc->M * sizeof(float2);
   } else {
     if (desc->N > 8192) return COMFUSE_ERR_UNSUPPORTED;
@@ -384,9 +412,9 @@ comfuse_status_t comfuse_workspace_size(const comfuse_gemm_desc_t* desc, size_t*
   return COMFUSE_OK;
 }
 
-comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const void* A, const void* B, void* Y,
-                                       const comfuse_epilogue_args_t* args, void* workspace, size_t workspace_bytes,
-                                       void* cuda_stream) {
+comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void* A, const void* B, void* Y,
+                                    const comfuse_epilogue_args_t* args, void* workspace, size_t workspace_bytes,
+                                    void* cuda_stream, int form_rows) {
   comfuse_status_t s = validate_gemm_desc(desc);
   if (s != COMFUSE_OK) return s;
   if (!A || !B || !Y) return COMFUSE_ERR_INVALID_ARG;
@@ -405,11 +433,11 @@ comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const vo
     return COMFUSE_ERR_ALIGNMENT;
 
   size_t need = 0;
-  s = comfuse_workspace_size(desc, &need);
+  s = workspace_need(desc, form_rows, &need);
   if (s != COMFUSE_OK) return s;
   // For rows that fit a cluster (N <= 4096) the two-kernel form is an optimisation, not a need: a fused call that brings no
   // (or too small a) workspace keeps the row on chip instead of being refused.
-  const bool split_optional = desc->fused && desc->N <= kWideRowBlock && need > 0 && fused_supported(desc, true) == COMFUSE_OK;
+  const bool split_optional = desc->fused && desc->N <= kWideRowBlock && need > 0 && fused_supported(desc, form_rows, true) == COMFUSE_OK;
   const bool have_ws = workspace && workspace_bytes >= need && aligned16(workspace);
   if (split_optional && !have_ws) need = 0;
   if (need > 0 && (!workspace || workspace_bytes < need)) return COMFUSE_ERR_WORKSPACE;
@@ -423,6 +451,11 @@ comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const vo
   const long long bsr = desc->batch > 1 ? desc->batch_stride_r : 0;
   const long long bsy = desc->batch > 1 ? desc->batch_stride_y : 0;
   const bool b_nk = (desc->flags & COMFUSE_FLAG_B_ROW_MAJOR_NK) != 0;
+  if (desc->fused && forced_split_block() < 0) {
+    const int wide_block = need > 0 ? wide_row_block(epi, desc->N, desc->K, form_row_pairs(desc, form_rows)) : 0;
+    const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, *dev);
+    if (few.mt) return run_few_rows(few, epi, *desc, a, A, B, Y, static_cast<float2*>(workspace), *dev, st, form_rows);
+  }
   GemmMaps maps;
   if (desc->fused) {
     if (!make_gemm_maps(&maps, A, B, a.residual, Y, desc->batch, desc->M, desc->N, desc->K, desc->lda, desc->ldb, desc->ldr,
@@ -465,7 +498,7 @@ comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const vo
     p.ldy = desc->ldy; p.batch_stride_y = bsy;
     p.row_max = a.row_max; p.row_argmax = a.row_argmax;
     p.mask = desc->mask == COMFUSE_MASK_ADDITIVE ? static_cast<const uint16_t*>(a.mask) : nullptr;
-    const long long row_pairs = static_cast<long long>(desc->batch) * ((desc->M + 255) / 256);
+    const long long row_pairs = form_row_pairs(desc, form_rows);
     const int wide_blocks = need > 0 ? wide_row_blocks(epi, desc->N, desc->K, row_pairs) : 0;
     if (wide_blocks) {
       p.wide_block = wide_row_block(epi, desc->N, desc->K, row_pairs);  // first kernel: per-block stage 1, un-normalised x to Y, partial statistics to the workspace
@@ -490,7 +523,7 @@ comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const vo
       r.Y = static_cast<uint16_t*>(Y);
       r.ldy = desc->ldy; r.batch_stride_y = bsy;
       r.row_max = a.row_max; r.row_argmax = a.row_argmax;
-      e = launch_wide_row_finish(epi, r, p.wide_partials, wide_blocks, p.wide_block, st);
+      e = launch_wide_row_finish(epi, r, p.wide_partials, wide_blocks, p.wide_block, static_cast<long long>(desc->batch) * form_rows, st);
     }
     return e == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
   }
@@ -519,6 +552,40 @@ comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const vo
   r.row_max = a.row_max; r.row_argmax = a.row_argmax;
   e = launch_row_epilogue(epi, r, st);
   return e == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
+}
+
+}  // namespace comfuse
+
+using namespace comfuse;
+
+extern "C" {
+
+const char* comfuse_status_string(comfuse_status_t s) {
+  switch (s) {
+    case COMFUSE_OK: return "ok";
+    case COMFUSE_ERR_INVALID_ARG: return "invalid argument";
+    case COMFUSE_ERR_UNSUPPORTED: return "unsupported shape or op list for the fused path";
+    case COMFUSE_ERR_ALIGNMENT: return "pointer or leading dimension not aligned";
+    case COMFUSE_ERR_WORKSPACE: return "workspace missing or too small";
+    case COMFUSE_ERR_ARCH: return "device is not compute capability 10.x";
+    case COMFUSE_ERR_CUDA: return "CUDA call failed";
+    case COMFUSE_ERR_TIMEOUT: return "bounded device-side wait expired";
+    case COMFUSE_ERR_BOUNDS: return "a bounds predicate of the checked build failed (access skipped)";
+    default: return "unknown status";
+  }
+}
+
+uint64_t comfuse_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
+
+comfuse_status_t comfuse_workspace_size(const comfuse_gemm_desc_t* desc, size_t* bytes) {
+  if (!bytes) return COMFUSE_ERR_INVALID_ARG;
+  return workspace_need(desc, desc ? desc->M : 0, bytes);
+}
+
+comfuse_status_t comfuse_gemm_epilogue(const comfuse_gemm_desc_t* desc, const void* A, const void* B, void* Y,
+                                       const comfuse_epilogue_args_t* args, void* workspace, size_t workspace_bytes,
+                                       void* cuda_stream) {
+  return gemm_epilogue_rows(desc, A, B, Y, args, workspace, workspace_bytes, cuda_stream, desc ? desc->M : 0);
 }
 
 static comfuse_status_t validate_b2b_desc(const comfuse_b2b_desc_t* d) {

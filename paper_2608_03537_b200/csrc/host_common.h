@@ -96,6 +96,10 @@ cudaError_t launch_gemm_elementwise(const GemmMaps& maps, FusedParams p, cudaStr
 #include "comfuse.h"
 
 namespace comfuse {
+// comfuse_gemm_epilogue on some rows of a call of `form_rows` rows (per batch): every choice of kernel and split is the whole
+// call's, so that a call cut into row ranges gives the bits of the uncut one.
+comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void* A, const void* B, void* Y, const comfuse_epilogue_args_t* args,
+                                    void* workspace, size_t workspace_bytes, void* cuda_stream, int form_rows);
 // Y = stage program(A . B) with the on-chip interpreter (EPI_PROGRAM).  `vecs` = the up to three row-vector parameters
 // the program's CHO_ROWVEC operands index, `residual` = its full-tensor parameter or null.  `query_only`: just say
 // whether an instantiation exists for N (no device is touched).

@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "../../include/comfuse.h"
+#include "host_common.h"
 
 namespace {
 
@@ -189,7 +190,7 @@ extern "C" comfuse_status_t comfuse_gemm_epilogue_host(const comfuse_gemm_desc_t
       if (ac.row_max) ac.row_max += r0;
       if (ac.row_argmax) ac.row_argmax += r0;
       unsigned char* wsc = workspace ? static_cast<unsigned char*>(workspace) + static_cast<size_t>(r0) * ws_rows_bytes : nullptr;
-      s = comfuse_gemm_epilogue(&dc, sA + offA, dB, sY + offY, &ac, wsc, wsc ? workspace_bytes - static_cast<size_t>(r0) * ws_rows_bytes : 0, cuda_stream);
+      s = comfuse::gemm_epilogue_rows(&dc, sA + offA, dB, sY + offY, &ac, wsc, wsc ? workspace_bytes - static_cast<size_t>(r0) * ws_rows_bytes : 0, cuda_stream, desc->M);
       if (s != COMFUSE_OK) return rejoin(s);
       if (cudaEventRecord(pipe->computed[c], st) != cudaSuccess || cudaStreamWaitEvent(pipe->out, pipe->computed[c], 0) != cudaSuccess)
         return rejoin(COMFUSE_ERR_CUDA);

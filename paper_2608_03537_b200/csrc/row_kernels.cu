@@ -229,7 +229,9 @@ __device__ __forceinline__ void unpack8_f16(const uint4 q4, float (&xf)[8]) {
 
 template <int KIND>
 __global__ void __launch_bounds__(256) wide_row_finish_kernel(const RowParams p, const float2* partials, int nblocks, int block, long long rows) {
-  // launched with programmatic stream serialization: everything above this line may overlap the first kernel's tail
+  // launched with programmatic stream serialization: what stands above the wait may overlap the first kernel's tail, and the
+  // next call's set-up this kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31;
   // rows from the last to the first: the first kernel wrote them in rising order, so the blocks that start first read what
@@ -322,6 +324,95 @@ __global__ void __launch_bounds__(256) wide_row_finish_kernel(const RowParams p,
   }
 }
 
+// The same for FEW rows: a block per row.  A warp per row leaves most of the machine idle there and walks the row's 16-byte
+// pieces one round trip after another; with 256 threads a row of up to 4096 columns is two loads per thread, issued before
+// the statistics are merged.
+template <int KIND>
+__global__ void __launch_bounds__(256) wide_row_finish_block_kernel(const RowParams p, const float2* partials, int nblocks, int block) {
+  __shared__ float s_red[8];
+  __shared__ int s_idx[8];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next call's set-up may overlap this kernel
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const long long r = blockIdx.x;
+  const int b = static_cast<int>(r / p.M);
+  const int i = static_cast<int>(r - static_cast<long long>(b) * p.M);
+  uint16_t* y = p.Y + static_cast<long long>(b) * p.batch_stride_y + static_cast<long long>(i) * p.ldy;
+  const int lane = threadIdx.x & 31;
+  const int nvec = p.N >> 3;
+  constexpr int VPT = 2;
+  uint4 xq[VPT];
+#pragma unroll
+  for (int u = 0; u < VPT; ++u) {
+    const int vi = threadIdx.x + u * 256;
+    if (vi < nvec) xq[u] = __ldcs(reinterpret_cast<const uint4*>(y) + vi);
+  }
+  // every warp merges the row's partials on its own: lane k takes blocks k, k + 32, ...
+  const float2* q = partials + r * nblocks;
+  const int last = p.N - (nblocks - 1) * block;
+  auto partial = [&](int k, float& n) {
+    float2 o = q[k];
+    n = static_cast<float>(block);
+    if (KIND == EPI_LN && k == nblocks - 1 && last != block) {  // a partial last block: its statistic counts block - last zeros
+      const float s_all = n * o.x, sxx = o.y + n * o.x * o.x;
+      n = static_cast<float>(last);
+      o.x = s_all / n;
+      o.y = fmaxf(sxx - n * o.x * o.x, 0.f);
+    }
+    return o;
+  };
+  float s = 0.f, mu = 0.f, n;
+  for (int k = lane; k < nblocks; k += 32) {
+    const float2 o = partial(k, n);
+    s += KIND == EPI_LN ? n * o.x : o.x;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  if constexpr (KIND == EPI_LN) {
+    mu = s / static_cast<float>(p.N);
+    s = 0.f;
+    for (int k = lane; k < nblocks; k += 32) {
+      const float2 o = partial(k, n);
+      const float d = o.x - mu;
+      s += o.y + n * d * d;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  }
+  const float rstd = rsqrtf(s / static_cast<float>(p.N) + p.eps);
+  float best = -INFINITY;
+  int best_col = 0x7FFFFFFF;
+  const uint4 one = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+  for (int v0 = 0; v0 < nvec; v0 += 256 * VPT) {
+#pragma unroll
+    for (int u = 0; u < VPT; ++u) {
+      const int vi = v0 + u * 256 + static_cast<int>(threadIdx.x);
+      if (vi >= nvec) continue;
+      float xf[8], gf[8], bf[8], o[8];
+      unpack8_f16(v0 == 0 ? xq[u] : __ldcs(reinterpret_cast<const uint4*>(y) + vi), xf);
+      unpack8(p.gamma ? __ldg(reinterpret_cast<const uint4*>(p.gamma) + vi) : one, gf);
+      unpack8((KIND == EPI_LN && p.beta) ? __ldg(reinterpret_cast<const uint4*>(p.beta) + vi) : make_uint4(0, 0, 0, 0), bf);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if constexpr (KIND == EPI_LN) {
+          o[j] = fmaf((xf[j] - mu) * rstd, gf[j], bf[j]);
+          if (p.post_relu) o[j] = fmaxf(o[j], 0.f);
+        } else {
+          o[j] = xf[j] * rstd * gf[j];
+          if (o[j] > best) { best = o[j]; best_col = vi * 8 + j; }
+        }
+      }
+      reinterpret_cast<uint4*>(y)[vi] = make_uint4(pack2(o[0], o[1]), pack2(o[2], o[3]), pack2(o[4], o[5]), pack2(o[6], o[7]));
+    }
+  }
+  if constexpr (KIND == EPI_RMS_MAX) {
+    row_argmax_reduce<256>(best, best_col, s_red, s_idx);
+    if (threadIdx.x == 0) {
+      p.row_max[r] = best;
+      p.row_argmax[r] = best_col;
+    }
+  }
+}
+
 // S = bf16(GELU_tanh(P + b1)), in place over a dense [rows, n] bf16 matrix (unfused B2B: the intermediate epilogue).
 __global__ void __launch_bounds__(256) bias_gelu_kernel(uint16_t* P, const uint16_t* bias, long long nvec_total, int nvec_row) {
   const long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -369,11 +460,12 @@ cudaError_t launch_row_epilogue(int kind, const RowParams& p, cudaStream_t st) {
   }
 }
 
-cudaError_t launch_wide_row_finish(int kind, const RowParams& p, const float2* partials, int nblocks, int block, cudaStream_t st) {
+cudaError_t launch_wide_row_finish(int kind, const RowParams& p, const float2* partials, int nblocks, int block, long long form_rows, cudaStream_t st) {
   const long long rows = static_cast<long long>(p.batch) * p.M;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  cfg.gridDim = dim3(static_cast<unsigned>((rows + 7) / 8), 1, 1);  // eight rows (warps) per block
+  const bool block_per_row = form_rows <= 1184;  // 8 blocks on each of 148 SMs; else eight rows (warps) per block
+  cfg.gridDim = dim3(static_cast<unsigned>(block_per_row ? rows : (rows + 7) / 8), 1, 1);
   cfg.blockDim = dim3(256, 1, 1);
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // its launch overlaps the first kernel's tail
@@ -381,6 +473,11 @@ cudaError_t launch_wide_row_finish(int kind, const RowParams& p, const float2* p
   cfg.attrs = attr;
   cfg.numAttrs = programmatic_launch_enabled() ? 1 : 0;
   count_launch();
+  if (block_per_row) {
+    if (kind == EPI_LN) return cudaLaunchKernelEx(&cfg, wide_row_finish_block_kernel<EPI_LN>, p, partials, nblocks, block);
+    if (kind == EPI_RMS_MAX) return cudaLaunchKernelEx(&cfg, wide_row_finish_block_kernel<EPI_RMS_MAX>, p, partials, nblocks, block);
+    return cudaErrorInvalidValue;
+  }
   if (kind == EPI_LN) return cudaLaunchKernelEx(&cfg, wide_row_finish_kernel<EPI_LN>, p, partials, nblocks, block, rows);
   if (kind == EPI_RMS_MAX) return cudaLaunchKernelEx(&cfg, wide_row_finish_kernel<EPI_RMS_MAX>, p, partials, nblocks, block, rows);
   return cudaErrorInvalidValue;

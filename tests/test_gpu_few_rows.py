@@ -1,0 +1,47 @@
+"""LayerNorm / RMSNorm kinds behind a GEMM of few rows (weights as the tensor core's 128-row operand, contraction split over a
+cluster), at the edges of its cuts: one row, full and partial row groups of 16 / 32 / 64, full and partial 128-column tiles,
+one and two tiles per CTA, 1 to 8 shares of the contraction, row slices that end empty, the two-kernel form with a partial last
+block, both storage orders of the weights.  Against the fp64 oracle with the bounds of the other fused forms."""
+import pytest
+import torch
+
+import paper_2608_03537_b200 as cf
+import workloads as wl
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 8, 8), (16, 128, 64), (17, 136, 768), (32, 256, 72), (33, 2056, 200), (63, 1000, 2056), (64, 1024, 1792), (65, 4096, 64),
+          (2, 264, 4104), (40, 4096, 4096), (5, 2048, 1024), (70, 2824, 1032), (300, 768, 768), (900, 520, 320)]
+
+
+@pytest.mark.parametrize("nk", [False, True])
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_few_rows(M, N, K, nk, cuda_device):
+    flags = cf.FLAG_B_ROW_MAJOR_NK if nk else 0
+    for w in (wl.post_norm(M, N, K, seed=M + N + K, affine=True, relu=bool(M & 1)), wl.complex_subgraph(M, N, K, seed=M + N, activation=not (M & 1))):
+        T = P.dev_tensors(w)
+        ln = w.kind == wl.KIND_BIAS_RES_LAYERNORM
+        B = T["B"].mT.contiguous() if nk else T["B"]
+        Y = P.guarded((M, N), torch.bfloat16, float("nan"), T["A"].device)
+        got = {"Y": Y}
+        kw = dict(bias=T["bias"], residual=T["residual"], gamma=T["gamma"], alpha=w.scalars["alpha"], eps=w.scalars["eps"])
+        if ln:
+            kw.update(beta=T["beta"], flags=flags | (cf.FLAG_POST_RELU if w.scalars.get("relu") else 0))
+        else:
+            got["row_max"] = kw["row_max"] = P.guarded((M,), torch.float32, float("nan"), T["A"].device)
+            got["row_argmax"] = kw["row_argmax"] = P.guarded((M,), torch.int32, -1, T["A"].device)
+            kw["flags"] = flags | (0 if w.scalars.get("activation", True) else cf.FLAG_NO_ACTIVATION)
+        kind = cf.EPI_BIAS_RES_LAYERNORM if ln else cf.EPI_BIAS_GELU_RES_RMSNORM_MAX
+        desc = cf.make_gemm_desc(T["A"], B, Y, kind, residual=T["residual"], flags=kw["flags"])
+        ws = P.guarded((max(16, cf.workspace_size(desc)),), torch.uint8, 0xEE, T["A"].device)
+        for _ in range(2):
+            cf.gemm_epilogue(T["A"], B, Y, kind, workspace=ws, **kw)
+        torch.cuda.synchronize()
+        P.check_canaries({"ws": ws, **got}, label=w.name)
+        ref = P.run_oracle(w)
+        ymax = float(abs(ref["Y"]).max())
+        bounds = {"norm_tol": P.TOL_NORM_MAX if ymax < 8.0 else 2.0 ** -7 * ymax}   # bf16 half-ulp of the largest magnitude, twice
+        if not ln:
+            bounds["rowmax_tol"] = 3e-2   # the two-kernel form takes the maximum from values that went through fp16
+        P.check_outputs(w, got, ref, label=f"{w.name} nk={nk}", **bounds)
