@@ -458,8 +458,12 @@ comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void*
   }
   GemmMaps maps;
   if (desc->fused) {
-    if (!make_gemm_maps(&maps, A, B, a.residual, Y, desc->batch, desc->M, desc->N, desc->K, desc->lda, desc->ldb, desc->ldr,
+    if (!make_gemm_maps(&maps, A, B, epi == EPI_SOFTMAX ? nullptr : a.residual, Y, desc->batch, desc->M, desc->N, desc->K, desc->lda, desc->ldb, desc->ldr,
                         desc->ldy, desc->batch_stride_a, desc->batch_stride_b, bsr, bsy, b_nk))
+      return COMFUSE_ERR_CUDA;
+    // the softmax kinds have no residual: its map is the mask's, in boxes of one epilogue warp's 32 rows
+    if (desc->mask == COMFUSE_MASK_ADDITIVE &&
+        !encode_tmap_bf16_3d(&maps.R, a.mask, desc->N, desc->M, 1, static_cast<uint64_t>(desc->N) * 2, static_cast<uint64_t>(desc->M) * desc->N * 2, 32))
       return COMFUSE_ERR_CUDA;
   } else {  // the GEMM's output is the dense bf16 Z in the workspace
     if (!make_gemm_maps(&maps, A, B, nullptr, workspace, desc->batch, desc->M, desc->N, desc->K, desc->lda, desc->ldb, 0, desc->N,

@@ -13,7 +13,8 @@ bool softmax_rows_supported(const FusedParams& p) { return p.K <= 256 && p.N >= 
 cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_t stream) {
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
-  auto kern = p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true> : softmax_rows_kernel<NSTAGES, YBOXES, false>;
+  auto kern = p.mask ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true> : softmax_rows_kernel<NSTAGES, YBOXES, false, true>)
+                     : (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, false>);
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
   constexpr int kMaxDev = 64;
@@ -40,10 +41,12 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
 
   int ncl = max_clusters[di].load(std::memory_order_acquire);
   if (ncl == 0) {
-    cudaError_t e = cudaFuncSetAttribute(softmax_rows_kernel<NSTAGES, YBOXES, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(softmax_rows_kernel<NSTAGES, YBOXES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    for (auto k : {softmax_rows_kernel<NSTAGES, YBOXES, false, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, false>,
+                   softmax_rows_kernel<NSTAGES, YBOXES, false, true>, softmax_rows_kernel<NSTAGES, YBOXES, true, true>}) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+      if (e != cudaSuccess) return e;
+    }
     int n = 0;
     cfg.gridDim = dim3(2 * dev->sm_count, 1, 1);
     e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
@@ -58,7 +61,7 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
   if (clusters <= 0) return cudaSuccess;
   cfg.gridDim = dim3(clusters * 2, 1, 1);
   count_launch();
-  return cudaLaunchKernelEx(&cfg, kern, maps.A, maps.B, maps.Y, p);
+  return cudaLaunchKernelEx(&cfg, kern, maps.A, maps.B, maps.R, maps.Y, p);
 }
 
 }  // namespace comfuse

@@ -59,10 +59,15 @@ struct RowSoftmaxCfg {
 
 // BKM: the B operand is stored [N, K] (one box of this CTA's 128 columns x 64 contraction elements per stage, K-major for the
 // UMMA, like A) instead of [K, N] (two boxes of 64 contraction rows x 64 columns, MN-major).
-template <int NSTAGES, int YBOXES, bool BKM>
+// ADD: an additive mask tensor [M, N].  A thread owns a row of the chunk, so reading the mask straight from global memory
+// touches 32 rows per load instruction (32 sectors for 512 bytes, in both passes): 96 batches of 504 x 504 scores took 47.0 us
+// that way, 36.3 with the boxes below.  Every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
+// take the result: read the box, overwrite it with the probabilities, store it.  The warp's elected lane asks for the box
+// of the unit after next as soon as a box is free, and issues the store itself (no barrier round trip through other warps).
+template <int NSTAGES, int YBOXES, bool BKM, bool ADD>
 __global__ void __launch_bounds__(32 * 20, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
+                    const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
   constexpr int CHUNK = Cfg::CHUNK;
 
@@ -115,6 +120,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     prefetch_tensormap(&tmA);
     prefetch_tensormap(&tmB);
     prefetch_tensormap(&tmY);
+    if (ADD) prefetch_tensormap(&tmM);
   }
   if (warp == 1) {
     tmem_alloc_pair(smem_u32(s_tmem_base), 2 * CHUNK);
@@ -220,7 +226,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else if (warp == Cfg::kStoreWarp) {
     // ------------------------------------------------------------------------------------------ store warp
     // Lane e mirrors epilogue warp e: per live chunk, wait until the box is staged, store it, hand the staging box back.
-    if (lane < Cfg::kEpiWarps) {
+    if (!ADD && lane < Cfg::kEpiWarps) {  // (with a mask the epilogue warps store their boxes themselves)
       const int e = lane;
       const int q = (e + 2) & 3;
       const int h = e >> 2;
@@ -258,7 +264,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // constant zero box in flight, walk them with a cursor of their own, independent of the epilogue (asynchronous
     // stores: plain stores would share the SM's memory-instruction queue with the epilogue's exponentials and
     // shared-memory traffic).  Few boxes in flight, so that a staged box never queues far behind zeros.
-    if (lane < Cfg::ZERO_TMA_LANES && p.causal) {
+    if (!ADD && lane < Cfg::ZERO_TMA_LANES && p.causal) {
       const uint64_t stream_out = l2_policy_evict_first();
       uint32_t k = 0;
       for (int r = 0; r < rounds; ++r) {
@@ -297,7 +303,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool capped = p.softcap > 0.f;
     const SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
     const float sc = capped ? 1.f : p.alpha * 1.4426950408889634f;
-    const bool additive = p.mask != nullptr;  // additive mask tensor, applied behind the scale / soft-cap
+    constexpr bool additive = ADD;  // additive mask tensor, applied behind the scale / soft-cap
     constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
 
 #ifdef COMFUSE_TRACE
@@ -321,6 +327,54 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       tcgen05_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster_noflush(tempty_leader + 8u * slot);
+    };
+
+    // ADD: unit n of this warp (passes 0 and 1 of every tile, the chunks in which its columns exist) uses box n % YBOXES; its mask
+    // is requested when unit n - YBOXES has finished with the box.
+    const int my_chunks = ADD ? (p.N - h * 64 + CHUNK - 1) / CHUNK : 0;  // (causal off: every chunk is live)
+    int load_r = -1, load_c = 0, load_row = 0;
+    bool load_pass1 = true;
+    uint32_t load_n = 0, mask_n = 0;
+    bool store_pending = false;
+    const uint64_t keep_mask = ADD ? l2_policy_evict_last() : 0, stream_box = ADD ? l2_policy_evict_first() : 0;
+    // the elected lane; steps through the units in the order in which they run (load_r = rounds: no further unit)
+    load_c = my_chunks;
+    auto request_mask = [&]() {
+      if (load_c >= my_chunks) {
+        load_c = 0;
+        load_pass1 = !load_pass1;
+        if (!load_pass1 && load_r < rounds) {
+          int lb, lm = 0, lL;
+          if (++load_r < rounds && !tile_at(load_r, lb, lm, lL)) load_r = rounds;
+          load_row = lm + static_cast<int>(pm) * 128 + q * 32;
+        }
+      }
+      if (my_chunks <= 0 || load_r >= rounds) return;
+      const uint32_t sel = load_n % YBOXES;
+      mbar_arrive_expect_tx(bar_yfull(e, sel), Cfg::WARP_BOX_BYTES);
+      tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_yfull(e, sel), load_c * CHUNK + h * 64, load_row, 0, keep_mask);
+      ++load_n;
+      ++load_c;
+    };
+    bool elected = false;
+    if constexpr (ADD) {
+      elected = elect_one();
+      if (elected)
+        for (int i = 0; i < YBOXES; ++i) request_mask();
+      __syncwarp();
+    }
+    // 32 mask values of half `half` of this thread's row of the box, as log2-domain addends
+    auto box_mask = [&](uint32_t box, int half, float2 (&m2)[16]) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t w4[4];
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w4[0]), "=r"(w4[1]), "=r"(w4[2]), "=r"(w4[3])
+                     : "r"(box + static_cast<uint32_t>(lane * 128 + (((half * 4 + i) ^ (lane & 7)) << 4)))
+                     : "memory");
+#pragma unroll
+        for (int k = 0; k < 4; ++k) m2[4 * i + k] = mul2(bf16x2_to_f2(w4[k]), splat2(1.4426950408889634f));
+      }
     };
 
     for (int r = 0; r < rounds; ++r) {
@@ -347,6 +401,23 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           wait_slot(slot);
           const uint32_t taddr = tmem_base + lane_sel + slot * CHUNK + h * 64;
           const int colg = c * CHUNK + h * 64;
+          const uint32_t msel = mask_n % YBOXES;
+          const uint32_t mbox = ybox0 + msel * Cfg::WARP_BOX_BYTES;
+          if constexpr (ADD) {
+            if (store_pending) {  // the previous unit's box: read out by now, it takes the mask of the unit after this one
+              if (elected) {
+                tma_store_wait_read<0>();
+                request_mask();
+              }
+              __syncwarp();
+              store_pending = false;
+            }
+            if (colg < p.N) {
+              mbar_wait<false>(bar_yfull(e, msel), (mask_n / YBOXES) & 1u, w);
+              __syncwarp();
+              ++mask_n;
+            }
+          }
           if (pass == 0) {
             // ---------------- pass 0: online (max, sum of 2^(t - max)) over this thread's columns of the chunk
 #pragma unroll
@@ -361,9 +432,9 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
               }
               float2 tv[16];
-              if (additive) {  // a full-tensor operand of the epilogue (Sec. 5.2): this thread's 32 mask values from global memory
+              if (additive) {  // a full-tensor operand of the epilogue (Sec. 5.2)
                 float2 m2[16];
-                load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
+                box_mask(mbox, half, m2);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) tv[j] = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
               } else {
@@ -399,6 +470,10 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
               }
             }
             release_slot(slot);
+            if (ADD && colg < p.N) {  // (release_slot converged the warp behind its reads)
+              if (elected) request_mask();
+              __syncwarp();
+            }
           } else {
             // ---------------- pass 1: the scores again, normalised, rounded once, staged and stored
             uint32_t pk[32];
@@ -419,7 +494,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 float2 ev[16];
                 if (additive) {
                   float2 m2[16];
-                  load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
+                  box_mask(mbox, half, m2);
 #pragma unroll
                   for (int j = 0; j < 16; ++j) {  // (a masked score is -inf, and so is -inf - off: its probability is an exact zero)
                     const float2 t01 = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), add2(m2[j], splat2(-off)));
@@ -445,10 +520,11 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
             release_slot(slot);
             if (colg < p.N) {
-              const uint32_t sel = nbox % YBOXES;
+              const uint32_t sel = ADD ? msel : nbox % YBOXES;
               const uint32_t ybox = ybox0 + sel * Cfg::WARP_BOX_BYTES;
-              // the store of the box's previous contents has read it out
-              mbar_wait<false>(bar_yfree(e, sel), ((nbox / YBOXES) & 1u) ^ 1u, w);
+              // the store of the box's previous contents has read it out (ADD: the box holds this unit's mask, every lane has
+              // read its own row of it and now overwrites that row)
+              if (!ADD) mbar_wait<false>(bar_yfree(e, sel), ((nbox / YBOXES) & 1u) ^ 1u, w);
               ++nbox;
               __syncwarp();
 #pragma unroll
@@ -460,7 +536,17 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
               }
               fence_proxy_async_smem();
               __syncwarp();
-              if (lane == 0) mbar_arrive(bar_yfull(e, sel));
+              if constexpr (ADD) {
+                if (elected) {
+                  if (COMFUSE_IN_BOUNDS(colg >= 0 && colg < p.N && (colg & 7) == 0 && mpair0 >= 0 && b >= 0 && b < p.batch, p.status))
+                  tma_store_3d_hint(&tmY, ybox, colg, m0 + q * 32, b, stream_box);
+                  tma_store_commit();
+                }
+                __syncwarp();
+                store_pending = true;
+              } else {
+                if (lane == 0) mbar_arrive(bar_yfull(e, sel));
+              }
             }
           }
         }
@@ -486,6 +572,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
     }
+    if (ADD && elected) tma_store_wait_read<0>();  // the boxes must outlive the last store's read
   }
 
   // -------------------------------------------------------------------------------------------- teardown
