@@ -266,9 +266,14 @@ comfuse_status_t run_few_rows(const FewRowsPlan& plan, int epi, const comfuse_ge
   p.wide = plan.wide ? 1 : 0;
   p.post_relu = (d.flags & COMFUSE_FLAG_POST_RELU) ? 1 : 0;
   p.no_activation = (d.flags & COMFUSE_FLAG_NO_ACTIVATION) ? 1 : 0;
-  p.bias = static_cast<const uint16_t*>(a.bias);
-  p.gamma = static_cast<const uint16_t*>(a.gamma);
-  p.beta = static_cast<const uint16_t*>(a.beta);
+  p.causal = d.mask == COMFUSE_MASK_CAUSAL ? 1 : 0;
+  p.softcap = d.softcap;
+  p.mask = d.mask == COMFUSE_MASK_ADDITIVE ? static_cast<const uint16_t*>(a.mask) : nullptr;
+  if (epi != EPI_SOFTMAX) {  // (the softmax kind takes none of the row vectors)
+    p.bias = static_cast<const uint16_t*>(a.bias);
+    p.gamma = static_cast<const uint16_t*>(a.gamma);
+    p.beta = static_cast<const uint16_t*>(a.beta);
+  }
   p.residual = static_cast<const uint16_t*>(a.residual);
   p.ldr = d.ldr; p.batch_stride_r = d.batch > 1 ? d.batch_stride_r : 0;
   p.Y = static_cast<uint16_t*>(Y);
@@ -451,7 +456,9 @@ comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void*
   const long long bsr = desc->batch > 1 ? desc->batch_stride_r : 0;
   const long long bsy = desc->batch > 1 ? desc->batch_stride_y : 0;
   const bool b_nk = (desc->flags & COMFUSE_FLAG_B_ROW_MAJOR_NK) != 0;
-  if (desc->fused && forced_split_block() < 0) {
+  // COMFUSE_SOFTMAX_CLUSTER forces the cluster kernel of the softmax kind, COMFUSE_SPLIT_BLOCK the tile kernel of the others
+  static const bool forced_cluster = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr;
+  if (desc->fused && (epi == EPI_SOFTMAX ? !forced_cluster : forced_split_block() < 0)) {
     const int wide_block = need > 0 ? wide_row_block(epi, desc->N, desc->K, form_row_pairs(desc, form_rows)) : 0;
     const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, *dev);
     if (few.mt) return run_few_rows(few, epi, *desc, a, A, B, Y, static_cast<float2*>(workspace), *dev, st, form_rows);

@@ -1,4 +1,4 @@
-// LayerNorm / RMSNorm kinds behind a GEMM of few rows.
+// LayerNorm, RMSNorm and softmax kinds behind a GEMM of few rows.
 //
 // What bounds it: the weights, and below a few megabytes of them the latency of one pass through the kernel.  A decoding step
 // of 40 rows through a 4096 x 4096 layer moves 33.5 MB of weights and multiplies almost nothing; the tile kernel (256-row CTA
@@ -14,6 +14,8 @@
 //     accesses, the row statistic is a shuffle reduction, and the CT partials of a row are exchanged through distributed
 //     shared memory as in the tile kernel.  16 epilogue warps, so that a warp has at most four rows and they advance
 //     together: with 8 warps and a loop over the rows the epilogue of 64 rows took 9000 clocks, now about 2000.
+//   * Softmax kind: the same, with (maximum, sum of exponentials) as the statistic.  A CTA exponentiates against the maximum
+//     of its own columns, so every score takes one exponential; the exchange yields the factor that corrects for the row.
 //   * Rows that the tile kernel would cut into 256-column blocks (the two-kernel form) are cut here too: x goes out as fp16
 //     with the block's statistic, and the finishing kernel normalises it.
 //
@@ -249,7 +251,9 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
         res[i][t] = zero;
-        if (p.residual && r < rv && in[t])
+        if (EPI == EPI_SOFTMAX && p.mask && r < rv && in[t])  // (the mask is the softmax kind's full-tensor operand)
+          res[i][t] = __ldg(reinterpret_cast<const uint2*>(p.mask + static_cast<long long>(row0 + r) * p.N + col[t]));
+        if (EPI != EPI_SOFTMAX && p.residual && r < rv && in[t])
           res[i][t] = __ldg(reinterpret_cast<const uint2*>(p.residual + static_cast<long long>(b) * p.batch_stride_r +
                                                            static_cast<long long>(row0 + r) * p.ldr + col[t]));
       }
@@ -354,55 +358,94 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             for (int j = 0; j < 4; ++j) x[i][t][j] += o[j];
           }
       }
-    float pa[RC], pb[RC];  // (mean, M2) or (sum of squares, unused) of this lane's columns
+    float pa[RC], pb[RC];  // (mean, M2), (sum of squares, unused) or (maximum, sum of exponentials) of this lane's columns
+    if constexpr (EPI == EPI_SOFTMAX) {
+      // scores in the log2 domain; masked ones and the columns from N on are -inf
+      const bool capped = p.softcap > 0.f;
+      const SoftcapLog2 cap_fn(alpha, capped ? p.softcap : 1.f);
+      const float sc = alpha * 1.4426950408889634f;
 #pragma unroll
-    for (int i = 0; i < RC; ++i) {
-      pa[i] = pb[i] = 0.f;
+      for (int i = 0; i < RC; ++i) {
+        const int last = p.causal ? row0 + e + i * Cfg::kEpiWarps : p.N - 1;  // last live column of the row
+        pa[i] = -INFINITY;
 #pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        float(&xx)[4] = x[i][t];
-        float2 z01 = fma2(splat2(alpha), make_float2(xx[0], xx[1]), bf16x2_to_f2(bias[t].x));
-        float2 z23 = fma2(splat2(alpha), make_float2(xx[2], xx[3]), bf16x2_to_f2(bias[t].y));
-        if (gelu) {
-          z01 = gelu_tanh_f32x2(z01);
-          z23 = gelu_tanh_f32x2(z23);
+        for (int t = 0; t < NT; ++t) {
+          float(&xx)[4] = x[i][t];
+          const float2 m01 = mul2(bf16x2_to_f2(res[i][t].x), splat2(1.4426950408889634f)), m23 = mul2(bf16x2_to_f2(res[i][t].y), splat2(1.4426950408889634f));
+          const float mk[4] = {m01.x, m01.y, m23.x, m23.y};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            xx[j] = capped ? cap_fn(xx[j]) + mk[j] : fmaf(xx[j], sc, mk[j]);
+            if (!in[t] || col[t] + j > last) xx[j] = -INFINITY;
+            pa[i] = fmaxf(pa[i], xx[j]);
+          }
         }
-        z01 = add2(z01, bf16x2_to_f2(res[i][t].x));
-        z23 = add2(z23, bf16x2_to_f2(res[i][t].y));
-        xx[0] = z01.x; xx[1] = z01.y; xx[2] = z23.x; xx[3] = z23.y;
-        // (columns from N on hold exact zeros: operands outside the matrix read as zeros, bias and residual are masked)
-        if constexpr (EPI == EPI_LN) {
-          pa[i] += (xx[0] + xx[1]) + (xx[2] + xx[3]);
-        } else {
-          const float2 sq = fma2(z23, z23, mul2(z01, z01));
-          pa[i] += sq.x + sq.y;
-        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) pa[i] = fmaxf(pa[i], __shfl_xor_sync(0xFFFFFFFFu, pa[i], o));  // every lane needs it
       }
-      if constexpr (EPI == EPI_LN) {
-        pa[i] *= inv_mean_n;
+#pragma unroll
+      for (int i = 0; i < RC; ++i) {
+        const float m = pa[i] == -INFINITY ? 0.f : pa[i];  // (a row without a live column here: every exponential is 0)
+        pb[i] = 0.f;
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float d = in[t] || p.wide ? x[i][t][j] - pa[i] : 0.f;
-            pb[i] = fmaf(d, d, pb[i]);
+            x[i][t][j] = ex2_approx(x[i][t][j] - m);
+            pb[i] += x[i][t][j];
           }
       }
-    }
-    if constexpr (EPI == EPI_LN) {
-      transposed_reduce<RC>(pa, pb, lane, [&](int step, float& a0, float& a1, float b0, float b1) {
-        const float d = b0 - a0;
-        a0 = fmaf(d, wb[step], a0);
-        a1 = a1 + b1 + d * d * wm[step];
-      });
+      transposed_reduce<RC>(pa, pb, lane, [&](int, float& a0, float& a1, float, float b1) { a1 += b1; });
     } else {
-      transposed_reduce<RC>(pa, pb, lane, [&](int, float& a0, float&, float b0, float) { a0 += b0; });
+#pragma unroll
+      for (int i = 0; i < RC; ++i) {
+        pa[i] = pb[i] = 0.f;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          float(&xx)[4] = x[i][t];
+          float2 z01 = fma2(splat2(alpha), make_float2(xx[0], xx[1]), bf16x2_to_f2(bias[t].x));
+          float2 z23 = fma2(splat2(alpha), make_float2(xx[2], xx[3]), bf16x2_to_f2(bias[t].y));
+          if (gelu) {
+            z01 = gelu_tanh_f32x2(z01);
+            z23 = gelu_tanh_f32x2(z23);
+          }
+          z01 = add2(z01, bf16x2_to_f2(res[i][t].x));
+          z23 = add2(z23, bf16x2_to_f2(res[i][t].y));
+          xx[0] = z01.x; xx[1] = z01.y; xx[2] = z23.x; xx[3] = z23.y;
+          // (columns from N on hold exact zeros: operands outside the matrix read as zeros, bias and residual are masked)
+          if constexpr (EPI == EPI_LN) {
+            pa[i] += (xx[0] + xx[1]) + (xx[2] + xx[3]);
+          } else {
+            const float2 sq = fma2(z23, z23, mul2(z01, z01));
+            pa[i] += sq.x + sq.y;
+          }
+        }
+        if constexpr (EPI == EPI_LN) {
+          pa[i] *= inv_mean_n;
+#pragma unroll
+          for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float d = in[t] || p.wide ? x[i][t][j] - pa[i] : 0.f;
+              pb[i] = fmaf(d, d, pb[i]);
+            }
+        }
+      }
+      if constexpr (EPI == EPI_LN) {
+        transposed_reduce<RC>(pa, pb, lane, [&](int step, float& a0, float& a1, float b0, float b1) {
+          const float d = b0 - a0;
+          a0 = fmaf(d, wb[step], a0);
+          a1 = a1 + b1 + d * d * wm[step];
+        });
+      } else {
+        transposed_reduce<RC>(pa, pb, lane, [&](int, float& a0, float&, float b0, float) { a0 += b0; });
+      }
     }
     {
       // lanes that hold the same row may differ in the last bit: all of them send the first one's value
       const int first_lane = lane & (32 - 32 / RC);
       const float s0 = __shfl_sync(0xFFFFFFFFu, pa[0], first_lane);
-      const float s1 = EPI == EPI_LN ? __shfl_sync(0xFFFFFFFFu, pb[0], first_lane) : 0.f;
+      const float s1 = EPI != EPI_RMS_MAX ? __shfl_sync(0xFFFFFFFFu, pb[0], first_lane) : 0.f;
       const int r = e + my_row * Cfg::kEpiWarps;
 #pragma unroll
       for (int k = 0; k < CPL; ++k) {
@@ -436,6 +479,19 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
           const float d = o[k].x - mu_l;
           sq_l += fmaf(range_n[k] * d, d, o[k].y);
         }
+      } else if constexpr (EPI == EPI_SOFTMAX) {
+        float m = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+          if (mlane + k * LPR >= p.ct || r >= rv) o[k].x = -INFINITY;
+          m = fmaxf(m, o[k].x);
+        }
+#pragma unroll
+        for (int d = LPR / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) sq_l += o[k].x == -INFINITY ? 0.f : o[k].y * ex2_approx(o[k].x - m);
+        const float own = r < rv ? s_stat[r * 16 + ct].x : -INFINITY;  // this CTA's exponentials are relative to its own maximum
+        mu_l = own == -INFINITY ? 0.f : ex2_approx(own - m);
       } else {
 #pragma unroll
         for (int k = 0; k < CPL; ++k) sq_l += o[k].x;
@@ -446,7 +502,9 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
       if (p.wide && ct == 0 && mlane == 0 && r < rv && COMFUSE_IN_BOUNDS(grow < p.M && nb < p.nblocks && b < p.batch, p.status))
         p.wide_partials[(static_cast<long long>(b) * p.M + grow) * p.nblocks + nb] = make_float2(EPI == EPI_LN ? mu_l : sq_l, EPI == EPI_LN ? sq_l : 0.f);
     }
-    const float rstd_l = rsqrtf(sq_l * inv_n_all + eps);
+    // factor of the row: 1 / standard deviation, or what turns this CTA's exponentials into probabilities (a row without a live
+    // column is all zero)
+    const float rstd_l = EPI == EPI_SOFTMAX ? (sq_l > 0.f ? mu_l / sq_l : 0.f) : rsqrtf(sq_l * inv_n_all + eps);
     const float shift_l = -mu_l * rstd_l;
     float rstd[RC], shift[RC], best[RC], best_col[RC];
 #pragma unroll
@@ -477,6 +535,8 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             if constexpr (EPI == EPI_LN) {
               y[j] = fmaf(fmaf(xx[j], rstd[i], shift[i]), gm[j], be[j]);
               if (p.post_relu) y[j] = fmaxf(y[j], 0.f);
+            } else if constexpr (EPI == EPI_SOFTMAX) {
+              y[j] = xx[j] * rstd[i];
             } else {
               y[j] = xx[j] * rstd[i] * gm[j];
               if (in[t] && y[j] > bv) { bv = y[j]; bc = col[t] + j; }
@@ -609,8 +669,8 @@ int resident_clusters(int size, const DeviceInfo& dev) {
 
 FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_block, const DeviceInfo& dev) {
   FewRowsPlan none, c;
-  if (epi != EPI_LN && epi != EPI_RMS_MAX) return none;
-  if (N > kWideRowBlock && wide_block != 256) return none;
+  if (epi != EPI_LN && epi != EPI_RMS_MAX && epi != EPI_SOFTMAX) return none;
+  if (N > kWideRowBlock && (wide_block != 256 || epi == EPI_SOFTMAX)) return none;
   // Rows of 2048 columns and more behind a long contraction keep the two-kernel form: 256-column blocks spread the weights
   // over the machine, a row's own cluster reaches 16 SMs (40 x 4096 x 4096: 12.8 us against 37).
   c.wide = wide_block == 256 && (N > kWideRowBlock || (N >= 2048 && K >= 1024));
@@ -623,6 +683,8 @@ FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_bloc
   // weights [N, K]): 128 x 256 x 256 7.7 / 4.6, 128 x 1024 x 1024 19.0 / 6.1, 512 x 768 x 768 13.4 / 5.7, 512 x 1024 x 2048
   // 17.8 / 9.2, 1024 x 512 x 1024 18.8 / 6.5, 4096 x 256 x 1024 11.6 / 7.4.  With a second round of clusters the two are level
   // or the tile kernel is ahead (1024 x 1024 x 64 10.8 / 9.3, 2048 x 768 x 64 8.9 / 9.4, 2048 x 1024 x 1024 19.4 / 20.9).
+  // Softmax kind, one round (row or cluster kernel / this one, K = 64): 8 x 64 x 512 11.0 / 4.4, 2 x 1024 x 1024 12.7 / 6.7,
+  // 140 x 64 x 128 11.6 / 5.4; two rounds: 16 x 512 x 512 causal 10.6 / 12.8, 2 x 1171 x 1176 masked 11.4 / 12.5.
   for (c.nt = 1; c.nt <= 2; ++c.nt) {
     c.ct = c.wide ? 2 : (N + 128 * c.nt - 1) / (128 * c.nt);
     if (c.ct > 16 || clusters > resident_clusters(c.ct, dev)) {
@@ -648,8 +710,9 @@ cudaError_t launch_few_rows(int epi, const FewRowsPlan& plan, const CUtensorMap&
   p.groups = (p.M + plan.mt - 1) / plan.mt;
 #define COMFUSE_CASE(NT, MT)                                                                                     \
   if (plan.nt == NT && plan.mt == MT)                                                                            \
-    return epi == EPI_LN ? launch_instance<EPI_LN, NT, MT>(plan, tmW, tmX, p, stream)                            \
-                         : launch_instance<EPI_RMS_MAX, NT, MT>(plan, tmW, tmX, p, stream);
+    return epi == EPI_LN        ? launch_instance<EPI_LN, NT, MT>(plan, tmW, tmX, p, stream)                     \
+           : epi == EPI_SOFTMAX ? launch_instance<EPI_SOFTMAX, NT, MT>(plan, tmW, tmX, p, stream)                \
+                                : launch_instance<EPI_RMS_MAX, NT, MT>(plan, tmW, tmX, p, stream);
   COMFUSE_CASE(1, 16)
   COMFUSE_CASE(1, 32)
   COMFUSE_CASE(1, 64)

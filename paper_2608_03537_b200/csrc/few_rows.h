@@ -1,4 +1,4 @@
-// The LayerNorm / RMSNorm kinds behind a GEMM of FEW ROWS (a decoding step, a small batch): plan and launch.
+// The fused kinds behind a GEMM of FEW ROWS (a decoding step, a small batch, the scores of a few heads): plan and launch.
 #pragma once
 
 #include <cuda.h>
@@ -24,6 +24,9 @@ struct FewRowsParams {
   int ct, ks, nblocks, groups;  // groups = row groups of mt rows
   float alpha, eps;
   int b_nk, wide, post_relu, no_activation;
+  int causal;             // softmax kind
+  float softcap;          // softmax kind, 0 = none
+  const uint16_t* mask;   // softmax kind: additive [M, N] mask shared by the batches, or null
   const uint16_t* bias;
   const uint16_t* gamma;
   const uint16_t* beta;

@@ -1,4 +1,4 @@
-"""LayerNorm / RMSNorm kinds behind a GEMM of few rows (weights as the tensor core's 128-row operand, contraction split over a
+"""Fused kinds behind a GEMM of few rows (weights as the tensor core's 128-row operand, contraction split over a
 cluster), at the edges of its cuts: one row, full and partial row groups of 16 / 32 / 64, full and partial 128-column tiles,
 one and two tiles per CTA, 1 to 8 shares of the contraction, row slices that end empty, the two-kernel form with a partial last
 block, both storage orders of the weights.  Against the fp64 oracle with the bounds of the other fused forms."""
@@ -45,3 +45,24 @@ def test_few_rows(M, N, K, nk, cuda_device):
         if not ln:
             bounds["rowmax_tol"] = 3e-2   # the two-kernel form takes the maximum from values that went through fp16
         P.check_outputs(w, got, ref, label=f"{w.name} nk={nk}", **bounds)
+
+
+@pytest.mark.parametrize("mask", ["none", "causal", "additive"])
+@pytest.mark.parametrize("batch,M,N,K,softcap", [(1, 1, 8, 8, 0.0), (3, 16, 128, 64, 0.0), (2, 17, 136, 72, 3.0), (5, 33, 1000, 64, 0.0), (1, 65, 2056, 64, 0.0), (2, 64, 2048, 776, 2.5),
+                                                 (1, 40, 4096, 2056, 0.0), (30, 130, 120, 64, 0.0)])
+def test_few_rows_softmax(batch, M, N, K, softcap, mask, cuda_device):
+    import numpy as np
+    if mask == "causal":
+        N = M = min(M * 8, 520)
+    w = wl.scaled_masked_softmax(batch, M, N, K, seed=M + N, causal=mask == "causal", softcap=softcap)
+    if mask == "additive":
+        g = np.random.default_rng(N)
+        m = (g.standard_normal((M, N)) * 2.0).astype(np.float32)
+        m[g.random((M, N)) < 0.2] = -np.inf
+        m[M // 2, :] = -np.inf                     # a row without a live column is all zero
+        m[0, : N // 2] = -np.inf                   # a row whose first column ranges have none
+        w.tensors["mask"] = wl.f32_to_bf16_bits(m)
+    got = P.run_gpu(w, P.dev_tensors(w), fused=True)
+    P.check_outputs(w, got, P.run_oracle(w), label=f"{w.name} {mask}", softmax_tol=P.TOL_SOFTMAX_MAX)
+    if mask == "additive":
+        assert (got["Y"][:, M // 2, :] == 0).all()
