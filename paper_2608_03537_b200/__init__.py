@@ -125,11 +125,12 @@ class ComfuseError(RuntimeError):
 
 
 _lib = None
+_bind = None   # the argument-marshalling extension, once the library is loaded
 
 
 def lib() -> ctypes.CDLL:
     """Load libcomfuse.so (built by ``python -m paper_2608_03537_b200.build``).  Fails loudly if absent."""
-    global _lib
+    global _lib, _bind
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(
@@ -178,8 +179,18 @@ def lib() -> ctypes.CDLL:
         L.comfuse_launch_count.restype = c_uint64
         L.comfuse_status_string.argtypes = [c_int32]
         L.comfuse_status_string.restype = ctypes.c_char_p
+        from . import _binding as b   # built with the library (csrc/binding.c)
+        b.bind(*(ctypes.cast(f, c_void_p).value for f in (L.comfuse_gemm_epilogue, L.comfuse_b2b_gemm, L.comfuse_gemm_spec)))
+        _bind = b
         _lib = L
     return _lib
+
+
+def _bound():
+    """The argument-marshalling extension, with the library's entry points in it."""
+    if _bind is None:
+        lib()
+    return _bind
 
 
 def _ptr(t):
@@ -187,33 +198,26 @@ def _ptr(t):
 
 
 def _stream(stream=None):
+    return c_void_p(stream.cuda_stream if stream is not None else _current_stream())
+
+
+def _current_stream() -> int:
+    """Handle of the current stream of the current device.  The first call goes through torch.cuda (which sets the device
+    up), the others ask for the bare handle: building a Stream object takes 3 us."""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return c_void_p(s.cuda_stream)
+    handle = torch.cuda.current_stream().cuda_stream
+    if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+        global _current_stream
+        raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        _current_stream = lambda: raw(device())  # noqa: E731
+    return handle
 
 
 def make_gemm_desc(A, B, Y, kind, *, residual=None, alpha=1.0, eps=1e-5, mask=MASK_NONE, fused=True, flags=0,
                    softcap=0.0) -> GemmDesc:
     """Describe A [b, M, K] (or [M, K]), B [b, K, N] (or [K, N]; with FLAG_B_ROW_MAJOR_NK in ``flags``: [b, N, K]),
     Y [b, M, N] from torch tensors' shapes and strides."""
-    batched = A.dim() == 3
-    batch = A.shape[0] if batched else 1
-    M, K = A.shape[-2], A.shape[-1]
-    b_nk = bool(int(flags) & FLAG_B_ROW_MAJOR_NK)
-    N = B.shape[-2] if b_nk else B.shape[-1]
-    assert (B.shape[-1] if b_nk else B.shape[-2]) == K and Y.shape[-2] == M and Y.shape[-1] == N
-    assert A.stride(-1) == 1 and B.stride(-1) == 1 and Y.stride(-1) == 1
-    d = GemmDesc()
-    d.batch, d.M, d.N, d.K = batch, M, N, K
-    d.lda, d.ldb, d.ldy = A.stride(-2), B.stride(-2), Y.stride(-2)
-    d.ldr = residual.stride(-2) if residual is not None else N
-    d.batch_stride_a = A.stride(0) if batched else M * d.lda
-    d.batch_stride_b = B.stride(0) if batched else (N if b_nk else K) * d.ldb
-    d.batch_stride_y = Y.stride(0) if batched else M * d.ldy
-    d.batch_stride_r = (residual.stride(0) if batched else M * d.ldr) if residual is not None else M * N
-    d.kind, d.mask, d.alpha, d.eps, d.fused, d.reserved = int(kind), int(mask), float(alpha), float(eps), int(bool(fused)), 0
-    d.flags, d.softcap = int(flags), float(softcap)
-    return d
+    return GemmDesc.from_buffer_copy(_bound().gemm_desc(A, B, Y, kind, residual, alpha, eps, mask, fused, flags, softcap))
 
 
 def workspace_size(desc: GemmDesc) -> int:
@@ -230,10 +234,8 @@ def gemm_epilogue(A, B, Y, kind, *, bias=None, residual=None, gamma=None, beta=N
     """Enqueue Y = subgraph(alpha * A.B) on the current (or given) stream.  Tensors are CUDA bf16 (row_max fp32,
     row_argmax int32).  ``workspace`` is a CUDA uint8 tensor of at least workspace_size(desc) bytes (unfused path, and fused LayerNorm /
     RMSNorm rows wider than 4096 columns)."""
-    d = make_gemm_desc(A, B, Y, kind, residual=residual, alpha=alpha, eps=eps, mask=mask, fused=fused, flags=flags, softcap=softcap)
-    args = EpilogueArgs(_ptr(bias), _ptr(residual), _ptr(gamma), _ptr(beta), _ptr(mask_tensor), _ptr(row_max), _ptr(row_argmax))
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    st = lib().comfuse_gemm_epilogue(byref(d), _ptr(A), _ptr(B), _ptr(Y), byref(args), ws_ptr, ws_bytes, _stream(stream))
+    st = (_bind or _bound()).gemm_epilogue(A, B, Y, kind, residual, alpha, eps, mask, fused, flags, softcap, bias, gamma, beta, mask_tensor,
+                                              row_max, row_argmax, workspace, _current_stream if stream is None else stream)
     if st != OK:
         raise ComfuseError(st, "comfuse_gemm_epilogue")
     return Y
@@ -265,14 +267,8 @@ def b2b_attention(Q, Kt, V, O, *, alpha, fused=True, workspace=None, stream=None
     """Enqueue O = softmax(alpha * Q.Kt).V per batch (the attention form of the back-to-back GEMM).  Dense CUDA bf16
     tensors Q [b, M, d], Kt [b, d, S] (keys already transposed) or, with ``keys_row_major``, the keys as [b, S, d];
     V [b, S, d2], O [b, M, d2]."""
-    nb, M, K = Q.shape
-    N1, N2 = V.shape[1], V.shape[2]
-    assert Kt.shape == ((nb, N1, K) if keys_row_major else (nb, K, N1)) and V.shape == (nb, N1, N2) and O.shape == (nb, M, N2)
-    for t in (Q, Kt, V, O):
-        assert t.is_contiguous()
-    d = make_b2b_desc(M, K, N1, N2, 0.0, fused, B2B_SOFTMAX_ATTENTION, nb, alpha, B2B_FLAG_KEYS_ROW_MAJOR if keys_row_major else 0)
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    st = lib().comfuse_b2b_gemm(byref(d), _ptr(Q), _ptr(Kt), None, _ptr(V), None, None, None, _ptr(O), ws_ptr, ws_bytes, _stream(stream))
+    st = (_bind or _bound()).b2b(B2B_SOFTMAX_ATTENTION, Q, Kt, None, V, None, None, None, O, 0.0, alpha, fused,
+                                    B2B_FLAG_KEYS_ROW_MAJOR if keys_row_major else 0, workspace, _current_stream if stream is None else stream)
     if st != OK:
         raise ComfuseError(st, "comfuse_b2b_gemm")
     return O
@@ -313,14 +309,8 @@ def b2b_workspace_size(desc: B2bDesc) -> int:
 
 def b2b_gemm(X, W1, b1, W2, b2, O, *, gamma=None, beta=None, eps=1e-5, fused=True, workspace=None, stream=None):
     """Enqueue O = LayerNorm(GELU_tanh(X.W1 + b1).W2 + b2 + X) * gamma + beta.  Dense row-major CUDA bf16 tensors."""
-    M, K = X.shape
-    N1, N2 = W1.shape[1], W2.shape[1]
-    for t in (X, W1, W2, O):
-        assert t.is_contiguous()
-    d = make_b2b_desc(M, K, N1, N2, eps, fused)
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    st = lib().comfuse_b2b_gemm(byref(d), _ptr(X), _ptr(W1), _ptr(b1), _ptr(W2), _ptr(b2), _ptr(gamma), _ptr(beta), _ptr(O),
-                                ws_ptr, ws_bytes, _stream(stream))
+    st = (_bind or _bound()).b2b(B2B_MLP_GELU_LAYERNORM, X, W1, b1, W2, b2, gamma, beta, O, eps, 1.0, fused, 0, workspace,
+                                    _current_stream if stream is None else stream)
     if st != OK:
         raise ComfuseError(st, "comfuse_b2b_gemm")
     return O
@@ -329,15 +319,8 @@ def b2b_gemm(X, W1, b1, W2, b2, O, *, gamma=None, beta=None, eps=1e-5, fused=Tru
 def b2b_mlp_relu(X, W1, b1, W2, b2, O, *, fused=True, workspace=None, stream=None):
     """Enqueue O = ReLU(ReLU(X.W1 + b1).W2 + b2) (the two-layer ReLU MLP form of the back-to-back GEMM).  Dense row-major
     CUDA bf16 tensors X [M, K], W1 [K, N1], W2 [N1, N2], O [M, N2]; b1, b2 may be None."""
-    M, K = X.shape
-    N1, N2 = W1.shape[1], W2.shape[1]
-    assert W1.shape == (K, N1) and W2.shape == (N1, N2) and O.shape == (M, N2)
-    for t in (X, W1, W2, O):
-        assert t.is_contiguous()
-    d = make_b2b_desc(M, K, N1, N2, 0.0, fused, B2B_MLP_RELU)
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    st = lib().comfuse_b2b_gemm(byref(d), _ptr(X), _ptr(W1), _ptr(b1), _ptr(W2), _ptr(b2), None, None, _ptr(O),
-                                ws_ptr, ws_bytes, _stream(stream))
+    st = (_bind or _bound()).b2b(B2B_MLP_RELU, X, W1, b1, W2, b2, None, None, O, 0.0, 1.0, fused, 0, workspace,
+                                    _current_stream if stream is None else stream)
     if st != OK:
         raise ComfuseError(st, "comfuse_b2b_gemm")
     return O
@@ -462,20 +445,8 @@ def gemm_spec(A, B, Y, spec: FusionSpec, *, params=(), row_out=(), fused=True, w
     (row vectors [N], tensors [batch, M, N]), ``row_out`` the per-row output tensors (fp32, int32 for an arg max);
     ``b_nk``: B is stored [batch, N, K].  ``fused``: 1 best path, 2 on-chip interpreter, 0 row program, GENERATED (3) the
     kernel compiled for this program (the first call compiles it: seconds)."""
-    batched = A.dim() == 3
-    batch = A.shape[0] if batched else 1
-    M, K = A.shape[-2], A.shape[-1]
-    N = B.shape[-2] if b_nk else B.shape[-1]
-    shape = make_gemm_shape(batch, M, N, K, A.stride(-2), B.stride(-2), Y.stride(-2),
-                            A.stride(0) if batched else None, B.stride(0) if batched else None, Y.stride(0) if batched else None,
-                            flags=FLAG_B_ROW_MAJOR_NK if b_nk else 0)
-    n = max(1, len(params))
-    pp = (c_void_p * n)(*[None if t is None else t.data_ptr() for t in params])
-    ld = (c_int64 * n)(*[0 if (t is None or t.dim() < 2) else t.stride(-2) for t in params])
-    ro = (c_void_p * max(1, len(row_out)))(*[t.data_ptr() for t in row_out])
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    st = lib().comfuse_gemm_spec(byref(spec), byref(shape), _ptr(A), _ptr(B), _ptr(Y), pp, ld, ro, int(fused),
-                                 ws_ptr, ws_bytes, _stream(stream))
+    st = (_bind or _bound()).gemm_spec(A, B, Y, ctypes.addressof(spec), params, row_out, fused, b_nk, workspace,
+                                          _current_stream if stream is None else stream)
     if st != OK:
         raise ComfuseError(st, "comfuse_gemm_spec")
     return Y

@@ -6,6 +6,8 @@
 kernels' bounds predicates are compiled in; a predicate that fails records COMFUSE_ERR_BOUNDS in the device status word and
 the access is skipped.  COMFUSE_LIB=<path> makes the Python binding load that library instead of libcomfuse.so.
 
+_binding.so (csrc/binding.c, the argument marshalling of the Python entry points) is built beside the library.
+
 Each translation unit is compiled in parallel to build/obj/*.o and linked into
 paper_2608_03537_b200/libcomfuse.so.  A unit is rebuilt when it, or any header in
 csrc/ or include/, is newer than its object.  The kernel headers are also embedded in the library as text
@@ -16,6 +18,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
@@ -23,6 +26,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(ROOT, "build", "obj")
 LIB_PATH = os.path.join(PKG_DIR, "libcomfuse.so")
+BINDING_PATH = os.path.join(PKG_DIR, "_binding.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -98,10 +102,25 @@ def _compile(src: str, obj: str, verbose: bool, checked: bool = False) -> None:
         raise RuntimeError(f"nvcc failed on {src}")
 
 
+def build_binding(force: bool = False) -> str:
+    """The argument-marshalling extension of the Python entry points (host code, one C file)."""
+    src = os.path.join(CSRC, "binding.c")
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(ROOT, "include", "comfuse.h")))
+    if force or not os.path.exists(BINDING_PATH) or os.path.getmtime(BINDING_PATH) < newest:
+        cmd = [os.environ.get("CC") or "gcc", "-O2", "-shared", "-fPIC", "-std=c11", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+               src, "-o", BINDING_PATH]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            sys.stderr.write(r.stdout + r.stderr)
+            raise RuntimeError(f"compiling {src} failed")
+    return BINDING_PATH
+
+
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
     obj_dir = OBJ_DIR + "_checked" if checked else OBJ_DIR
     lib_path = os.path.join(PKG_DIR, "libcomfuse_checked.so") if checked else LIB_PATH
     os.makedirs(obj_dir, exist_ok=True)
+    build_binding(force)
     sources = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
     hdr_m = _newest_header_mtime()
     jobs, objs = [], []

@@ -254,6 +254,7 @@ void disk_cache_store(const std::string& path, const CompiledKernel& k) {
 
 std::mutex g_cache_mutex;
 std::unordered_map<std::string, std::unique_ptr<CompiledKernel>> g_cache;     // key: instance name + constant table
+std::unordered_map<std::string, CompiledKernel*> g_recent;                      // key: program bytes, N, contraction
 std::unordered_map<std::string, std::string> g_failed;                         // key -> reason (not retried)
 
 }  // namespace
@@ -289,6 +290,23 @@ cudaError_t launch_compiled_program(const GemmMaps& maps, const FusedParams& p, 
   // the last bit, towards the exact value.  COMFUSE_GENERATED_FMAD=0 compiles without contraction: bit-identical results.
   const char* fmad = std::getenv("COMFUSE_GENERATED_FMAD");
   const bool contract = !(fmad && fmad[0] == '0');
+  // The kernels a process has used lately, by the program's bytes (row-output pointers apart), so that a call does not write
+  // the program's source text out to find its kernel again (about 4 us).  Bounded: cleared when it is full; the kernels
+  // themselves stay in g_cache.
+  StageProgram bytes = p.program;
+  for (auto& o : bytes.out) o.ptr = nullptr;
+  std::string quick(reinterpret_cast<const char*>(&bytes), sizeof(bytes));
+  quick.append(reinterpret_cast<const char*>(&p.N), sizeof(p.N));
+  quick.push_back(contract ? 1 : 0);
+  {
+    std::unique_lock<std::mutex> lock(g_cache_mutex);
+    const auto it = g_recent.find(quick);
+    if (it != g_recent.end() && (!launch || it->second->kernel)) {
+      CompiledKernel* k = it->second;
+      lock.unlock();
+      return launch ? launch_pair_kernel(reinterpret_cast<const void*>(k->kernel), k->max_clusters, sh, name, maps, p, st) : cudaSuccess;
+    }
+  }
   const std::string table = constant_table(p.program);
   const std::string key = std::string(name) + (contract ? "\n" : " no-contraction\n") + table;
   CompiledKernel* k = nullptr;
@@ -325,9 +343,11 @@ cudaError_t launch_compiled_program(const GemmMaps& maps, const FusedParams& p, 
       }
     }
   }
-  if (!launch) return cudaSuccess;
   {
     std::lock_guard<std::mutex> lock(g_cache_mutex);
+    if (g_recent.size() >= 64) g_recent.clear();
+    g_recent[quick] = k;
+    if (!launch) return cudaSuccess;
     if (!k->kernel) {
       if (cudaLibraryLoadData(&k->library, k->image.data(), nullptr, nullptr, 0, nullptr, nullptr, 0) != cudaSuccess) return cudaGetLastError();
       if (cudaLibraryGetKernel(&k->kernel, k->library, k->lowered_name.c_str()) != cudaSuccess) return cudaGetLastError();

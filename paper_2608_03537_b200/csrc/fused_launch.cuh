@@ -75,11 +75,15 @@ template <int EPI, int BNS0, int BNS1, int CN, int NSTAGES, int LOCK = 0, int EP
 cudaError_t launch_pair_instance(const GemmMaps& maps, const FusedParams& p, cudaStream_t stream) {
   using Cfg = PairCfg<EPI, BNS0, BNS1, CN, NSTAGES, LOCK, EPW>;
   static std::atomic<int> max_clusters[kMaxLaunchDevices];
-  char what[96];
-  std::snprintf(what, sizeof(what), "epi=%d bns=%d+%d cn=%d stages=%d lock=%d epw=%d, %d staging boxes/warp", EPI, BNS0, BNS1, CN, NSTAGES, LOCK,
-                EPW, Cfg::YBOXES);
+  struct What {  // (named once, not on every launch)
+    char text[96];
+    What() {
+      std::snprintf(text, sizeof(text), "epi=%d bns=%d+%d cn=%d stages=%d lock=%d epw=%d, %d staging boxes/warp", EPI, BNS0, BNS1, CN, NSTAGES, LOCK, EPW, Cfg::YBOXES);
+    }
+  };
+  static const What what;
   return launch_pair_kernel(reinterpret_cast<const void*>(&fused_pair_kernel<EPI, BNS0, BNS1, CN, NSTAGES, LOCK, EPW>), max_clusters,
-                            PairLaunchShape{Cfg::kThreads, Cfg::SMEM_BYTES, 2 * CN}, what, maps, p, stream);
+                            PairLaunchShape{Cfg::kThreads, Cfg::SMEM_BYTES, 2 * CN}, what.text, maps, p, stream);
 }
 
 // The stage-program instantiations (tile widths, cluster size, pipeline depth, lock-step) by row length N:

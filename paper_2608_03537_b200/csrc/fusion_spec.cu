@@ -1000,12 +1000,8 @@ comfuse_status_t comfuse_gemm_spec_prepare(const comfuse_fusion_spec_t* spec, co
   return prepare_compiled_program(shape->N, dc.stage_prog);
 }
 
-comfuse_status_t comfuse_gemm_spec_workspace_size(const comfuse_fusion_spec_t* spec, const comfuse_gemm_shape_t* shape, int32_t fused,
-                                                  size_t* bytes) {
-  if (!bytes || fused < 0 || fused > 3) return COMFUSE_ERR_INVALID_ARG;
-  Decision dc;
-  comfuse_status_t s = decide(spec, shape, fused, dc);
-  if (s != COMFUSE_OK) return s;
+// Workspace bytes of a decided program.
+static comfuse_status_t decided_workspace(const Decision& dc, const comfuse_gemm_shape_t* shape, int32_t fused, size_t* bytes) {
   if (fused == 3 && !dc.on_chip) return COMFUSE_ERR_UNSUPPORTED;
   if (dc.fused) {
     *bytes = dc.fused_inner_ws + dc.fused_scratch;
@@ -1018,10 +1014,18 @@ comfuse_status_t comfuse_gemm_spec_workspace_size(const comfuse_fusion_spec_t* s
   RowProgram P;
   std::memset(&P, 0, sizeof(P));
   int ni, ns;
-  s = lower_row_program(dc.an, shape->N, P, ni, ns);
+  const comfuse_status_t s = lower_row_program(dc.an, shape->N, P, ni, ns);
   if (s != COMFUSE_OK) return s;
   *bytes = static_cast<size_t>(shape->batch) * shape->M * shape->N * 2;
   return COMFUSE_OK;
+}
+
+comfuse_status_t comfuse_gemm_spec_workspace_size(const comfuse_fusion_spec_t* spec, const comfuse_gemm_shape_t* shape, int32_t fused,
+                                                  size_t* bytes) {
+  if (!bytes || fused < 0 || fused > 3) return COMFUSE_ERR_INVALID_ARG;
+  Decision dc;
+  const comfuse_status_t s = decide(spec, shape, fused, dc);
+  return s == COMFUSE_OK ? decided_workspace(dc, shape, fused, bytes) : s;
 }
 
 comfuse_status_t comfuse_gemm_spec(const comfuse_fusion_spec_t* spec, const comfuse_gemm_shape_t* shape, const void* A, const void* B,
@@ -1054,7 +1058,7 @@ comfuse_status_t comfuse_gemm_spec(const comfuse_fusion_spec_t* spec, const comf
     if (!row_out || !row_out[r]) return COMFUSE_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(Y)) & 15u) return COMFUSE_ERR_ALIGNMENT;
   size_t need = 0;
-  s = comfuse_gemm_spec_workspace_size(spec, shape, fused, &need);
+  s = decided_workspace(dc, shape, fused, &need);
   if (s != COMFUSE_OK) return s;
   if (need > 0 && (!workspace || workspace_bytes < need)) return COMFUSE_ERR_WORKSPACE;
   if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 15u)) return COMFUSE_ERR_ALIGNMENT;

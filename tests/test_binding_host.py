@@ -1,0 +1,53 @@
+"""The argument-marshalling extension: descriptors read from tensors' shapes and strides, refusals, argument conversions.  Host
+only: shapes, strides and addresses of CPU tensors, no call reaches a kernel."""
+import pytest
+import torch
+
+import paper_2608_03537_b200 as cf
+
+bf = torch.bfloat16
+
+
+def _fields(d):
+    return {n: getattr(d, n) for n, _ in d._fields_}
+
+
+@pytest.mark.parametrize("nk", [False, True])
+@pytest.mark.parametrize("batch", [None, 1, 3])
+def test_descriptor_follows_shapes_and_strides(batch, nk):
+    M, N, K = 5, 24, 16
+    lead = () if batch is None else (batch,)
+    A = torch.zeros(*lead, M, K + 8, dtype=bf)[..., :K]                       # leading dimension K + 8
+    B = torch.zeros(*lead, *((N, K + 16) if nk else (K, N)), dtype=bf)[..., : K if nk else N]
+    Y, R = torch.zeros(*lead, M, N + 8, dtype=bf)[..., :N], torch.zeros(*lead, M, N, dtype=bf)
+    d = cf.make_gemm_desc(A, B, Y, cf.EPI_BIAS_RES_LAYERNORM, residual=R, alpha=2, eps=0.25, fused=[], flags=(cf.FLAG_B_ROW_MAJOR_NK if nk else 0) | cf.FLAG_POST_RELU)
+    ldb = K + 16 if nk else N
+    want = dict(batch=batch or 1, M=M, N=N, K=K, lda=K + 8, ldb=ldb, ldr=N, ldy=N + 8, batch_stride_a=M * (K + 8), batch_stride_b=(N if nk else K) * ldb,
+                batch_stride_r=M * N, batch_stride_y=M * (N + 8), kind=0, mask=0, alpha=2.0, eps=0.25, fused=0,
+                flags=(4 if nk else 0) | 1, softcap=0.0, reserved=0)
+    assert _fields(d) == want
+    d = cf.make_gemm_desc(A, B, Y, cf.EPI_SCALE_MASK_SOFTMAX, mask=cf.MASK_CAUSAL, softcap=1.5, flags=cf.FLAG_B_ROW_MAJOR_NK if nk else 0)
+    assert (d.ldr, d.batch_stride_r, d.kind, d.mask, d.softcap, d.fused) == (N, M * N, 2, 1, 1.5, 1)
+    assert d.eps == torch.tensor(1e-5).item()
+
+
+def test_what_the_python_side_refuses():
+    A, B, Y = torch.zeros(5, 16, dtype=bf), torch.zeros(16, 24, dtype=bf), torch.zeros(5, 24, dtype=bf)
+    for bad in ((A, B.mT, Y), (A, B, Y[:, :16]), (A.mT, B, Y), (torch.zeros(16, 5, dtype=bf).mT, B, Y)):
+        with pytest.raises(AssertionError):
+            cf.make_gemm_desc(*bad, 0)
+    with pytest.raises(IndexError):
+        cf.make_gemm_desc(A[0], B, Y, 0)
+    with pytest.raises(TypeError):
+        cf.make_gemm_desc(A, B, Y, 0, alpha="1")
+    with pytest.raises(AttributeError):
+        cf.gemm_epilogue(A, B, 3, 0)
+    W2 = torch.zeros(24, 16, dtype=bf)
+    with pytest.raises(AssertionError):
+        cf.b2b_mlp_relu(A, B, None, W2, None, torch.zeros(5, 8, dtype=bf))     # O of another width
+    with pytest.raises(AssertionError):
+        cf.b2b_gemm(A, B, None, torch.zeros(16, 24, dtype=bf).mT, None, Y)      # not dense
+    with pytest.raises(ValueError):
+        cf.b2b_gemm(A[None], B, None, W2, None, Y)
+    with pytest.raises(AssertionError):
+        cf.b2b_attention(torch.zeros(2, 5, 16, dtype=bf), torch.zeros(2, 16, 24, dtype=bf), torch.zeros(2, 25, 16, dtype=bf), torch.zeros(2, 5, 16, dtype=bf), alpha=1.0)
