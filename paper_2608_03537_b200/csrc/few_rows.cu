@@ -685,7 +685,10 @@ FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_bloc
   // or the tile kernel is ahead (1024 x 1024 x 64 10.8 / 9.3, 2048 x 768 x 64 8.9 / 9.4, 2048 x 1024 x 1024 19.4 / 20.9).
   // Softmax kind, one round (row or cluster kernel / this one, K = 64): 8 x 64 x 512 11.0 / 4.4, 2 x 1024 x 1024 12.7 / 6.7,
   // 140 x 64 x 128 11.6 / 5.4; two rounds: 16 x 512 x 512 causal 10.6 / 12.8, 2 x 1171 x 1176 masked 11.4 / 12.5.
-  for (c.nt = 1; c.nt <= 2; ++c.nt) {
+  // Two tiles per CTA halve the CTAs where one does not fit: 3000 x 512 x 768 16.3 / 10.1, 2000 x 768 x 1536 18.7 / 14.1, level from
+  // K = 3072 on.  Not for normalised rows of up to 256 columns, which the tile kernel holds in one CTA pair (5923 x 256 x 256
+  // 7.9 / 7.8, x 1536 14.1 / 15.7).
+  for (c.nt = 1; c.nt <= (N <= 256 && epi != EPI_SOFTMAX ? 1 : 2); ++c.nt) {
     c.ct = c.wide ? 2 : (N + 128 * c.nt - 1) / (128 * c.nt);
     if (c.ct > 16 || clusters > resident_clusters(c.ct, dev)) {
       if (c.wide) return none;
