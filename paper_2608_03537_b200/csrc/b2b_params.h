@@ -9,6 +9,7 @@ namespace comfuse {
 struct B2bParams {
   int M, K, N1, N2;
   int mblocks, mpairs;  // 128-row blocks and pairs of them (per batch)
+  int item_rows;        // attention form: query rows per work item, 128 or 256 (mpairs counts the items of a batch)
   int batch;            // attention form: X, W1, W2, O are [batch, ., .]; MLP form: 1
   int mode;             // 0: F = GELU(. + b1), tail = + b2 + X, LayerNorm; 1: F = softmax(alpha * .), tail = none;
                         // 2: F = ReLU(. + b1), tail = ReLU(. + b2) (the streamed-K kernel)
