@@ -438,7 +438,7 @@ def measure(name, args, env, full):
         roof["kernel"] = {cf.SPEC_PATH_FUSED_KERNEL: "fused_pair_kernel (compiled kind)", cf.SPEC_PATH_FUSED_PROGRAM: "fused_pair_kernel<EPI_PROGRAM> (generated for the program)" if generated else "fused_pair_kernel<EPI_PROGRAM> (on-chip interpreter)",
                           cf.SPEC_PATH_ROW_PROGRAM: "fused_pair_kernel<EPI_NONE> + row_program_kernel"}[plan.path if fused else cf.SPEC_PATH_ROW_PROGRAM]
     elif b2b:
-        roof["kernel"] = "b2b_stream_kernel" if relu_mlp else ("b2b_attention_kernel" if attention else "b2b_mlp_kernel")
+        roof["kernel"] = "b2b_stream_kernel" if relu_mlp else ("b2b_pair_kernel" if attention else "b2b_mlp_kernel")
     elif w.kind == wl.KIND_SCALE_MASK_SOFTMAX and d["K"] <= 256:
         roof["kernel"] = "softmax_rows_kernel"      # short K: score chunks computed twice, no cluster exchange
     elif fused and ws_bytes > 0:

@@ -9,7 +9,7 @@ namespace comfuse {
 struct B2bParams {
   int M, K, N1, N2;
   int mblocks, mpairs;  // 128-row blocks and pairs of them (per batch)
-  int item_rows;        // attention form: query rows per work item, 128 or 256 (mpairs counts the items of a batch)
+  int item_rows;        // attention form in 128-row tiles: query rows per work item, 128 or 256 (mpairs counts the items of a batch)
   int batch;            // attention form: X, W1, W2, O are [batch, ., .]; MLP form: 1
   int mode;             // 0: F = GELU(. + b1), tail = + b2 + X, LayerNorm; 1: F = softmax(alpha * .), tail = none;
                         // 2: F = ReLU(. + b1), tail = ReLU(. + b2) (the streamed-K kernel)
@@ -29,8 +29,10 @@ struct B2bParams {
 };
 
 bool b2b_fused_supported(int K, int N1, int N2, int mode);
-// the attention form (b2b_gemm.cu)
+// the attention form: CTA pairs and 256-position sub-tiles (b2b_gemm.cu), which hands short sources and few queries on to
+// 128-position blocks (b2b_attention.cu)
 cudaError_t launch_b2b_fused(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st);
+cudaError_t launch_b2b_attention(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st);
 // the MLP form (GELU, + b2 + X, LayerNorm) with the four stages on warps of their own (b2b_mlp.cu)
 bool b2b_mlp_supported(int K, int N1, int N2);
 cudaError_t launch_b2b_mlp(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st);
