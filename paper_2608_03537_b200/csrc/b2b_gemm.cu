@@ -561,7 +561,7 @@ cudaError_t launch_b2b_fused(const void* X, const void* W1, const void* W2, B2bP
   // Short sources would fill a 256-position sub-tile with masked ones, and few queries of many batches a second round of
   // 256-row pairs with rows that do not exist: both take the form in 128-position blocks and 128-row tiles.  (One round of
   // longer sources stays here: 7 x 96 queries of 216 keys 6.8 us against 7.1 in blocks; 83 x 35 of 320 13.9 against 9.0.)
-  if (p.N1 <= 128 || (p.M <= 128 && p.batch > dev->sm_count / 2)) return launch_b2b_attention(X, W1, W2, p, st);
+  if (p.N1 <= 128 || (p.M <= 128 && p.form_units > dev->sm_count / 2)) return launch_b2b_attention(X, W1, W2, p, st);
   CUtensorMap tmX, tmW1, tmW2, tmO;
   const uint64_t M = p.M, K = p.K, N1 = p.N1, N2 = p.N2;
   if (p.batch < 1) p.batch = 1;

@@ -10,6 +10,8 @@ struct B2bParams {
   int M, K, N1, N2;
   int mblocks, mpairs;  // 128-row blocks and pairs of them (per batch)
   int item_rows;        // attention form in 128-row tiles: query rows per work item, 128 or 256 (mpairs counts the items of a batch)
+  int form_units;       // rows (MLP forms) or batches (attention form) of the whole call: the choice of kernel follows them, so that
+                        // a call cut into ranges gives the bits of the uncut one
   int batch;            // attention form: X, W1, W2, O are [batch, ., .]; MLP form: 1
   int mode;             // 0: F = GELU(. + b1), tail = + b2 + X, LayerNorm; 1: F = softmax(alpha * .), tail = none;
                         // 2: F = ReLU(. + b1), tail = ReLU(. + b2) (the streamed-K kernel)
@@ -39,5 +41,9 @@ cudaError_t launch_b2b_mlp(const void* X, const void* W1, const void* W2, B2bPar
 // the ReLU MLP form with K streamed through the first GEMM (b2b_stream.cu)
 bool b2b_stream_supported(int K, int N1, int N2);
 cudaError_t launch_b2b_stream(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st);
+
+// the GELU + LayerNorm MLP form for few rows, the hidden layer side by side in a cluster (few_rows_mlp.cu): does a call of M rows take it?
+bool few_rows_mlp_fits(int M, int N1, int N2);
+cudaError_t launch_few_rows_mlp(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st);
 
 }  // namespace comfuse

@@ -642,6 +642,15 @@ comfuse_status_t comfuse_b2b_workspace_size(const comfuse_b2b_desc_t* desc, size
 comfuse_status_t comfuse_b2b_gemm(const comfuse_b2b_desc_t* desc, const void* X, const void* W1, const void* b1,
                                   const void* W2, const void* b2, const void* gamma, const void* beta, void* O,
                                   void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  return b2b_gemm_units(desc, X, W1, b1, W2, b2, gamma, beta, O, workspace, workspace_bytes, cuda_stream,
+                        !desc ? 0 : desc->kind == COMFUSE_B2B_SOFTMAX_ATTENTION ? desc->batch : desc->M);
+}
+
+}  // extern "C"
+
+comfuse_status_t comfuse::b2b_gemm_units(const comfuse_b2b_desc_t* desc, const void* X, const void* W1, const void* b1,
+                                  const void* W2, const void* b2, const void* gamma, const void* beta, void* O,
+                                  void* workspace, size_t workspace_bytes, void* cuda_stream, int form_units) {
   comfuse_status_t s = validate_b2b_desc(desc);
   if (s != COMFUSE_OK) return s;
   if (!X || !W1 || !W2 || !O) return COMFUSE_ERR_INVALID_ARG;
@@ -666,6 +675,7 @@ comfuse_status_t comfuse_b2b_gemm(const comfuse_b2b_desc_t* desc, const void* X,
   if (desc->fused) {
     B2bParams bp = {};
     bp.M = M; bp.K = K; bp.N1 = N1; bp.N2 = N2;
+    bp.form_units = form_units;
     bp.batch = desc->batch; bp.mode = attention ? 1 : (relu_mlp ? 2 : 0); bp.alpha = desc->alpha;
     bp.keys_row_major = (desc->flags & COMFUSE_B2B_FLAG_KEYS_ROW_MAJOR) ? 1 : 0;
     bp.eps = desc->eps;
@@ -681,7 +691,9 @@ comfuse_status_t comfuse_b2b_gemm(const comfuse_b2b_desc_t* desc, const void* X,
     if (const char* tp = std::getenv("COMFUSE_TRACE_PTR")) bp.trace = reinterpret_cast<unsigned long long*>(std::strtoull(tp, nullptr, 0));
     if (const char* tf = std::getenv("COMFUSE_TRACE_FLAGS")) bp.trace_flags = std::atoi(tf);
 #endif
-    cudaError_t e = relu_mlp ? launch_b2b_stream(X, W1, W2, bp, st)
+    const bool few = !attention && !relu_mlp && few_rows_mlp_fits(form_units, N1, N2);
+    cudaError_t e = few ? launch_few_rows_mlp(X, W1, W2, bp, st)
+                    : relu_mlp ? launch_b2b_stream(X, W1, W2, bp, st)
                     : attention ? launch_b2b_fused(X, W1, W2, bp, st)
                                 : launch_b2b_mlp(X, W1, W2, bp, st);
     return e == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
@@ -748,6 +760,8 @@ comfuse_status_t comfuse_b2b_gemm(const comfuse_b2b_desc_t* desc, const void* X,
   r.Y = static_cast<uint16_t*>(O); r.ldy = N2;
   return launch_row_epilogue(EPI_LN, r, st) == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
 }
+
+extern "C" {
 
 comfuse_status_t comfuse_last_device_status(void* cuda_stream) {
   const DeviceInfo* dev = nullptr;

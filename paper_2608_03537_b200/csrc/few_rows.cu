@@ -55,25 +55,6 @@ struct FewRowsCfg {
   static_assert(SMEM_BYTES <= 232448 && SMEM_BYTES > 116 * 1024, "one CTA per SM (tensor-memory allocation never waits)");
 };
 
-// 8 consecutive fp32 columns of this thread's lane; the wait names the registers so that no use moves in front of it
-__device__ __forceinline__ void tmem_ld_issue_8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait_8(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
-               :
-               : "memory");
-}
-// Bulk copy of this CTA's shared memory into a peer's, counted on a barrier of the peer.
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_cluster),
-               "r"(src), "r"(bytes), "r"(bar_cluster)
-               : "memory");
-}
 // Merge R rows' partials (a[i], b[i]) over the 32 lanes.  At step s (lane distance 16 >> s) a lane keeps one half of the rows
 // it still holds and hands the other half to its partner, so R rows take R - 1 + (5 - log2 R) exchanges instead of 5 R.
 // The result for row transposed_row<R>(lane) ends up in a[0], b[0].  merge(step, a0, a1, b0, b1): own partial, partner's.

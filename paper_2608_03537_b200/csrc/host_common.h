@@ -100,6 +100,10 @@ namespace comfuse {
 // call's, so that a call cut into row ranges gives the bits of the uncut one.
 comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void* A, const void* B, void* Y, const comfuse_epilogue_args_t* args,
                                     void* workspace, size_t workspace_bytes, void* cuda_stream, int form_rows);
+// comfuse_b2b_gemm on some of the `form_units` rows (MLP kinds) or batches (attention kind) of a call, likewise.
+comfuse_status_t b2b_gemm_units(const comfuse_b2b_desc_t* desc, const void* X, const void* W1, const void* b1, const void* W2, const void* b2,
+                                const void* gamma, const void* beta, void* O, void* workspace, size_t workspace_bytes, void* cuda_stream,
+                                int form_units);
 // Y = stage program(A . B) with the on-chip interpreter (EPI_PROGRAM).  `vecs` = the up to three row-vector parameters
 // the program's CHO_ROWVEC operands index, `residual` = its full-tensor parameter or null.  `query_only`: just say
 // whether an instantiation exists for N (no device is touched).

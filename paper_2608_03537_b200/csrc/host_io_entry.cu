@@ -287,9 +287,9 @@ extern "C" comfuse_status_t comfuse_b2b_gemm_host(const comfuse_b2b_desc_t* desc
       if (attn) dc.batch = static_cast<int32_t>(n);
       else dc.M = static_cast<int32_t>(n);
       unsigned char* wsc = workspace ? static_cast<unsigned char*>(workspace) + u0 * ws_unit : nullptr;
-      s = comfuse_b2b_gemm(&dc, dX + u0 * ux, attn ? static_cast<const void*>(dW1 + u0 * u1) : W1, b1,
+      s = comfuse::b2b_gemm_units(&dc, dX + u0 * ux, attn ? static_cast<const void*>(dW1 + u0 * u1) : W1, b1,
                            attn ? static_cast<const void*>(dW2 + u0 * u2) : W2, b2, gamma, beta, dO + u0 * uo, wsc,
-                           wsc ? workspace_bytes - u0 * ws_unit : 0, cuda_stream);
+                           wsc ? workspace_bytes - u0 * ws_unit : 0, cuda_stream, static_cast<int>(units));
       if (s != COMFUSE_OK) return rejoin(s);
       if (cudaEventRecord(pipe->computed[c], st) != cudaSuccess || cudaStreamWaitEvent(pipe->out, pipe->computed[c], 0) != cudaSuccess)
         return rejoin(COMFUSE_ERR_CUDA);
