@@ -13,8 +13,10 @@ bool softmax_rows_supported(const FusedParams& p) { return p.K <= 256 && p.N >= 
 cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_t stream) {
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
-  auto kern = p.mask ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true> : softmax_rows_kernel<NSTAGES, YBOXES, false, true>)
-                     : (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, false>);
+  const bool resident = p.mask && p.N <= 2 * Cfg::CHUNK;
+  auto kern = resident ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true, true> : softmax_rows_kernel<NSTAGES, YBOXES, false, true, true>)
+              : p.mask ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, true, false>)
+                       : (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, false, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, false, false>);
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
   constexpr int kMaxDev = 64;
@@ -42,8 +44,9 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
   int ncl = max_clusters[di].load(std::memory_order_acquire);
   if (ncl == 0) {
     cudaError_t e = cudaSuccess;
-    for (auto k : {softmax_rows_kernel<NSTAGES, YBOXES, false, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, false>,
-                   softmax_rows_kernel<NSTAGES, YBOXES, false, true>, softmax_rows_kernel<NSTAGES, YBOXES, true, true>}) {
+    for (auto k : {softmax_rows_kernel<NSTAGES, YBOXES, false, false, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, false, false>,
+                   softmax_rows_kernel<NSTAGES, YBOXES, false, true, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, true, false>,
+                   softmax_rows_kernel<NSTAGES, YBOXES, false, true, true>, softmax_rows_kernel<NSTAGES, YBOXES, true, true, true>}) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
       if (e != cudaSuccess) return e;
     }

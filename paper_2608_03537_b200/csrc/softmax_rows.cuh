@@ -61,10 +61,14 @@ struct RowSoftmaxCfg {
 // UMMA, like A) instead of [K, N] (two boxes of 64 contraction rows x 64 columns, MN-major).
 // ADD: an additive mask tensor [M, N].  A thread owns a row of the chunk, so reading the mask straight from global memory
 // touches 32 rows per load instruction (32 sectors for 512 bytes, in both passes): 96 batches of 504 x 504 scores took 47.0 us
-// that way, 36.3 with the boxes below.  Every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
+// that way, 36.3 with the boxes below (33.5 with RES).  Every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
 // take the result: read the box, overwrite it with the probabilities, store it.  The warp's elected lane asks for the box
 // of the unit after next as soon as a box is free, and issues the store itself (no barrier round trip through other warps).
-template <int NSTAGES, int YBOXES, bool BKM, bool ADD>
+// RES (with ADD): rows of at most 512 columns.  Both chunks of the row stay in their accumulator slots: pass 0 writes the finished
+// scores (capped, scaled, masked, log2 domain, fp32) back over the accumulators and pass 1 only exponentiates them -- one UMMA, one
+// mask box and one soft-cap per chunk instead of two.  Device time without / with: 96 x 504 x 504 35.7 / 33.5 us, 40 x 512 x 512
+// 23.5 / 21.6, 8 x 1379 x 424 14.4 / 13.0.  What is left is the exponentials of both passes and the 4 KB stores.
+template <int NSTAGES, int YBOXES, bool BKM, bool ADD, bool RES>
 __global__ void __launch_bounds__(32 * 20, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
@@ -160,7 +164,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int b, mpair0, L;
         if (!tile_at(r, b, mpair0, L)) continue;
         const int m0 = mpair0 + static_cast<int>(pm) * 128;
-        for (int u = 0; u < 2 * L && ok; ++u) {
+        for (int u = 0; u < (RES ? 1 : 2) * L && ok; ++u) {
         const int c = u < L ? u : u - L;  // pass 0 over the live chunks, then pass 1
         for (int kb = 0; kb < KB; ++kb) {
           if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) { ok = false; break; }  // passes on a fresh barrier
@@ -194,7 +198,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       uint32_t total_units = 0;
       for (int r = 0; r < rounds; ++r) {
         int b, mpair0, L;
-        if (tile_at(r, b, mpair0, L)) total_units += 2u * L;
+        if (tile_at(r, b, mpair0, L)) total_units += (RES ? 1u : 2u) * L;
       }
       while (ok && unit < total_units) {
         const int slot = static_cast<int>(unit & 1u);
@@ -342,7 +346,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     auto request_mask = [&]() {
       if (load_c >= my_chunks) {
         load_c = 0;
-        load_pass1 = !load_pass1;
+        load_pass1 = !RES && !load_pass1;
         if (!load_pass1 && load_r < rounds) {
           int lb, lm = 0, lL;
           if (++load_r < rounds && !tile_at(load_r, lb, lm, lL)) load_r = rounds;
@@ -350,7 +354,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
       if (my_chunks <= 0 || load_r >= rounds) return;
-      const uint32_t sel = load_n % YBOXES;
+      const uint32_t sel = RES ? (my_chunks == 2 ? static_cast<uint32_t>(load_c) : 0u) : load_n % YBOXES;
       mbar_arrive_expect_tx(bar_yfull(e, sel), Cfg::WARP_BOX_BYTES);
       tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_yfull(e, sel), load_c * CHUNK + h * 64, load_row, 0, keep_mask);
       ++load_n;
@@ -360,9 +364,19 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if constexpr (ADD) {
       elected = elect_one();
       if (elected)
-        for (int i = 0; i < YBOXES; ++i) request_mask();
+        for (int i = 0; i < (RES && my_chunks < YBOXES ? my_chunks : YBOXES); ++i) request_mask();
       __syncwarp();
     }
+    // the previous unit's box, once its store has read it, takes the mask of the unit after this one
+    auto reclaim_box = [&]() {
+      if (!store_pending) return;
+      if (elected) {
+        tma_store_wait_read<0>();
+        if (!RES || my_chunks == 2) request_mask();
+      }
+      __syncwarp();
+      store_pending = false;
+    };
     // 32 mask values of half `half` of this thread's row of the box, as log2-domain addends
     auto box_mask = [&](uint32_t box, int half, float2 (&m2)[16]) {
 #pragma unroll
@@ -396,24 +410,20 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           // 2 = all 32 columns live for all 32 rows, 0 = none live for any row, 1 = mixed
           auto frag_state = [&](int col0) { return col0 + 31 <= lim_lo ? 2 : (col0 > lim_hi ? 0 : 1); };
 
-          const int slot = static_cast<int>(unit & 1u);
-          ++unit;
-          wait_slot(slot);
+          const int slot = static_cast<int>((RES && pass == 1 ? unit - static_cast<uint32_t>(L - c) : unit) & 1u);
+          if (!RES || pass == 0) {
+            ++unit;
+            wait_slot(slot);
+          }
           const uint32_t taddr = tmem_base + lane_sel + slot * CHUNK + h * 64;
           const int colg = c * CHUNK + h * 64;
-          const uint32_t msel = mask_n % YBOXES;
+          // RES: the masks of a row of two chunks take a box each, which pass 1 then fills; of one chunk box 0, pass 1 fills box 1
+          const uint32_t msel = !RES ? mask_n % YBOXES : my_chunks == 2 ? static_cast<uint32_t>(c) : (pass == 0 ? 0u : 1u);
           const uint32_t mbox = ybox0 + msel * Cfg::WARP_BOX_BYTES;
           if constexpr (ADD) {
-            if (store_pending) {  // the previous unit's box: read out by now, it takes the mask of the unit after this one
-              if (elected) {
-                tma_store_wait_read<0>();
-                request_mask();
-              }
-              __syncwarp();
-              store_pending = false;
-            }
-            if (colg < p.N) {
-              mbar_wait<false>(bar_yfull(e, msel), (mask_n / YBOXES) & 1u, w);
+            if (!RES || pass == 0) reclaim_box();
+            if (colg < p.N && (!RES || pass == 0)) {
+              mbar_wait<false>(bar_yfull(e, msel), (RES && my_chunks < 2 ? mask_n : mask_n / YBOXES) & 1u, w);
               __syncwarp();
               ++mask_n;
             }
@@ -448,6 +458,14 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                   if (col0 + 2 * j + 1 > lim) tv[j].y = -INFINITY;
                 }
               }
+              if constexpr (RES) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                  v[2 * j] = __float_as_uint(tv[j].x);
+                  v[2 * j + 1] = __float_as_uint(tv[j].y);
+                }
+                tmem_st_32cols(taddr + half * 32, v);
+              }
               float mx0 = m_run, mx1 = -INFINITY;
 #pragma unroll
               for (int j = 0; j < 16; j += 2) {
@@ -469,9 +487,11 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 m_run = m_new;
               }
             }
-            release_slot(slot);
-            if (ADD && colg < p.N) {  // (release_slot converged the warp behind its reads)
-              if (elected) request_mask();
+            if constexpr (RES) tmem_st_wait();
+            else release_slot(slot);
+            if (ADD && colg < p.N) {
+              __syncwarp();  // every lane has read its row of the box
+              if (elected && (!RES || my_chunks < 2)) request_mask();
               __syncwarp();
             }
           } else {
@@ -487,12 +507,18 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
               } else {
                 uint32_t v[32];
                 tmem_ld_32cols(taddr + half * 32, v);
-                if (capped) {
+                if (!RES && capped) {
 #pragma unroll
                   for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
                 }
                 float2 ev[16];
-                if (additive) {
+                if constexpr (RES) {
+#pragma unroll
+                  for (int j = 0; j < 16; ++j) {  // (a masked score is -inf, and so is -inf - off: its probability is an exact zero)
+                    const float2 t01 = add2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(-off));
+                    ev[j] = make_float2(ex2_approx(t01.x), ex2_approx(t01.y));
+                  }
+                } else if constexpr (additive) {
                   float2 m2[16];
                   box_mask(mbox, half, m2);
 #pragma unroll
@@ -519,6 +545,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
               }
             }
             release_slot(slot);
+            if (RES) reclaim_box();  // (no accumulator wait in front of this unit: the store has had the arithmetic's time instead)
             if (colg < p.N) {
               const uint32_t sel = ADD ? msel : nbox % YBOXES;
               const uint32_t ybox = ybox0 + sel * Cfg::WARP_BOX_BYTES;
