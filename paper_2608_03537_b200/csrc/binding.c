@@ -35,6 +35,17 @@ static int to_i64(PyObject* o, int64_t* out) {  // int(o); wraps like a C intege
   Py_DECREF(v);
   return !PyErr_Occurred();
 }
+static int to_f64(PyObject* o, double* out) {  // float(o): numbers, tensors of one element, texts
+  if (PyFloat_CheckExact(o)) {
+    *out = PyFloat_AS_DOUBLE(o);
+    return 1;
+  }
+  PyObject* v = PyNumber_Float(o);
+  if (!v) return 0;
+  *out = PyFloat_AS_DOUBLE(v);
+  Py_DECREF(v);
+  return 1;
+}
 static int tuple_i64(PyObject* t, int64_t* out, int* n) {
   PyObject* seq = t ? PySequence_Fast(t, "a shape or stride") : NULL;
   Py_XDECREF(t);
@@ -142,12 +153,8 @@ static int fill_desc(PyObject* const* a, comfuse_gemm_desc_t* d) {
     d->batch_stride_r = batched ? R.stride[0] : M * d->ldr;
   }
   if (!to_i64(a[3], &kind) || !to_i64(a[7], &mask)) return 0;
-  const double alpha = PyFloat_AsDouble(a[5]);
-  if (alpha == -1.0 && PyErr_Occurred()) return 0;
-  const double eps = PyFloat_AsDouble(a[6]);
-  if (eps == -1.0 && PyErr_Occurred()) return 0;
-  const double softcap = PyFloat_AsDouble(a[10]);
-  if (softcap == -1.0 && PyErr_Occurred()) return 0;
+  double alpha, eps, softcap;
+  if (!to_f64(a[5], &alpha) || !to_f64(a[6], &eps) || !to_f64(a[10], &softcap)) return 0;
   const int fused = PyObject_IsTrue(a[8]);
   if (fused < 0) return 0;
   d->kind = (int32_t)kind;
@@ -219,10 +226,8 @@ static PyObject* py_b2b(PyObject* self, PyObject* const* a, Py_ssize_t n) {
       return NULL;
   }
   if (!contiguous(a[1]) || !contiguous(a[2]) || !contiguous(a[4]) || !contiguous(a[8])) return NULL;
-  const double eps = PyFloat_AsDouble(a[9]);
-  if (eps == -1.0 && PyErr_Occurred()) return NULL;
-  const double alpha = PyFloat_AsDouble(a[10]);
-  if (alpha == -1.0 && PyErr_Occurred()) return NULL;
+  double eps, alpha;
+  if (!to_f64(a[9], &eps) || !to_f64(a[10], &alpha)) return NULL;
   const int fused = PyObject_IsTrue(a[11]);
   if (fused < 0) return NULL;
   d.M = (int32_t)M;

@@ -38,8 +38,9 @@ def test_what_the_python_side_refuses():
             cf.make_gemm_desc(*bad, 0)
     with pytest.raises(IndexError):
         cf.make_gemm_desc(A[0], B, Y, 0)
-    with pytest.raises(TypeError):
-        cf.make_gemm_desc(A, B, Y, 0, alpha="1")
+    for bad, why in (("one", ValueError), ([], TypeError), (None, TypeError)):
+        with pytest.raises(why):
+            cf.make_gemm_desc(A, B, Y, 0, alpha=bad)
     with pytest.raises(AttributeError):
         cf.gemm_epilogue(A, B, 3, 0)
     W2 = torch.zeros(24, 16, dtype=bf)
@@ -51,3 +52,12 @@ def test_what_the_python_side_refuses():
         cf.b2b_gemm(A[None], B, None, W2, None, Y)
     with pytest.raises(AssertionError):
         cf.b2b_attention(torch.zeros(2, 5, 16, dtype=bf), torch.zeros(2, 16, 24, dtype=bf), torch.zeros(2, 25, 16, dtype=bf), torch.zeros(2, 5, 16, dtype=bf), alpha=1.0)
+
+
+def test_scalars_are_taken_as_float_takes_them():
+    import numpy as np
+    cf.lib()
+    A, B, Y = torch.zeros(5, 16, dtype=bf), torch.zeros(16, 24, dtype=bf), torch.zeros(5, 24, dtype=bf)
+    for v in (2, 0.25, "0.25", True, np.float32(0.5), np.array(1.5), torch.tensor(3.0)):
+        d = cf.make_gemm_desc(A, B, Y, cf.EPI_SCALE_MASK_SOFTMAX, alpha=v, eps=v, softcap=v)
+        assert (d.alpha, d.eps, d.softcap) == (float(v),) * 3
