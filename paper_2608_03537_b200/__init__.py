@@ -179,17 +179,23 @@ def lib() -> ctypes.CDLL:
         L.comfuse_launch_count.restype = c_uint64
         L.comfuse_status_string.argtypes = [c_int32]
         L.comfuse_status_string.restype = ctypes.c_char_p
-        from . import _binding as b   # built with the library (csrc/binding.c)
-        b.bind(*(ctypes.cast(f, c_void_p).value for f in (L.comfuse_gemm_epilogue, L.comfuse_b2b_gemm, L.comfuse_gemm_spec)))
-        _bind = b
+        try:
+            from . import _binding as b   # built with the library (csrc/binding.c)
+            b.bind(*(ctypes.cast(f, c_void_p).value for f in (L.comfuse_gemm_epilogue, L.comfuse_b2b_gemm, L.comfuse_gemm_spec)))
+            _bind = b
+        except ImportError:
+            _bind = None   # the calls that need it say so (_bound); everything else works without
         _lib = L
     return _lib
 
 
 def _bound():
-    """The argument-marshalling extension, with the library's entry points in it."""
+    """The argument-marshalling extension, with the library's entry points in it.  Fails loudly if absent."""
     if _bind is None:
         lib()
+    if _bind is None:
+        raise ImportError("the _binding extension of paper_2608_03537_b200 was not built for this Python: build it first "
+                          "(python -m paper_2608_03537_b200.build)")
     return _bind
 
 
@@ -217,7 +223,26 @@ def make_gemm_desc(A, B, Y, kind, *, residual=None, alpha=1.0, eps=1e-5, mask=MA
                    softcap=0.0) -> GemmDesc:
     """Describe A [b, M, K] (or [M, K]), B [b, K, N] (or [K, N]; with FLAG_B_ROW_MAJOR_NK in ``flags``: [b, N, K]),
     Y [b, M, N] from torch tensors' shapes and strides."""
-    return GemmDesc.from_buffer_copy(_bound().gemm_desc(A, B, Y, kind, residual, alpha, eps, mask, fused, flags, softcap))
+    if _bind is not None:   # (the same in native code, a third of the time)
+        return GemmDesc.from_buffer_copy(_bind.gemm_desc(A, B, Y, kind, residual, alpha, eps, mask, fused, flags, softcap))
+    batched = A.dim() == 3
+    batch = A.shape[0] if batched else 1
+    M, K = A.shape[-2], A.shape[-1]
+    b_nk = bool(int(flags) & FLAG_B_ROW_MAJOR_NK)
+    N = B.shape[-2] if b_nk else B.shape[-1]
+    assert (B.shape[-1] if b_nk else B.shape[-2]) == K and Y.shape[-2] == M and Y.shape[-1] == N
+    assert A.stride(-1) == 1 and B.stride(-1) == 1 and Y.stride(-1) == 1
+    d = GemmDesc()
+    d.batch, d.M, d.N, d.K = batch, M, N, K
+    d.lda, d.ldb, d.ldy = A.stride(-2), B.stride(-2), Y.stride(-2)
+    d.ldr = residual.stride(-2) if residual is not None else N
+    d.batch_stride_a = A.stride(0) if batched else M * d.lda
+    d.batch_stride_b = B.stride(0) if batched else (N if b_nk else K) * d.ldb
+    d.batch_stride_y = Y.stride(0) if batched else M * d.ldy
+    d.batch_stride_r = (residual.stride(0) if batched else M * d.ldr) if residual is not None else M * N
+    d.kind, d.mask, d.alpha, d.eps, d.fused, d.reserved = int(kind), int(mask), float(alpha), float(eps), int(bool(fused)), 0
+    d.flags, d.softcap = int(flags), float(softcap)
+    return d
 
 
 def workspace_size(desc: GemmDesc) -> int:

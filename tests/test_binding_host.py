@@ -1,5 +1,9 @@
 """The argument-marshalling extension: descriptors read from tensors' shapes and strides, refusals, argument conversions.  Host
 only: shapes, strides and addresses of CPU tensors, no call reaches a kernel."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -61,3 +65,62 @@ def test_scalars_are_taken_as_float_takes_them():
     for v in (2, 0.25, "0.25", True, np.float32(0.5), np.array(1.5), torch.tensor(3.0)):
         d = cf.make_gemm_desc(A, B, Y, cf.EPI_SCALE_MASK_SOFTMAX, alpha=v, eps=v, softcap=v)
         assert (d.alpha, d.eps, d.softcap) == (float(v),) * 3
+
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _child(code, **env):
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, PYTHONPATH=ROOT, **env), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-1000:] + r.stderr[-3000:]
+
+
+def test_without_the_extension_only_the_calls_that_need_it_refuse():
+    _child("""
+import sys
+sys.modules["paper_2608_03537_b200._binding"] = None      # as if it had not been built
+import torch, paper_2608_03537_b200 as cf
+A, B, Y = torch.zeros(5, 16, dtype=torch.bfloat16), torch.zeros(16, 24, dtype=torch.bfloat16), torch.zeros(5, 24, dtype=torch.bfloat16)
+d = cf.make_gemm_desc(A, B, Y, cf.EPI_BIAS_RES_LAYERNORM, fused=False)
+assert cf.workspace_size(d) == 5 * 24 * 2 and cf.launch_count() == 0
+try:
+    cf.gemm_epilogue(A, B, Y, cf.EPI_BIAS_RES_LAYERNORM)
+except ImportError as e:
+    assert "python -m paper_2608_03537_b200.build" in str(e), e
+else:
+    raise SystemExit("not refused")
+""")
+
+
+def test_a_descriptor_needs_no_library():
+    _child("""
+import torch, paper_2608_03537_b200 as cf
+z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16)
+args = [(z(3, 5, 24)[..., :16], z(3, 16, 24), z(3, 5, 24), 0, dict(residual=z(3, 5, 32)[..., :24], flags=1)),
+        (z(5, 16), z(24, 16), z(5, 24), 2, dict(mask=1, flags=4, softcap=2, alpha=0.5, fused=[])), (z(5, 16), z(16, 24), z(5, 24), 1, dict(eps=1))]
+fields = lambda d: {n: getattr(d, n) for n, _ in d._fields_}
+assert cf._bind is None
+plain = [fields(cf.make_gemm_desc(*a[:4], **a[4])) for a in args]
+assert cf._bind is None
+try:
+    cf.lib()
+except ImportError:
+    pass
+else:
+    raise SystemExit("the library was to be absent")
+""".replace("", ""), COMFUSE_LIB="/nonexistent/libcomfuse.so")
+
+
+def test_both_ways_to_a_descriptor_agree():
+    z = lambda *s: torch.zeros(*s, dtype=bf)  # noqa: E731
+    native = cf._bound()
+    for A, B, Y, kind, kw in ((z(3, 5, 24)[..., :16], z(3, 16, 24), z(3, 5, 24), 0, dict(residual=z(3, 5, 32)[..., :24], flags=1)),
+                              (z(5, 16), z(24, 16), z(5, 24), 2, dict(mask=1, flags=4, softcap=2, alpha=0.5, fused=[])),
+                              (z(1, 2, 5, 16), z(16, 24), z(5, 24), 1, dict(eps=1))):
+        a = _fields(cf.make_gemm_desc(A, B, Y, kind, **kw))
+        cf._bind = None
+        try:
+            b = _fields(cf.make_gemm_desc(A, B, Y, kind, **kw))
+        finally:
+            cf._bind = native
+        assert a == b
