@@ -6,7 +6,8 @@
 kernels' bounds predicates are compiled in; a predicate that fails records COMFUSE_ERR_BOUNDS in the device status word and
 the access is skipped.  COMFUSE_LIB=<path> makes the Python binding load that library instead of libcomfuse.so.
 
-_binding.so (csrc/binding.c, the argument marshalling of the Python entry points) is built beside the library.
+_binding.<Python's tag>.so (csrc/binding.c, the argument marshalling of the Python entry points) is built beside the library, with
+the C compiler ($CC, else gcc) and the headers of the Python that runs this; another Python version does not load it.
 
 Each translation unit is compiled in parallel to build/obj/*.o and linked into
 paper_2608_03537_b200/libcomfuse.so.  A unit is rebuilt when it, or any header in
@@ -26,7 +27,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(ROOT, "build", "obj")
 LIB_PATH = os.path.join(PKG_DIR, "libcomfuse.so")
-BINDING_PATH = os.path.join(PKG_DIR, "_binding.so")
+BINDING_PATH = os.path.join(PKG_DIR, "_binding" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -106,8 +107,14 @@ def build_binding(force: bool = False) -> str:
     """The argument-marshalling extension of the Python entry points (host code, one C file)."""
     src = os.path.join(CSRC, "binding.c")
     newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(ROOT, "include", "comfuse.h")))
+    untagged = os.path.join(PKG_DIR, "_binding.so")   # what a build once wrote: any Python version would load it
+    if untagged != BINDING_PATH and os.path.exists(untagged):
+        os.remove(untagged)
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        raise RuntimeError(f"{include}/Python.h not found: the headers of this Python are needed to compile {src}")
     if force or not os.path.exists(BINDING_PATH) or os.path.getmtime(BINDING_PATH) < newest:
-        cmd = [os.environ.get("CC") or "gcc", "-O2", "-shared", "-fPIC", "-std=c11", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+        cmd = [os.environ.get("CC") or "gcc", "-O2", "-shared", "-fPIC", "-std=c11", "-I", include, "-I", os.path.join(ROOT, "include"),
                src, "-o", BINDING_PATH]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:

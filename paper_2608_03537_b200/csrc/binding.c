@@ -1,4 +1,4 @@
-// Argument marshalling of the Python entry points, as a CPython extension (_binding.so).
+// Argument marshalling of the Python entry points, as a CPython extension (_binding.<tag>.so).
 //
 // A call of a small problem is bound by the time its Python caller spends on it: building the descriptor field by field
 // through ctypes, wrapping every pointer and asking for the current stream took 9 of the 13.5 us that a 16 x 256 x 64

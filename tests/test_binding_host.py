@@ -124,3 +124,12 @@ def test_both_ways_to_a_descriptor_agree():
         finally:
             cf._bind = native
         assert a == b
+
+
+def test_the_extension_carries_the_tag_of_its_python():
+    import importlib.machinery
+
+    from paper_2608_03537_b200 import build
+    tag = importlib.machinery.EXTENSION_SUFFIXES[0]
+    assert "cpython" in tag and build.BINDING_PATH.endswith("_binding" + tag)
+    assert cf._bound().__file__ == build.BINDING_PATH and not os.path.exists(os.path.join(build.PKG_DIR, "_binding.so"))
