@@ -253,15 +253,38 @@ static PyObject* py_b2b(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   return PyLong_FromLong((long)st);
 }
 
+// A sequence of tensors (something with a length: a generator's tensors would be gone before the launch is enqueued), held for the
+// length of a call, and zeroed room for `arrays` 8-byte values of each.  The library reads as many entries as the program
+// names, so there is room for the most that a program can name, however few were given.
+#define MIN_ROOM (COMFUSE_SPEC_MAX_PARAMS > COMFUSE_SPEC_MAX_ROW_OUTPUTS ? COMFUSE_SPEC_MAX_PARAMS : COMFUSE_SPEC_MAX_ROW_OUTPUTS)
+typedef struct {
+  PyObject* seq;
+  Py_ssize_t n, room;
+  int64_t* values;
+} Held;
+static int hold(PyObject* o, int arrays, Held* h) {
+  if (PyObject_Size(o) < 0) return 0;
+  h->seq = PySequence_Fast(o, "a sequence of tensors is expected");
+  if (!h->seq) return 0;
+  h->n = PySequence_Fast_GET_SIZE(h->seq);
+  h->room = h->n > MIN_ROOM ? h->n : MIN_ROOM;
+  h->values = PyMem_Calloc((size_t)(h->room * arrays), sizeof(int64_t));
+  if (!h->values) PyErr_NoMemory();
+  return h->values != NULL;
+}
+static void let_go(Held* h) {
+  PyMem_Free(h->values);
+  Py_XDECREF(h->seq);
+}
+
 // gemm_spec(A, B, Y, address of the comfuse_fusion_spec_t, params, row_out, fused, b_nk, workspace, stream) -> status
-#define MAX_TENSORS 64
-static PyObject* py_gemm_spec(PyObject* self, PyObject* const* a, Py_ssize_t n) {
+static int gemm_spec_call(PyObject* const* a, Held* params, Held* rows, comfuse_status_t* st) {
   Geometry A, B, Y;
   comfuse_gemm_shape_t s;
   int64_t spec, fused;
-  if (!fixed_args(n, 10, "gemm_spec") || !geometry(a[0], &A) || !geometry(a[1], &B) || !geometry(a[2], &Y) || !to_i64(a[3], &spec) || !to_i64(a[6], &fused)) return NULL;
+  if (!geometry(a[0], &A) || !geometry(a[1], &B) || !geometry(a[2], &Y) || !to_i64(a[3], &spec) || !to_i64(a[6], &fused)) return 0;
   const int b_nk = PyObject_IsTrue(a[7]);
-  if (b_nk < 0) return NULL;
+  if (b_nk < 0) return 0;
   const int batched = A.n == 3;
   memset(&s, 0, sizeof(s));
   const int64_t M = A.size[A.n - 2], K = A.size[A.n - 1], N = B.size[B.n - (b_nk ? 2 : 1)];
@@ -276,48 +299,38 @@ static PyObject* py_gemm_spec(PyObject* self, PyObject* const* a, Py_ssize_t n) 
   s.batch_stride_b = batched && B.stride[0] ? B.stride[0] : (b_nk ? N : K) * s.ldb;
   s.batch_stride_y = batched && Y.stride[0] ? Y.stride[0] : M * s.ldy;
   s.flags = b_nk ? COMFUSE_FLAG_B_ROW_MAJOR_NK : 0;
-  const void* params[MAX_TENSORS] = {0};
-  int64_t ld[MAX_TENSORS] = {0};
-  void* rows[MAX_TENSORS] = {0};
-  PyObject* seq = PySequence_Fast(a[4], "params must be a sequence");
-  if (!seq) return NULL;
-  Py_ssize_t np = PySequence_Fast_GET_SIZE(seq);
-  if (np > MAX_TENSORS) np = MAX_TENSORS;  // (the library reads no more than COMFUSE_SPEC_MAX_PARAMS of them)
-  int ok = 1;
-  for (Py_ssize_t i = 0; ok && i < np; ++i) {
-    PyObject* t = PySequence_Fast_GET_ITEM(seq, i);
+  if (!hold(a[4], 2, params) || !hold(a[5], 1, rows)) return 0;
+  int64_t* ld = params->values + params->room;
+  for (Py_ssize_t i = 0; i < params->n; ++i) {
+    PyObject* t = PySequence_Fast_GET_ITEM(params->seq, i);
     int64_t dims = 0;
     Geometry g;
-    ok = pointer(t, params + i);
-    if (!ok || t == Py_None) continue;
-    ok = method_i64(t, s_dim, &dims);
-    if (ok && dims >= 2) {
-      ok = geometry(t, &g);
-      ld[i] = ok ? g.stride[g.n - 2] : 0;
-    }
+    if (t == Py_None) continue;
+    if (!method_i64(t, s_data_ptr, params->values + i) || !method_i64(t, s_dim, &dims)) return 0;
+    if (dims < 2) continue;
+    if (!geometry(t, &g)) return 0;
+    ld[i] = g.stride[g.n - 2];
   }
-  Py_DECREF(seq);
-  if (!ok) return NULL;
-  seq = PySequence_Fast(a[5], "row_out must be a sequence");
-  if (!seq) return NULL;
-  Py_ssize_t nr = PySequence_Fast_GET_SIZE(seq);
-  if (nr > MAX_TENSORS) nr = MAX_TENSORS;
-  for (Py_ssize_t i = 0; ok && i < nr; ++i) {
-    int64_t v = 0;
-    ok = method_i64(PySequence_Fast_GET_ITEM(seq, i), s_data_ptr, &v);
-    rows[i] = (void*)(uintptr_t)v;
-  }
-  Py_DECREF(seq);
-  if (!ok) return NULL;
+  for (Py_ssize_t i = 0; i < rows->n; ++i)
+    if (!method_i64(PySequence_Fast_GET_ITEM(rows->seq, i), s_data_ptr, rows->values + i)) return 0;
   const void *pA, *pB, *pY;
   void *ws, *stream;
   size_t ws_bytes;
-  if (!workspace_of(a[8], &ws, &ws_bytes) || !pointer(a[0], &pA) || !pointer(a[1], &pB) || !pointer(a[2], &pY) || !stream_of(a[9], &stream)) return NULL;
-  comfuse_status_t st;
+  if (!workspace_of(a[8], &ws, &ws_bytes) || !pointer(a[0], &pA) || !pointer(a[1], &pB) || !pointer(a[2], &pY) || !stream_of(a[9], &stream)) return 0;
   Py_BEGIN_ALLOW_THREADS
-  st = f_gemm_spec((const comfuse_fusion_spec_t*)(uintptr_t)spec, &s, pA, pB, (void*)pY, params, ld, rows, (int32_t)fused, ws, ws_bytes, stream);
+  *st = f_gemm_spec((const comfuse_fusion_spec_t*)(uintptr_t)spec, &s, pA, pB, (void*)pY, (const void* const*)params->values, ld, (void* const*)rows->values,
+                    (int32_t)fused, ws, ws_bytes, stream);
   Py_END_ALLOW_THREADS
-  return PyLong_FromLong((long)st);
+  return 1;
+}
+static PyObject* py_gemm_spec(PyObject* self, PyObject* const* a, Py_ssize_t n) {
+  Held params = {0}, rows = {0};
+  comfuse_status_t st;
+  if (!fixed_args(n, 10, "gemm_spec")) return NULL;
+  const int ok = gemm_spec_call(a, &params, &rows, &st);
+  let_go(&params);
+  let_go(&rows);
+  return ok ? PyLong_FromLong((long)st) : NULL;
 }
 
 // bind(address of comfuse_gemm_epilogue, of comfuse_b2b_gemm, of comfuse_gemm_spec): the loaded library's entry points

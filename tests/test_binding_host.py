@@ -133,3 +133,87 @@ def test_the_extension_carries_the_tag_of_its_python():
     tag = importlib.machinery.EXTENSION_SUFFIXES[0]
     assert "cpython" in tag and build.BINDING_PATH.endswith("_binding" + tag)
     assert cf._bound().__file__ == build.BINDING_PATH and not os.path.exists(os.path.join(build.PKG_DIR, "_binding.so"))
+
+
+class _Recorder:
+    """Stands in for comfuse_gemm_spec behind the binding, so that no call reaches the library: what it was given, and INVALID_ARG."""
+
+    def __init__(self):
+        import ctypes as c
+        proto = c.CFUNCTYPE(c.c_int32, c.c_void_p, c.c_void_p, c.c_void_p, c.c_void_p, c.c_void_p, c.POINTER(c.c_uint64), c.POINTER(c.c_int64),
+                            c.POINTER(c.c_uint64), c.c_int32, c.c_void_p, c.c_size_t, c.c_void_p)
+        self.seen = []
+        self.count = 12
+        self.during = lambda: None
+        self.fn = proto(self.call)
+
+    def call(self, spec, shape, A, B, Y, params, ld, rows, fused, ws, ws_bytes, stream):
+        self.during()
+        self.seen.append((params[: self.count], ld[: self.count], rows[:8], stream))
+        return cf.ERR_INVALID_ARG
+
+    def __enter__(self):
+        import ctypes as c
+        L, b = cf.lib(), cf._bound()
+        at = lambda f: c.cast(f, c.c_void_p).value  # noqa: E731
+        b.bind(at(L.comfuse_gemm_epilogue), at(L.comfuse_b2b_gemm), at(self.fn))
+        return self
+
+    def __exit__(self, *exc):
+        import ctypes as c
+        L = cf.lib()
+        cf._bound().bind(*(c.cast(f, c.c_void_p).value for f in (L.comfuse_gemm_epilogue, L.comfuse_b2b_gemm, L.comfuse_gemm_spec)))
+
+
+class _Stream:
+    cuda_stream = 77
+
+
+def _spec_call(**kw):
+    z = lambda *s: torch.zeros(*s, dtype=bf)  # noqa: E731
+    spec = cf.make_spec([("acc", -1, -1, -1, 0.0)], 0)
+    kw = dict(dict(spec=spec, stream=_Stream()), **kw)
+    with pytest.raises(cf.ComfuseError) as e:
+        cf.gemm_spec(z(5, 16), z(16, 24), z(5, 24), kw.pop("spec"), **kw)
+    assert e.value.status == cf.ERR_INVALID_ARG
+
+
+def test_parameter_lists_have_a_length_and_are_passed_whole():
+    many = [torch.zeros(3, 8, dtype=bf)[:, : 4 + i % 2] if i % 3 else None for i in range(70)]
+    with _Recorder() as r:
+        r.count = 70
+        _spec_call(params=many, row_out=tuple(t for t in many if t is not None))
+        params, ld, rows, _ = r.seen.pop()
+        assert params == [0 if t is None else t.data_ptr() for t in many] and ld == [0 if t is None else 8 for t in many]
+        assert rows == [t.data_ptr() for t in many if t is not None][:8]
+        r.count = 12                                 # fewer than a program can name: the others are null
+        _spec_call(params={"bias": many[1]}.values())
+        assert r.seen.pop()[0] == [many[1].data_ptr()] + [0] * 11
+        _spec_call()
+        assert r.seen.pop()[:3] == ([0] * 12, [0] * 12, [0] * 8)
+        for bad in (dict(params=(t for t in many)), dict(row_out=(t for t in many[1:2])), dict(params=3), dict(row_out=None)):
+            with pytest.raises(TypeError):
+                _spec_call(**bad)
+        assert not r.seen
+
+
+def test_tensors_of_a_sequence_live_until_the_launch_is_enqueued():
+    import gc
+    import weakref
+
+    class Fresh:                                     # makes its tensors as it is read
+        def __len__(self):
+            return 1
+
+        def __getitem__(self, i):
+            if i:
+                raise IndexError
+            t = torch.zeros(24, dtype=bf)
+            refs.append(weakref.ref(t))
+            return t
+
+    refs, alive = [], []
+    with _Recorder() as r:
+        r.during = lambda: (gc.collect(), alive.extend(w() is not None for w in refs))
+        _spec_call(params=Fresh(), row_out=Fresh())
+    assert alive == [True, True]
