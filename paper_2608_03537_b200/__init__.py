@@ -470,6 +470,8 @@ def gemm_spec(A, B, Y, spec: FusionSpec, *, params=(), row_out=(), fused=True, w
     (row vectors [N], tensors [batch, M, N]), ``row_out`` the per-row output tensors (fp32, int32 for an arg max);
     ``b_nk``: B is stored [batch, N, K].  ``fused``: 1 best path, 2 on-chip interpreter, 0 row program, GENERATED (3) the
     kernel compiled for this program (the first call compiles it: seconds)."""
+    if not isinstance(spec, FusionSpec):   # (its address is all that the extension gets)
+        raise ctypes.ArgumentError(f"spec: a FusionSpec from make_spec is expected, got {type(spec).__name__}")
     st = (_bind or _bound()).gemm_spec(A, B, Y, ctypes.addressof(spec), params, row_out, fused, b_nk, workspace,
                                           _current_stream if stream is None else stream)
     if st != OK:

@@ -217,3 +217,12 @@ def test_tensors_of_a_sequence_live_until_the_launch_is_enqueued():
         r.during = lambda: (gc.collect(), alive.extend(w() is not None for w in refs))
         _spec_call(params=Fresh(), row_out=Fresh())
     assert alive == [True, True]
+
+
+def test_only_a_program_is_taken_for_a_program():
+    import ctypes
+    with _Recorder() as r:
+        for bad in (cf.make_gemm_shape(1, 5, 24, 16), ctypes.c_int64(0), 0, None):
+            with pytest.raises((ctypes.ArgumentError, TypeError)):
+                _spec_call(spec=bad)
+        assert not r.seen
