@@ -109,9 +109,9 @@ static int require(int cond, const char* what) {
   if (!cond) PyErr_SetString(PyExc_AssertionError, what);
   return cond;
 }
-// a stream object, or a callable that returns the current stream's handle
+// a stream object (which may be callable), or the function that returns the current stream's handle
 static int stream_of(PyObject* s, void** out) {
-  PyObject* v = PyCallable_Check(s) ? PyObject_CallNoArgs(s) : PyObject_GetAttr(s, s_cuda_stream);
+  PyObject* v = PyFunction_Check(s) ? PyObject_CallNoArgs(s) : PyObject_GetAttr(s, s_cuda_stream);
   int64_t h = 0;
   if (!v) return 0;
   const int ok = to_i64(v, &h);

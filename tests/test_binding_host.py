@@ -226,3 +226,13 @@ def test_only_a_program_is_taken_for_a_program():
             with pytest.raises((ctypes.ArgumentError, TypeError)):
                 _spec_call(spec=bad)
         assert not r.seen
+
+
+def test_a_stream_object_may_be_callable():
+    class Callable(_Stream):
+        def __call__(self):
+            return 13
+
+    with _Recorder() as r:
+        _spec_call(stream=Callable())
+        assert r.seen.pop()[3] == 77
