@@ -22,7 +22,7 @@ static b2b_gemm_fn f_b2b_gemm;
 static gemm_spec_fn f_gemm_spec;
 static PyObject *s_data_ptr, *s_shape, *s_stride, *s_dim, *s_is_contiguous, *s_numel, *s_element_size, *s_cuda_stream;
 
-#define MAX_DIMS 8
+#define MAX_DIMS 64  // (tensors have no more)
 typedef struct {
   int n;
   int64_t size[MAX_DIMS], stride[MAX_DIMS];

@@ -236,3 +236,10 @@ def test_a_stream_object_may_be_callable():
     with _Recorder() as r:
         _spec_call(stream=Callable())
         assert r.seen.pop()[3] == 77
+
+
+def test_tensors_of_many_dimensions_describe_their_last_two():
+    cf._bound()
+    one = (1,) * 9
+    d = cf.make_gemm_desc(torch.zeros(*one, 5, 16, dtype=bf), torch.zeros(*one, 16, 24, dtype=bf), torch.zeros(*one, 5, 24, dtype=bf), 0)
+    assert (d.batch, d.M, d.N, d.K, d.lda, d.ldb, d.ldy) == (1, 5, 24, 16, 16, 24, 24)
