@@ -260,6 +260,13 @@ uint64_t comfuse_launch_count(void);
  * expired or aborted wait (all 64). */
 comfuse_status_t comfuse_selftest_bounded_wait(uint32_t timeout_ms, void* cuda_stream, uint32_t* expired_waits);
 
+/* Failure-detection self-test (the paper has no counterpart).  Launches one cluster of two CTAs; one waits, with a limit of
+ * `timeout_ms` (1..300), for a copy that the other sends only after that limit.  The wait must expire (status word
+ * COMFUSE_ERR_TIMEOUT), and the CTA must still be there when the copy lands.  Synchronises the stream; `*seen` (a HOST pointer)
+ * receives 1 = the wait expired, 2 / 4 = the receiver / the sender took the way out for expired waits, 8 = the copy landed
+ * before anyone left: 15. */
+comfuse_status_t comfuse_selftest_late_copy(uint32_t timeout_ms, void* cuda_stream, uint32_t* seen);
+
 /* Checked-build self-test (the paper has no counterpart).  Launches one small kernel that evaluates a bounds predicate
  * which is false, in front of an access it therefore skips.  In a library built with -DCOMFUSE_CHECKED the device status
  * word then reads COMFUSE_ERR_BOUNDS; in the ordinary build the predicates are compiled out, the kernel does nothing and

@@ -56,6 +56,7 @@ EXPORTED_SYMBOLS = (
     "comfuse_last_device_status",
     "comfuse_launch_count",
     "comfuse_selftest_bounded_wait",
+    "comfuse_selftest_late_copy",
     "comfuse_status_string",
 )
 
@@ -173,6 +174,8 @@ def lib() -> ctypes.CDLL:
         L.comfuse_last_device_status.restype = c_int32
         L.comfuse_selftest_bounded_wait.argtypes = [ctypes.c_uint32, c_void_p, POINTER(ctypes.c_uint32)]
         L.comfuse_selftest_bounded_wait.restype = c_int32
+        L.comfuse_selftest_late_copy.argtypes = [ctypes.c_uint32, c_void_p, POINTER(ctypes.c_uint32)]
+        L.comfuse_selftest_late_copy.restype = c_int32
         L.comfuse_selftest_bounds_predicate.argtypes = [c_void_p, POINTER(c_int32)]
         L.comfuse_selftest_bounds_predicate.restype = c_int32
         L.comfuse_launch_count.argtypes = []
@@ -491,6 +494,17 @@ def selftest_bounded_wait(timeout_ms: int = 20, stream=None) -> int:
     st = lib().comfuse_selftest_bounded_wait(int(timeout_ms), _stream(stream), byref(n))
     if st != OK:
         raise ComfuseError(st, "comfuse_selftest_bounded_wait")
+    return int(n.value)
+
+
+def selftest_late_copy(timeout_ms: int = 20, stream=None) -> int:
+    """Run the late-copy self-test kernel (a copy between two CTAs that is sent after its receiver's wait has expired): 15 when the wait
+    expired, both CTAs took the way out for expired waits and the copy landed before either left.  The device status word
+    reads ERR_TIMEOUT afterwards."""
+    n = ctypes.c_uint32(0)
+    st = lib().comfuse_selftest_late_copy(int(timeout_ms), _stream(stream), byref(n))
+    if st != OK:
+        raise ComfuseError(st, "comfuse_selftest_late_copy")
     return int(n.value)
 
 

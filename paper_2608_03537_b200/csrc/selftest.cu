@@ -30,6 +30,54 @@ __global__ void bounded_wait_selftest_kernel(unsigned int* status, unsigned long
 
 __device__ unsigned int g_selftest_counter = 0;
 
+// Two CTAs: rank 1 sends 64 bytes to rank 0 only after rank 0's wait for them has expired.  Rank 0 must still be there when they
+// arrive (tell_cluster and mbar_drain, the way out of the kernels whose CTAs send into each other's shared memory).
+__global__ void __cluster_dims__(2, 1, 1) late_copy_selftest_kernel(unsigned int* status, unsigned long long timeout_ns, unsigned int* seen) {
+  __shared__ __align__(16) unsigned int src[16], dst[16];
+  __shared__ unsigned long long bar;
+  __shared__ int abort_flag, told;
+  const uint32_t rank = cluster_ctarank();
+  if (threadIdx.x < 16) {
+    src[threadIdx.x] = 0xC0DE0000u + threadIdx.x;
+    dst[threadIdx.x] = 0u;
+  }
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar), 1);
+    abort_flag = 0;
+    told = 0;
+    fence_mbar_init();
+    mbar_arrive_expect_tx(smem_u32(&bar), rank == 0 ? sizeof(dst) : 0);
+  }
+  fence_proxy_async_smem();
+  __syncthreads();
+  cluster_sync_all();
+  const WaitCtx w{&abort_flag, status, timeout_ns};
+  unsigned int bits = 0;
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    if (rank == 0) {
+      ok = mbar_wait<true>(smem_u32(&bar), 0, w);
+      bits |= ok ? 0u : 1u;
+    } else {
+      const uint64_t t0 = globaltimer_ns();
+      while (globaltimer_ns() - t0 < 2 * timeout_ns) {
+      }
+      bulk_copy_to_peer(map_to_cta(smem_u32(dst), 0), smem_u32(src), sizeof(src), map_to_cta(smem_u32(&bar), 0));
+    }
+  }
+  if (!ok) tell_cluster(&told, 2);
+  __syncthreads();
+  cluster_sync_after_init();
+  if (*static_cast<volatile int*>(&told)) {
+    if (threadIdx.x == 0) {
+      bits |= rank == 0 ? 2u : 4u;  // both CTAs know
+      if (rank == 0 && mbar_drain(smem_u32(&bar), 0, w) && dst[0] == 0xC0DE0000u && dst[15] == 0xC0DE000Fu) bits |= 8u;
+    }
+    cluster_sync_all();
+  }
+  if (bits) atomicOr(seen, bits);
+}
+
 // One element past the end of a 32-element array: the predicate is false, the store is skipped (checked build), or the
 // predicate is compiled out and the kernel's own `false &&` keeps the store from happening (ordinary build).
 __global__ void bounds_predicate_selftest_kernel(unsigned int* status, unsigned int* arr, int n) {
@@ -66,6 +114,22 @@ extern "C" comfuse_status_t comfuse_selftest_bounded_wait(uint32_t timeout_ms, v
     *expired_waits = h;
   }
   return COMFUSE_OK;
+}
+
+extern "C" comfuse_status_t comfuse_selftest_late_copy(uint32_t timeout_ms, void* cuda_stream, uint32_t* seen) {
+  if (!seen || timeout_ms == 0 || timeout_ms > 300) return COMFUSE_ERR_INVALID_ARG;
+  const DeviceInfo* dev = current_device_info();
+  if (!dev) return COMFUSE_ERR_CUDA;
+  if (dev->cc_major != 10) return COMFUSE_ERR_ARCH;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  void* counter = nullptr;
+  if (cudaGetSymbolAddress(&counter, g_selftest_counter) != cudaSuccess) return COMFUSE_ERR_CUDA;
+  if (cudaMemsetAsync(counter, 0, sizeof(unsigned int), st) != cudaSuccess) return COMFUSE_ERR_CUDA;
+  count_launch();
+  late_copy_selftest_kernel<<<2, 64, 0, st>>>(dev->status_word, static_cast<unsigned long long>(timeout_ms) * 1000000ull, static_cast<unsigned int*>(counter));
+  if (cudaGetLastError() != cudaSuccess) return COMFUSE_ERR_CUDA;
+  if (cudaMemcpyAsync(seen, counter, sizeof(*seen), cudaMemcpyDeviceToHost, st) != cudaSuccess) return COMFUSE_ERR_CUDA;
+  return cudaStreamSynchronize(st) == cudaSuccess ? COMFUSE_OK : COMFUSE_ERR_CUDA;
 }
 
 extern "C" comfuse_status_t comfuse_selftest_bounds_predicate(void* cuda_stream, int32_t* checked_build) {

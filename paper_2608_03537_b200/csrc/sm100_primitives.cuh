@@ -165,6 +165,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
   }
 }
 
+// After a wait has expired (mbar_wait then returns at once everywhere in the CTA): wait, with a limit of its own and whatever the
+// abort flag says, for a phase that copies or UMMAs already under way complete.  What they touch -- this CTA's shared and tensor
+// memory -- is handed to the next CTA when this one ends.
+__device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, const WaitCtx& w) {
+  const uint64_t t0 = globaltimer_ns();
+  while (!mbar_try_wait_cluster(bar, parity))
+    if (globaltimer_ns() - t0 > w.timeout_ns) return false;
+  return true;
+}
+
+// A thread whose wait has failed tells every CTA of its cluster (`told`: a shared word of each CTA, zeroed before any peer can
+// write) in front of the cluster barrier at the kernel's end.  Where no wait failed, all that was sent between the CTAs has been
+// waited for by its receiver and that barrier is enough.  Where `told` is set behind it, the sends -- which are issued
+// whatever expired -- may still be under way: the receivers drain them and the cluster meets once more before anyone leaves.
+__device__ __forceinline__ void tell_cluster(volatile int* told, uint32_t cluster_size) {
+  for (uint32_t c = 0; c < cluster_size; ++c)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(smem_u32(const_cast<int*>(told)), c)), "r"(1) : "memory");
+  asm volatile("fence.acq_rel.cluster;" ::: "memory");
+}
+
 // ----------------------------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
