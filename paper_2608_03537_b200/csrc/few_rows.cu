@@ -129,7 +129,6 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   const int KB = (p.K + 63) >> 6;
   const int kb0 = KB * ks / p.ks, kb1 = KB * (ks + 1) / p.ks;
   const WaitCtx w{s_abort, p.status, p.timeout_ns};
-  const uint32_t cluster = static_cast<uint32_t>(p.ct * p.ks);
   griddep_launch_dependents();  // the next kernel's set-up may overlap this kernel (it waits before touching memory)
 
   // -------------------------------------------------------------------------------------------- set-up
@@ -172,7 +171,6 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) {  // passes on a fresh barrier
           *s_issued = kb - kb0;
-          tell_cluster(s_told, cluster);
           break;
         }
         const uint32_t sw = smem_base + stage * Cfg::STAGE_BYTES;
@@ -196,10 +194,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
       const uint32_t wstep = wkm ? 2u : 128u;
       const uint32_t idesc = wkm ? make_idesc_bf16(128, MT, false, false) : make_idesc_bf16(128, MT, true, false);
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait<false>(bar_full(stage), phase, w)) {
-          tell_cluster(s_told, cluster);
-          break;
-        }
+        if (!mbar_wait<false>(bar_full(stage), phase, w)) break;
         tcgen05_fence_after_sync();
         const uint32_t sw = smem_base + stage * Cfg::STAGE_BYTES;
         const uint64_t xdesc = make_smem_desc_sw128(sw + Cfg::W_BYTES, 16, 1024);
@@ -215,6 +210,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
       }
       umma_commit(bar_acc);
+      mbar_drain(bar_acc, 0, w);  // nothing may still be writing tensor memory when it is freed
     }
   } else {
     // ------------------------------------------------------------------------------------------ epilogue warps
@@ -286,7 +282,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     const int my_row = transposed_row<RC>(lane);  // which of the warp's RC rows a reduction leaves in this lane
     const bool gelu = EPI == EPI_RMS_MAX && !p.no_activation;
 
-    bool ok = mbar_wait<false>(bar_acc, 0, w);  // none of this thread's waits has expired
+    mbar_wait<false>(bar_acc, 0, w);
     __syncwarp();
     tcgen05_fence_after_sync();
     // accumulators -> [row][column] in the ring, which nothing uses any more (every load has landed and has been multiplied)
@@ -316,7 +312,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                             smem_base + lane * rs * Cfg::ROW_BYTES, bytes, map_to_cta(bar_recv, peer));
       }
       __syncwarp();
-      ok &= mbar_wait<true>(bar_recv, 0, w);
+      mbar_wait<true>(bar_recv, 0, w);
     } else {
       named_barrier_sync(1, 32 * Cfg::kEpiWarps);
     }
@@ -448,7 +444,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
           st_async_f32x2(map_to_cta(stat_addr + static_cast<uint32_t>((r * 16 + ct) * 8), peer), s0, s1, map_to_cta(bar_stat, peer));
       }
     }
-    ok &= mbar_wait<true>(bar_stat, 0, w);
+    mbar_wait<true>(bar_stat, 0, w);
     __syncwarp();
 
     // ---------------- stage 2: merge the CT partials of the rows (the same order in every CTA), normalise, store
@@ -557,7 +553,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         st_async_f32x2(map_to_cta(max_addr + static_cast<uint32_t>((rm * 16 + ct) * 8), peer), best[0], best_col[0], map_to_cta(bar_max, peer));
       }
       if (ct == 0) {
-        ok &= mbar_wait<true>(bar_max, 0, w);
+        mbar_wait<true>(bar_max, 0, w);
         __syncwarp();
         const float2* s_max = s_stat + Cfg::STAT_BYTES / 8;
         const int r = e + mrow * Cfg::kEpiWarps;
@@ -575,30 +571,33 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         }
       }
     }
-    if (!ok) tell_cluster(s_told, cluster);
   }
 
   // -------------------------------------------------------------------------------------------- teardown
   tcgen05_fence_before_sync();
   __syncthreads();
-  if (warp == 1) {  // (the UMMAs are this CTA's own, and complete unless a wait expired; bar_acc is committed to in every case)
-    if (*s_told) mbar_drain(bar_acc, 0, w);
-    __syncwarp();
-    tcgen05_fence_after_sync();
-    tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
-  }
+  if (threadIdx.x == 0 && *s_abort) tell_cluster(s_told, static_cast<uint32_t>(p.ct * p.ks));
   // No CTA may leave while a peer still sends into its shared memory.  Everything that is sent here has been waited for by
   // its receiver, and a bulk copy's source has been read when its destination counts it: arriving is all that is needed, no
   // flush of this CTA's stores (the release form waited 1000 clocks for the result's stores to reach the L2).
   cluster_sync_after_init();
-  if (*s_told) {  // ... unless a wait expired: loads and the peers' sends may still be under way
-    if (threadIdx.x == 0) {
+  if (warp == 1) {
+    __syncwarp();
+    tcgen05_fence_after_sync();
+    tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
+  }
+  // Unless a wait expired: then loads and the peers' sends, which are issued whatever expired, may still be under way.  (One warp
+  // looks, and meets the other CTAs' once more; the others leave at once.  40 x 4096 x 4096 13.35 -> 13.39 us; with every thread
+  // looking, and the outcomes of its waits carried along, 13.50.)
+  if (warp == 0 && *s_told) {
+    if (lane == 0) {
       const int issued = *s_issued;
       for (int u = issued > NSTAGES ? issued - NSTAGES : 0; u < issued; ++u) mbar_drain(bar_full(u % NSTAGES), (u / NSTAGES) & 1u, w);
       mbar_drain(bar_recv, 0, w);
       mbar_drain(bar_stat, 0, w);
       if (EPI == EPI_RMS_MAX && !p.wide) mbar_drain(bar_max, 0, w);
     }
+    __syncwarp();
     cluster_sync_all();
   }
 }

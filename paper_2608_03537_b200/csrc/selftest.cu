@@ -53,11 +53,9 @@ __global__ void __cluster_dims__(2, 1, 1) late_copy_selftest_kernel(unsigned int
   cluster_sync_all();
   const WaitCtx w{&abort_flag, status, timeout_ns};
   unsigned int bits = 0;
-  bool ok = true;
   if (threadIdx.x == 0) {
     if (rank == 0) {
-      ok = mbar_wait<true>(smem_u32(&bar), 0, w);
-      bits |= ok ? 0u : 1u;
+      if (!mbar_wait<true>(smem_u32(&bar), 0, w)) bits |= 1u;
     } else {
       const uint64_t t0 = globaltimer_ns();
       while (globaltimer_ns() - t0 < 2 * timeout_ns) {
@@ -65,14 +63,15 @@ __global__ void __cluster_dims__(2, 1, 1) late_copy_selftest_kernel(unsigned int
       bulk_copy_to_peer(map_to_cta(smem_u32(dst), 0), smem_u32(src), sizeof(src), map_to_cta(smem_u32(&bar), 0));
     }
   }
-  if (!ok) tell_cluster(&told, 2);
   __syncthreads();
+  if (threadIdx.x == 0 && abort_flag) tell_cluster(&told, 2);
   cluster_sync_after_init();
-  if (*static_cast<volatile int*>(&told)) {
+  if (threadIdx.x < 32 && *static_cast<volatile int*>(&told)) {  // (the other warp leaves at once)
     if (threadIdx.x == 0) {
       bits |= rank == 0 ? 2u : 4u;  // both CTAs know
       if (rank == 0 && mbar_drain(smem_u32(&bar), 0, w) && dst[0] == 0xC0DE0000u && dst[15] == 0xC0DE000Fu) bits |= 8u;
     }
+    __syncwarp();
     cluster_sync_all();
   }
   if (bits) atomicOr(seen, bits);

@@ -175,10 +175,10 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, const 
   return true;
 }
 
-// A thread whose wait has failed tells every CTA of its cluster (`told`: a shared word of each CTA, zeroed before any peer can
-// write) in front of the cluster barrier at the kernel's end.  Where no wait failed, all that was sent between the CTAs has been
-// waited for by its receiver and that barrier is enough.  Where `told` is set behind it, the sends -- which are issued
-// whatever expired -- may still be under way: the receivers drain them and the cluster meets once more before anyone leaves.
+// One thread of a CTA in which a wait has expired tells every CTA of its cluster (`told`: a shared word of each CTA, zeroed before any
+// peer can write) in front of the cluster barrier at the kernel's end.  Where no wait expired, all that was sent between the
+// CTAs has been waited for by its receiver and that barrier is enough.  Where `told` is set behind it, the sends -- which are
+// issued whatever expired -- may still be under way: the receivers drain them and meet once more before they leave.
 __device__ __forceinline__ void tell_cluster(volatile int* told, uint32_t cluster_size) {
   for (uint32_t c = 0; c < cluster_size; ++c)
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(smem_u32(const_cast<int*>(told)), c)), "r"(1) : "memory");
