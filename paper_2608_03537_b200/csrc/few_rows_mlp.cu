@@ -78,6 +78,8 @@ few_rows_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
   const uint32_t bar_recv = bar_d1 + 32u;                 // the peers' shares have arrived
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(smem + Cfg::OFF_MISC);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + Cfg::OFF_MISC + 4);
+  volatile int* s_told = s_abort + 1;    // a wait expired in some CTA of the cluster
+  volatile int* s_issued = s_abort + 2;  // K blocks whose loads are issued (fewer than all where the producer's wait expires)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -104,6 +106,8 @@ few_rows_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     mbar_init(bar_d2, 1);
     mbar_init(bar_recv, 1);
     *s_abort = 0;
+    *s_told = 0;
+    *s_issued = KB;
     fence_mbar_init();
     mbar_arrive_expect_tx(bar_recv, static_cast<uint32_t>((hc - 1) * rv * Cfg::ROW_BYTES));  // armed before any peer can send
     prefetch_tensormap(&tmX);
@@ -127,7 +131,10 @@ few_rows_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
       int stage = 0;
       uint32_t phase = 0;
       for (int kb = 0; kb < KB; ++kb) {
-        if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) break;  // passes on a fresh barrier
+        if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) {  // passes on a fresh barrier
+          *s_issued = kb;
+          break;
+        }
         const uint32_t sw = smem_base + stage * Cfg::STAGE_BYTES;
         mbar_arrive_expect_tx(bar_full(stage), Cfg::STAGE_BYTES);
         tma_load_3d(sw, &tmW1, bar_full(stage), n0, kb * 64, 0);
@@ -172,6 +179,7 @@ few_rows_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
         }
       }
       umma_commit(bar_d2);
+      mbar_drain(bar_d2, 0, w);  // nothing may still be writing tensor memory when it is freed
     }
   } else {
     // ------------------------------------------------------------------------------------------ epilogue warps
@@ -307,11 +315,22 @@ few_rows_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 
   tcgen05_fence_before_sync();
   __syncthreads();
+  if (threadIdx.x == 0 && *s_abort) tell_cluster(s_told, static_cast<uint32_t>(hc));
   cluster_sync_after_init();  // what is sent here has been waited for by its receiver: arriving is enough (see few_rows.cu)
   if (warp == 1) {
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
+  }
+  if (warp == 0 && *s_told) {  // ... unless a wait expired: loads and the peers' sends may still be under way
+    if (lane == 0) {
+      const int issued = *s_issued;
+      for (int u = issued > NSTAGES ? issued - NSTAGES : 0; u < issued; ++u) mbar_drain(bar_full(u % NSTAGES), (u / NSTAGES) & 1u, w);
+      if (issued > 0) mbar_drain(bar_w2, 0, w);
+      mbar_drain(bar_recv, 0, w);
+    }
+    __syncwarp();
+    cluster_sync_all();
   }
 }
 
