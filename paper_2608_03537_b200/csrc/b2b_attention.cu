@@ -3,9 +3,13 @@
 // (b2b_gemm.cu holds the form for longer sources, and the rule that chooses.)
 //
 // What bounds it: the chain scores -> row maximum -> exponentials -> S.V of one row tile, which leaves the tensor core and
-// the MUFU unit (128 x 128 exponentials are 1024 clocks of it) waiting for one another.  A CTA works on TWO tiles of 128 query
-// rows that share their keys and values, and alternates: while one tile's warps exponentiate, the tensor core computes the
-// other tile's scores and S.V.  Source positions come in blocks of 128:
+// the MUFU unit (128 x 128 exponentials are 1024 clocks of it) waiting for one another.  Source positions come in blocks of 128,
+// query rows in tiles of 128, and a CTA's work item is one of two things:
+//
+//   up to 128 positions    TWO tiles that share the one block of keys and values, in alternation: while one tile's warps
+//                          exponentiate, the tensor core computes the other tile's scores and S.V  (tile B's warps idle where the
+//                          second 128 rows do not exist, or where every tile has a CTA of its own)
+//   up to 128 queries      ONE tile, walking the source's blocks  (tile A; tile B's warps idle)
 //
 //   tensor memory    scores of tile A (128 columns), of tile B (128), output of A (128), of B (128)
 //   S                bf16, written over the first half of the tile's own score columns: S.V takes it from tensor memory as its
@@ -18,9 +22,10 @@
 //                    the blocks of consecutive work items form one sequence
 //
 // Measured (device time, CTA-pair form of b2b_gemm.cu / this one): 109 x 1116 queries of 32 keys 28.0 / 16.8 us, 4 x 23 of 64
-// 6.8 / 4.7, 83 x 35 of 320 13.9 / 9.0; but 32 x 4096 of 256 22.3 / 22.8 and 256 x 512 of 512 38.7 / 40.0.  A block of a tile takes
-// 3200 clocks there: scores read 150, row maximum 320, exponentials 1550 (1024 of the MUFU unit), S.V and the next scores 1000;
-// the score UMMAs of single CTAs read both operands from shared memory at its full rate, a pair halves one of them.
+// 6.8 / 4.7, 83 x 35 of 320 13.9 / 9.0.  Two tiles over several blocks (longer sources of more queries) were built too and
+// stay with the pair form, 32 x 4096 of 256 22.3 / 22.8 and 256 x 512 of 512 38.7 / 40.0: a block of a tile took 3200 clocks there
+// (scores read 150, row maximum 320, exponentials 1550, S.V and the next scores 1000), and the score UMMAs of single CTAs
+// read both operands from shared memory at its full rate, where a pair halves one of them.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -52,7 +57,7 @@ struct AttnSmem {
   static constexpr int OFF_KV = OFF_Q + 2 * kBlockBytes;          // ring of key and value blocks
   static constexpr int OFF_OUT = OFF_KV + kKvSlots * kBlockBytes; // two 32 x 64 output boxes per finish warp
   static constexpr int OFF_BAR = OFF_OUT + 8 * 4096;
-  static constexpr int NUM_BARS = 2 * kKvSlots + 10 * 2 + 1;
+  static constexpr int NUM_BARS = 2 * kKvSlots + 9 * 2 + 1;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
   static constexpr int OFF_SUM = OFF_MISC + 16;                   // float [2 tiles][128]: rescaling factors, then row sums
   static constexpr int BYTES = OFF_SUM + 2 * 128 * 4 + 1024;
@@ -104,9 +109,9 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   auto bar_lfull = [&](int t) { return bar_tile + 8u * (6 + t); };   // row sums of the work item written
   auto bar_ofull = [&](int t) { return bar_tile + 8u * (8 + t); };   // output of the work item complete
   auto bar_oempty = [&](int t) { return bar_tile + 8u * (10 + t); }; // output read
-  auto bar_ffull = [&](int t) { return bar_tile + 8u * (16 + t); };  // rescaling factors of a block written
-  auto bar_fdone = [&](int t) { return bar_tile + 8u * (18 + t); };  // output rescaled
-  const uint32_t bar_drain = bar_tile + 8u * 20;
+  const uint32_t bar_ffull = bar_tile + 8u * 16;  // (tile A) rescaling factors of a block written
+  const uint32_t bar_fdone = bar_tile + 8u * 17;  // (tile A) output rescaled
+  const uint32_t bar_drain = bar_tile + 8u * 18;
   float* s_sum = reinterpret_cast<float*>(smem + AttnSmem::OFF_SUM);
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(smem + AttnSmem::OFF_MISC);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + AttnSmem::OFF_MISC + 4);
@@ -149,11 +154,11 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       mbar_init(bar_pfull(t, 0), 4);  // one arrival per softmax warp of the tile
       mbar_init(bar_pfull(t, 1), 4);
       mbar_init(bar_lfull(t), 4);
-      mbar_init(bar_ffull(t), 4);
-      mbar_init(bar_fdone(t), 4);
       mbar_init(bar_ofull(t), 1);
       mbar_init(bar_oempty(t), 4);
     }
+    mbar_init(bar_ffull, 4);
+    mbar_init(bar_fdone, 4);
     mbar_init(bar_drain, 1);
     *s_abort = 0;
     fence_mbar_init();
@@ -223,7 +228,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         constexpr uint32_t idesc_qk = make_idesc_bf16(128, 128, false, !KM);
         constexpr uint32_t idesc_pv = make_idesc_bf16(128, 128, false, true);
         int slot = 0;
-        uint32_t phase = 0, quse[2] = {0, 0}, puse[2] = {0, 0}, ouse[2] = {0, 0}, fuse[2] = {0, 0};
+        uint32_t phase = 0, quse[2] = {0, 0}, puse[2] = {0, 0}, ouse[2] = {0, 0}, fuse = 0;
         bool ok = true;
         // the next slot of the ring, landed; it is handed back (commit) when its last UMMAs have been issued
         auto take_slot = [&](uint32_t& addr) {
@@ -255,9 +260,9 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
           if (j == 0) {
             if (!ok || !mbar_wait<false>(bar_oempty(t), (ouse[t] & 1u) ^ 1u, w)) { ok = false; return; }
             ++ouse[t];
-          } else {
-            if (!ok || !mbar_wait<false>(bar_fdone(t), fuse[t] & 1u, w)) { ok = false; return; }
-            ++fuse[t];
+          } else {  // (tile A: items of several blocks have no tile B)
+            if (!ok || !mbar_wait<false>(bar_fdone, fuse & 1u, w)) { ok = false; return; }
+            ++fuse;
           }
           const uint64_t vd = make_smem_desc_sw128(va, /*next 64 columns*/ kBoxBytes, /*next 8 positions*/ 1024);
 #pragma unroll
@@ -355,9 +360,9 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
           m = ref;
           sum = mul2(sum, splat2(f));
           sum1 = mul2(sum1, splat2(f));
-          s_sum[t * 128 + q * 32 + lane] = f;
+          s_sum[q * 32 + lane] = f;
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_ffull(t));
+          if (lane == 0) mbar_arrive(bar_ffull);
         }
         const float2 sc2 = splat2(sc), nm = splat2(-m);
 #pragma unroll
@@ -366,8 +371,8 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const float2 d = fma2(f2_from_bits(v[c][2 * e], v[c][2 * e + 1]), sc2, nm);
-            // (all exponentials on the MUFU unit: an eighth / a quarter / a half on the FMA pipe 37.8 / 38.5 / 41.7 us for 256 x 512
-            // x 512 against 38.1 without)
+            // (all exponentials on the MUFU unit: with an eighth / a quarter / a half of them on the FMA pipe, 256 x 512 x 512 took 37.8 /
+            // 38.5 / 41.7 us against 38.1 in the version that still ran it, before every block had its own maximum)
             const float2 ex = make_float2(ex2_approx(d.x), ex2_approx(d.y));
             if (e & 1) sum1 = add2(sum1, ex);
             else sum = add2(sum, ex);
@@ -385,7 +390,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       // the row sums for the finish warps, once they have read what the array held: the last block's factors, or the previous
       // item's sums (read before the output's last columns)
       fcount += static_cast<uint32_t>(nblk - 1);
-      if (nblk > 1) mbar_wait<false>(bar_fdone(t), (fcount - 1u) & 1u, w);
+      if (nblk > 1) mbar_wait<false>(bar_fdone, (fcount - 1u) & 1u, w);
       else if (oitem > 0) mbar_wait<false>(bar_oempty(t), (oitem - 1u) & 1u, w);
       s_sum[t * 128 + q * 32 + lane] = (sum.x + sum.y) + (sum1.x + sum1.y);
       ++oitem;
@@ -398,46 +403,44 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     const int q = warp & 3;
     const uint32_t lane_sel = static_cast<uint32_t>(q * 32) << 16;
     const uint32_t box0 = smem_base + AttnSmem::OFF_OUT + q * 2 * 4096;
-    uint32_t b_uses = 0, fphase = 0;  // phase of bar_ffull: bit t
+    uint32_t b_uses = 0, fphase = 0;
     ItemWalk it(p);
     for (int i = 0; i < my_items; ++i, it.next()) {
       const int bz = it.bz, m0 = it.m0();
-      // rescale the output so far to the reference of each further block, under that block's exponentials (S.V of the previous
+      // rescale tile A's output so far to the reference of each further block, under that block's exponentials (S.V of the previous
       // blocks is complete: the scores of this one were issued behind it, and the softmax warps have read them)
 #pragma unroll 1
-      for (int j = 1; j < nblk; ++j)
+      for (int j = 1; j < nblk; ++j) {
+        mbar_wait<false>(bar_ffull, fphase & 1u, w);
+        ++fphase;
+        __syncwarp();
+        tcgen05_fence_after_sync();
+        const float f = s_sum[q * 32 + lane];
+        if (__any_sync(0xFFFFFFFFu, f != 1.f)) {
 #pragma unroll 1
-        for (int t = 0; t < (it.has_b(p.M) ? 2 : 1); ++t) {
-          mbar_wait<false>(bar_ffull(t), (fphase >> t) & 1u, w);
-          fphase ^= 1u << t;
-          __syncwarp();
-          tcgen05_fence_after_sync();
-          const float f = s_sum[t * 128 + q * 32 + lane];
-          if (__any_sync(0xFFFFFFFFu, f != 1.f)) {
-#pragma unroll 1
-            for (int c = 0; c < 128; c += 64) {
-              uint32_t o[2][32];
-              const uint32_t addr = tmem_base + lane_sel + 256 + t * 128 + c;
-              tmem_ld_issue_32cols(addr, o[0]);
-              tmem_ld_issue_32cols(addr + 32, o[1]);
+          for (int c = 0; c < 128; c += 64) {
+            uint32_t o[2][32];
+            const uint32_t addr = tmem_base + lane_sel + 256 + c;
+            tmem_ld_issue_32cols(addr, o[0]);
+            tmem_ld_issue_32cols(addr + 32, o[1]);
 #pragma unroll
-              for (int k = 0; k < 2; ++k) {
-                tmem_ld_wait_32(o[k]);
+            for (int k = 0; k < 2; ++k) {
+              tmem_ld_wait_32(o[k]);
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                  const float2 v2 = mul2(f2_from_bits(o[k][e], o[k][e + 1]), splat2(f));
-                  o[k][e] = __float_as_uint(v2.x);
-                  o[k][e + 1] = __float_as_uint(v2.y);
-                }
-                tmem_st_32cols(addr + 32 * k, o[k]);
+              for (int e = 0; e < 32; e += 2) {
+                const float2 v2 = mul2(f2_from_bits(o[k][e], o[k][e + 1]), splat2(f));
+                o[k][e] = __float_as_uint(v2.x);
+                o[k][e + 1] = __float_as_uint(v2.y);
               }
+              tmem_st_32cols(addr + 32 * k, o[k]);
             }
-            tmem_st_wait();
           }
-          tcgen05_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_fdone(t));
+          tmem_st_wait();
         }
+        tcgen05_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_fdone);
+      }
 #pragma unroll 1
       for (int t = 0; t < (it.has_b(p.M) ? 2 : 1); ++t) {
         const uint32_t n = t ? b_uses++ : static_cast<uint32_t>(i);  // items of this tile before this one
@@ -500,6 +503,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
 cudaError_t launch_b2b_attention(const void* X, const void* W1, const void* W2, B2bParams p, cudaStream_t st) {
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
+  if (p.N1 > 128 && p.M > 128) return cudaErrorInvalidValue;  // two tiles share one block, or one tile walks several
   CUtensorMap tmX, tmW1, tmW2, tmO;
   const uint64_t M = p.M, K = p.K, N1 = p.N1, N2 = p.N2;
   if (p.batch < 1) p.batch = 1;

@@ -1,7 +1,8 @@
-"""Attention form for short sources and few queries, blocks of 128 source positions and tiles of 128 query rows: one to four blocks with a partial last one, one and two
-tiles per work item (the second one missing, partial or full), fewer and more work items than SMs, both key layouts; scores that
-grow from block to block, so that a row's running maximum is raised (and its output rescaled) after every block, and ones that
-never raise it."""
+"""Attention form for short sources and few queries, blocks of 128 source positions and tiles of 128 query rows: one block, full and
+partial, under one and two tiles per work item (the second one missing, partial or full); one tile over two to four blocks with
+a partial last one; fewer and more work items than SMs, both key layouts; scores that grow from block to block, so that a row's
+running maximum is raised (and its output rescaled) after every block, and ones that never raise it.  (3, 129, 136) lies
+just across the line to the CTA-pair form."""
 import numpy as np
 import pytest
 import torch
