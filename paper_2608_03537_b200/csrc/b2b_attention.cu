@@ -115,6 +115,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   float* s_sum = reinterpret_cast<float*>(smem + AttnSmem::OFF_SUM);
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(smem + AttnSmem::OFF_MISC);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + AttnSmem::OFF_MISC + 4);
+  volatile uint32_t* s_issued = reinterpret_cast<volatile uint32_t*>(smem + AttnSmem::OFF_MISC + 8);  // key / value blocks, query tiles: loads issued
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -183,7 +184,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       // ------------------------------------------------------------------------------------------ TMA producer
       if (elect_one()) {
         int slot = 0;
-        uint32_t phase = 0, quse[2] = {0, 0};
+        uint32_t phase = 0, quse[2] = {0, 0}, blocks = 0;
         bool ok = true;
         auto next_slot = [&](uint32_t& dst, uint32_t& full) {
           if (!ok || !mbar_wait<false>(bar_kvempty(slot), phase ^ 1u, w)) { ok = false; return false; }  // passes on a fresh barrier
@@ -191,6 +192,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
           full = bar_kvfull(slot);
           mbar_arrive_expect_tx(full, kBlockBytes);
           if (++slot == kKvSlots) { slot = 0; phase ^= 1u; }
+          ++blocks;
           return true;
         };
         ItemWalk it(p);
@@ -221,6 +223,8 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
             tma_load_3d(dst + kBoxBytes, &tmW2, full, 64, j * 128, bz);
           }
         }
+        s_issued[0] = blocks;
+        s_issued[1] = (quse[0] ? 2u - (quse[0] & 1u) : 0u) | (quse[1] ? 2u - (quse[1] & 1u) : 0u) << 8;  // (none, or a count of the same parity)
       }
     } else if (warp == 1) {
       // ------------------------------------------------------------------------------------------ UMMA issuer
@@ -306,7 +310,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
           b_now = b_next;
         }
         umma_commit(bar_drain);  // nothing may still be writing tensor memory when it is freed
-        mbar_wait<false>(bar_drain, 0, w);
+        mbar_drain(bar_drain, 0, w);
       }
     }
   } else if (warp < kFirstFinishWarp) {
@@ -495,6 +499,14 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0 && *s_abort) {  // a wait expired: loads that nobody waited for may still be landing
+    const uint32_t blocks = s_issued[0];
+    for (uint32_t u = blocks > kKvSlots ? blocks - kKvSlots : 0; u < blocks; ++u) mbar_drain(bar_kvfull(u % kKvSlots), (u / kKvSlots) & 1u, w);
+    for (int t = 0; t < 2; ++t) {
+      const uint32_t uses = (s_issued[1] >> (8 * t)) & 255u;
+      if (uses) mbar_drain(bar_qfull(t), (uses - 1u) & 1u, w);
+    }
   }
 }
 

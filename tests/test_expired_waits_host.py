@@ -12,6 +12,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 # per file: the barriers that must be drained -- the last commit in front of the deallocation, landing loads, peers' sends
 DRAINED = {
+    "b2b_attention.cu": ["bar_drain", "bar_kvfull(", "bar_qfull("],
     "few_rows.cu": ["bar_acc", "bar_full(", "bar_recv", "bar_stat", "bar_max"],
     "few_rows_mlp.cu": ["bar_d2", "bar_full(", "bar_w2", "bar_recv"],
 }
