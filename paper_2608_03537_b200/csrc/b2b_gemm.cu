@@ -265,7 +265,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         ring.skip(2);  // V(k) belongs to the other lane
       }
       umma_commit_pair(bar_drain);
-      mbar_wait<false>(bar_drain, 0, w);
+      mbar_drain(bar_drain, 0, w);
     }
   } else if (warp == kMl2Warp) {
     // ------------------------------------------------------------------------------------------ S.V UMMAs (even CTA)
@@ -314,7 +314,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (k < 30) B2B_TRACE_AT(301 + 2 * k);
       }
       umma_commit_pair(bar_drain2);
-      mbar_wait<false>(bar_drain2, 0, w);
+      mbar_drain(bar_drain2, 0, w);
     }
   } else if (warp < 2 + kB2bEpiWarps) {
     // ------------------------------------------------------------------------------------------ softmax warps
@@ -541,6 +541,7 @@ b2b_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
   }
+  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 #ifdef COMFUSE_TRACE
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 64) p.trace[63] = globaltimer_ns();  // kernel exit
 #endif

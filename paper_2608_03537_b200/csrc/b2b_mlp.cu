@@ -303,7 +303,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
         if (++j1 == NC) { j1 = 0; ++t1; }
       }
       umma_commit_pair(bar_drain);
-      mbar_wait<false>(bar_drain, 0, w);
+      mbar_drain(bar_drain, 0, w);
     }
   } else if (warp == kMl2Warp) {
     // ------------------------------------------------------------------------------------------ ML2 lane (even CTA)
@@ -348,7 +348,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
         if (++j2 == NC) { j2 = 0; ++t2; }
       }
       umma_commit_pair(bar_drain + 8u);
-      mbar_wait<false>(bar_drain + 8u, 0, w);
+      mbar_drain(bar_drain + 8u, 0, w);
     }
   } else {
     // the row vectors, widened to fp32 once, by the epilogue warps (idle until the first P chunk is complete)
@@ -603,6 +603,7 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
   }
+  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 #ifdef COMFUSE_TRACE
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 64) { p.trace[252] = globaltimer_ns(); p.trace[249] = clock64(); }  // kernel exit
 #endif

@@ -300,7 +300,7 @@ b2b_stream_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       }
       if (!LOCK && nunits > 0 && ok) ml2(nunits - 1);
       umma_commit_pair(bar_drain);  // nothing may still be writing either CTA's TMEM when it is freed
-      mbar_wait<false>(bar_drain, 0, w);
+      mbar_drain(bar_drain, 0, w);
     }
   } else {
     // ------------------------------------------------------------------------------------------ epilogue warps
@@ -429,6 +429,7 @@ b2b_stream_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
   }
+  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 }
 
 }  // namespace

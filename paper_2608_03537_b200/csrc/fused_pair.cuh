@@ -371,7 +371,7 @@ fused_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       }
       umma_commit_pair(bar_drain);  // nothing may still be writing either CTA's TMEM when it is freed
-      mbar_wait<false>(bar_drain, 0, w);
+      mbar_drain(bar_drain, 0, w);
     }
   } else if (warp == Cfg::kStoreWarp) {
     // ------------------------------------------------------------------------------------------ store warp
@@ -1448,6 +1448,7 @@ COMFUSE_PROGRAM_LOOP
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, Cfg::TMEM_COLS);
   }
+  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 #ifdef COMFUSE_TRACE
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 64) p.trace[63] = globaltimer_ns();  // kernel exit
 #endif

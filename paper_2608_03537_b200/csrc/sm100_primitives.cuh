@@ -175,6 +175,17 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, const 
   return true;
 }
 
+// The last thing that one thread of a kernel does whose copies in flight are not counted one by one, behind the cluster's last
+// barrier (by then everything has been issued, and the issuers have drained their UMMAs): where a wait has expired in this CTA,
+// stay for a millisecond.  Loads and peers' stores that are under way take microseconds; a CTA that nothing is missing in
+// has none left.
+__device__ __forceinline__ void linger_behind_expired_wait(const WaitCtx& w) {
+  if (!*w.abort_flag) return;
+  const uint64_t t0 = globaltimer_ns();
+  while (globaltimer_ns() - t0 < 1000000ull) {
+  }
+}
+
 // One thread of a CTA in which a wait has expired tells every CTA of its cluster (`told`: a shared word of each CTA, zeroed before any
 // peer can write) in front of the cluster barrier at the kernel's end.  Where no wait expired, all that was sent between the
 // CTAs has been waited for by its receiver and that barrier is enough.  Where `told` is set behind it, the sends -- which are

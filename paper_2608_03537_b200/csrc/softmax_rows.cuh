@@ -225,7 +225,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         umma_commit_pair_both(bar_tfull(slot));
       }
       umma_commit_pair(bar_drain);  // nothing may still be writing either CTA's TMEM when it is freed
-      mbar_wait<false>(bar_drain, 0, w);
+      mbar_drain(bar_drain, 0, w);
     }
   } else if (warp == Cfg::kStoreWarp) {
     // ------------------------------------------------------------------------------------------ store warp
@@ -611,6 +611,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 2 * CHUNK);
   }
+  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 }
 
 }  // namespace comfuse
