@@ -456,9 +456,10 @@ comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void*
   const long long bsr = desc->batch > 1 ? desc->batch_stride_r : 0;
   const long long bsy = desc->batch > 1 ? desc->batch_stride_y : 0;
   const bool b_nk = (desc->flags & COMFUSE_FLAG_B_ROW_MAJOR_NK) != 0;
-  // COMFUSE_SOFTMAX_CLUSTER forces the cluster kernel of the softmax kind, COMFUSE_SPLIT_BLOCK the tile kernel of the others
-  static const bool forced_cluster = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr;
-  if (desc->fused && (epi == EPI_SOFTMAX ? !forced_cluster : forced_split_block() < 0)) {
+  // A switch that asks something of the tile kernels keeps the call on them: COMFUSE_SOFTMAX_CLUSTER and COMFUSE_SOFTMAX_STAGES (the
+  // softmax kind), COMFUSE_SPLIT_BLOCK (the others).  (COMFUSE_REDUCE_MODE does not: both modes promise the same bits.)
+  static const bool softmax_forced = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr || std::getenv("COMFUSE_SOFTMAX_STAGES") != nullptr;
+  if (desc->fused && (epi == EPI_SOFTMAX ? !softmax_forced : forced_split_block() < 0)) {
     const int wide_block = need > 0 ? wide_row_block(epi, desc->N, desc->K, form_row_pairs(desc, form_rows)) : 0;
     const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, *dev);
     if (few.mt) return run_few_rows(few, epi, *desc, a, A, B, Y, static_cast<float2*>(workspace), *dev, st, form_rows);
