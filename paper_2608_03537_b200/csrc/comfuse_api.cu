@@ -57,6 +57,32 @@ bool mult8(long long v) { return (v & 7) == 0; }
 
 }  // namespace
 
+int ResidentClusters::of(const void* kernel, int threads, int smem_bytes, int size, const DeviceInfo& dev) {
+  std::atomic<int>& slot = known_[dev.device < kMaxDev ? dev.device : kMaxDev - 1][size];
+  const int known = slot.load(std::memory_order_relaxed);
+  if (known) return known - 1;
+  int n = 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(static_cast<unsigned>(size * dev.sm_count), 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+  cfg.dynamicSmemBytes = smem_bytes;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(size);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // leave no error behind: the call takes the tile kernel
+    return 0;
+  }
+  slot.store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 // COMFUSE_REDUCE_MODE=leader selects leader-follower aggregation of the row statistics, anything else all-to-all.

@@ -637,36 +637,12 @@ cudaError_t launch_instance(const FewRowsPlan& plan, const CUtensorMap& tmW, con
   return cudaLaunchKernelEx(&cfg, kern, tmW, tmX, p);
 }
 
-// How many clusters of `size` CTAs of this kernel the current device holds at once (0: it could not be asked).  Every
-// instantiation puts one CTA on an SM, so one of them answers for all.
+// Clusters of `size` CTAs of this kernel that are resident at once; every instantiation puts one CTA on an SM, so one of them
+// answers for all.
 int resident_clusters(int size, const DeviceInfo& dev) {
-  constexpr int kMaxDev = 64;
-  static std::atomic<int> cache[kMaxDev][17];  // 1 + the answer; 0 = not asked yet
-  std::atomic<int>& slot = cache[dev.device < kMaxDev ? dev.device : kMaxDev - 1][size];
-  const int known = slot.load(std::memory_order_relaxed);
-  if (known) return known - 1;
+  static ResidentClusters cache;
   using Cfg = FewRowsCfg<1, 64>;
-  const auto kern = few_rows_kernel<EPI_LN, 1, 64>;
-  int n = 0;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  cfg.gridDim = dim3(static_cast<unsigned>(size * dev.sm_count), 1, 1);
-  cfg.blockDim = dim3(Cfg::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(size);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-    cudaGetLastError();  // leave no error behind: the call takes the tile kernel
-    return 0;
-  }
-  slot.store(n + 1, std::memory_order_relaxed);
-  return n;
+  return cache.of(reinterpret_cast<const void*>(&few_rows_kernel<EPI_LN, 1, 64>), Cfg::kThreads, Cfg::SMEM_BYTES, size, dev);
 }
 
 }  // namespace

@@ -367,23 +367,10 @@ cudaError_t prepare() {  // the kernel's attributes, once per device
   return cudaSuccess;
 }
 
-// Clusters of `size` CTAs that are resident at once (one CTA per SM in every instantiation); 0 if the device cannot be asked.
+// Clusters of `size` CTAs that are resident at once (one CTA per SM in every instantiation)
 int resident_clusters(int size, const DeviceInfo& dev) {
-  constexpr int kMaxDev = 64;
-  static std::atomic<int> cache[kMaxDev][17];  // 1 + the answer
-  std::atomic<int>& slot = cache[dev.device < kMaxDev ? dev.device : kMaxDev - 1][size];
-  const int known = slot.load(std::memory_order_relaxed);
-  if (known) return known - 1;
-  int n = 0;
-  cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = launch_config<64>(size, static_cast<unsigned>(size * dev.sm_count), attr, nullptr);
-  cfg.numAttrs = 1;
-  if (prepare<64>() != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, few_rows_mlp_kernel<64>, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  slot.store(n + 1, std::memory_order_relaxed);
-  return n;
+  static ResidentClusters cache;
+  return cache.of(reinterpret_cast<const void*>(&few_rows_mlp_kernel<64>), FewMlpCfg<64>::kThreads, FewMlpCfg<64>::SMEM_BYTES, size, dev);
 }
 
 int rows_per_item(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : 64; }

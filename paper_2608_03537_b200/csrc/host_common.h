@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "comfuse.h"
 #include "fused_params.h"
 
@@ -22,6 +24,18 @@ struct DeviceInfo {
 const DeviceInfo* current_device_info();
 
 void count_launch();
+
+// How many clusters of `size` (1 .. 16) CTAs of one kernel the current device holds at once: asked once per device and size, 0 where it
+// could not be asked.
+class ResidentClusters {
+ public:
+  int of(const void* kernel, int threads, int smem_bytes, int size, const DeviceInfo& dev);
+
+ private:
+  static constexpr int kMaxDev = 64;
+  std::atomic<int> known_[kMaxDev][17] = {};  // 1 + the answer; 0 = not asked yet
+};
+
 // Kernels are launched with programmatic stream serialization (their set-up overlaps the previous kernel's tail; they
 // wait for that kernel before touching global memory) unless COMFUSE_PDL=0.
 bool programmatic_launch_enabled();

@@ -464,7 +464,9 @@ cudaError_t launch_wide_row_finish(int kind, const RowParams& p, const float2* p
   const long long rows = static_cast<long long>(p.batch) * p.M;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const bool block_per_row = form_rows <= 1184;  // 8 blocks on each of 148 SMs; else eight rows (warps) per block
+  const DeviceInfo* dev = current_device_info();
+  if (!dev) return cudaErrorInvalidDevice;
+  const bool block_per_row = form_rows <= 8ll * dev->sm_count;  // eight blocks on each SM; else eight rows (warps) per block
   cfg.gridDim = dim3(static_cast<unsigned>(block_per_row ? rows : (rows + 7) / 8), 1, 1);
   cfg.blockDim = dim3(256, 1, 1);
   cfg.stream = st;
