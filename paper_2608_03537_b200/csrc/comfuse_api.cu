@@ -102,6 +102,16 @@ bool programmatic_launch_enabled() {
   return on;
 }
 
+// COMFUSE_FEW_ROWS=0 keeps calls of few rows on the kernels that calls of many rows take (few_rows.cu and few_rows_mlp.cu off): for
+// comparisons, and for testing those kernels' edges at small sizes.
+static bool few_rows_enabled() {
+  static const bool on = [] {
+    const char* e = std::getenv("COMFUSE_FEW_ROWS");
+    return !(e && e[0] == '0');
+  }();
+  return on;
+}
+
 // COMFUSE_SPLIT_BLOCK=<width> forces the tile kernel, in the two-kernel form with that block width where N is a multiple of
 // it (0 = never)
 static int forced_split_block() {
@@ -485,7 +495,7 @@ comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void*
   // A switch that asks something of the tile kernels keeps the call on them: COMFUSE_SOFTMAX_CLUSTER and COMFUSE_SOFTMAX_STAGES (the
   // softmax kind), COMFUSE_SPLIT_BLOCK (the others).  (COMFUSE_REDUCE_MODE does not: both modes promise the same bits.)
   static const bool softmax_forced = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr || std::getenv("COMFUSE_SOFTMAX_STAGES") != nullptr;
-  if (desc->fused && (epi == EPI_SOFTMAX ? !softmax_forced : forced_split_block() < 0)) {
+  if (desc->fused && few_rows_enabled() && (epi == EPI_SOFTMAX ? !softmax_forced : forced_split_block() < 0)) {
     const int wide_block = need > 0 ? wide_row_block(epi, desc->N, desc->K, form_row_pairs(desc, form_rows)) : 0;
     const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, *dev);
     if (few.mt) return run_few_rows(few, epi, *desc, a, A, B, Y, static_cast<float2*>(workspace), *dev, st, form_rows);
@@ -718,7 +728,7 @@ comfuse_status_t comfuse::b2b_gemm_units(const comfuse_b2b_desc_t* desc, const v
     if (const char* tp = std::getenv("COMFUSE_TRACE_PTR")) bp.trace = reinterpret_cast<unsigned long long*>(std::strtoull(tp, nullptr, 0));
     if (const char* tf = std::getenv("COMFUSE_TRACE_FLAGS")) bp.trace_flags = std::atoi(tf);
 #endif
-    const bool few = !attention && !relu_mlp && few_rows_mlp_fits(form_units, N1, N2);
+    const bool few = !attention && !relu_mlp && few_rows_enabled() && few_rows_mlp_fits(form_units, N1, N2);
     cudaError_t e = few ? launch_few_rows_mlp(X, W1, W2, bp, st)
                     : relu_mlp ? launch_b2b_stream(X, W1, W2, bp, st)
                     : attention ? launch_b2b_fused(X, W1, W2, bp, st)

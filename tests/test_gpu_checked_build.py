@@ -4,7 +4,8 @@ In that build every kernel evaluates a predicate in front of its global stores -
 the indices of the row-statistic and partial-statistic writes -- and a predicate that fails records a bit in the device
 status word and skips the access (nothing traps).  The ordinary build compiles the predicates out.  Here a child process
 loads the checked library in place of the ordinary one (COMFUSE_LIB), runs one case of every kernel family against the fp64
-oracle, and requires the status word to stay clear; the predicate machinery itself is exercised by a self-test kernel whose
+oracle -- as the library chooses, and with the form for few rows off, in which the small cases run on the tile kernels -- and
+requires the status word to stay clear; the predicate machinery itself is exercised by a self-test kernel whose
 predicate is false by construction and whose access is therefore skipped.
 """
 import os
@@ -32,6 +33,11 @@ torch.cuda.set_device(0)
 assert cf.selftest_bounds_predicate() is True
 assert cf.last_device_status() == cf.ERR_BOUNDS       # recorded, and cleared by the read
 assert cf.last_device_status() == cf.OK
+import numpy as np
+MASKED = wl.scaled_masked_softmax(90, 129, 200, 64, seed=21, causal=False)
+mask = np.random.default_rng(21).standard_normal((129, 200)).astype(np.float32)
+mask[:, 150:] = -np.inf
+MASKED.tensors["mask"] = wl.f32_to_bf16_bits(mask)
 cases = [
     wl.post_norm(300, 768, 200, seed=11, affine=True),
     wl.complex_subgraph(150, 4096, 128, seed=12),
@@ -41,6 +47,9 @@ cases = [
     wl.target_attention(2, 300, 256, 128, seed=16),
     wl.dlrm_bottom_mlp(600, 320, 512, 128, seed=18),
     wl.post_norm(130, 8192, 64, seed=17, affine=True, relu=True),
+    wl.target_attention(3, 300, 96, 128, seed=19),
+    wl.target_attention(200, 40, 264, 128, seed=20),
+    MASKED,
     wl.config(1),
 ]
 for i, w in enumerate(cases):
@@ -52,7 +61,6 @@ for i, w in enumerate(cases):
                             softmax_tol=P.TOL_SOFTMAX_MAX if fused else P.TOL_SOFTMAX_UNFUSED,
                             norm_tol=P.TOL_NORM_MAX if fused else 4e-2)
 # an epilogue program on the interpreter and as a generated kernel (compiled with the predicates as well)
-import numpy as np
 from oracle import fusion_spec_oracle as spo
 prog = wl.spec_range_normalise()
 M, N, K = 300, 1024, 72
@@ -79,13 +87,14 @@ def test_ordinary_build_has_no_predicates(cuda_device):
     assert cf.last_device_status() == cf.OK
 
 
-def test_checked_build_runs_every_kernel_family_with_a_clear_status_word(cuda_device):
+@pytest.mark.parametrize("few_rows", ["1", "0"])
+def test_checked_build_runs_every_kernel_family_with_a_clear_status_word(few_rows, cuda_device):
     try:
         cf_build.build(checked=True)     # incremental: nothing happens when the library is up to date
     except Exception as e:               # no nvcc on this machine: a library that came with the tree will do
         if not os.path.exists(CHECKED_LIB):
             pytest.skip(f"checked library not built: {e}")
-    env = dict(os.environ, COMFUSE_LIB=CHECKED_LIB, PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    env = dict(os.environ, COMFUSE_LIB=CHECKED_LIB, COMFUSE_FEW_ROWS=few_rows, PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
     r = subprocess.run([sys.executable, "-c", CHILD], cwd=ROOT, env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
     assert "checked build ok" in r.stdout

@@ -43,7 +43,8 @@ def test_few_rows(M, N, K, nk, cuda_device):
         ymax = float(abs(ref["Y"]).max())
         bounds = {"norm_tol": P.TOL_NORM_MAX if ymax < 8.0 else 2.0 ** -7 * ymax}   # bf16 half-ulp of the largest magnitude, twice
         if not ln:
-            bounds["rowmax_tol"] = 3e-2   # the two-kernel form takes the maximum from values that went through fp16
+            if cf.workspace_size(desc) > 0:
+                bounds["rowmax_tol"] = 3e-2   # the two-kernel form takes the maximum from values that went through fp16
         P.check_outputs(w, got, ref, label=f"{w.name} nk={nk}", **bounds)
 
 

@@ -1,5 +1,6 @@
 """Cross-CTA aggregation modes of the row statistics (Sec. 3.1): leader-follower must give the same bits as all-to-all,
-because both merge the CTAs' partials in rank order.  The mode is read once per process, so each mode runs in a child."""
+because both merge the CTAs' partials in rank order.  The mode is read once per process, so each mode runs in a child, with the
+form for few rows off (it only exchanges all-to-all)."""
 import os
 import subprocess
 import sys
@@ -30,9 +31,10 @@ np.savez(sys.argv[1], **out)
 
 
 def _run(mode, path):
-    env = dict(os.environ, COMFUSE_REDUCE_MODE=mode, PYTHONPATH=ROOT)
+    env = dict(os.environ, COMFUSE_REDUCE_MODE=mode, COMFUSE_FEW_ROWS="0", COMFUSE_VERBOSE="1", PYTHONPATH=ROOT)
     r = subprocess.run([sys.executable, "-c", CHILD, path], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stderr.count("comfuse: kernel epi=") == 3, r.stderr[-2000:]   # three cluster kernels, one per case
     return np.load(path)
 
 

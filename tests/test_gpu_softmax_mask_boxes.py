@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("batch,M,N,K,softcap", [(1, 1, 64, 8, 0.0), (3, 31, 72, 64, 0.0), (90, 129, 200, 64, 0.0), (160, 33, 256, 64, 3.0), (80, 257, 264, 32, 0.0),
-                                                 (40, 130, 520, 128, 0.0), (40, 300, 776, 64, 2.0), (35, 70, 1032, 256, 0.0)])
+                                                 (40, 130, 520, 128, 0.0), (40, 300, 776, 64, 2.0), (35, 70, 1032, 256, 0.0), (160, 33, 64, 64, 0.0), (160, 31, 72, 64, 0.0)])
 def test_additive_mask_boxes(batch, M, N, K, softcap, cuda_device):
     w = wl.scaled_masked_softmax(batch, M, N, K, seed=M + N, causal=False, softcap=softcap)
     g = np.random.default_rng(N)

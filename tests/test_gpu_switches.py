@@ -31,4 +31,5 @@ def test_switches_reach_calls_of_few_rows(cuda_device):
     assert len(two) == 1 and "stages=2 lock=0" in two[0], two
     stages = _launched(COMFUSE_SOFTMAX_STAGES="3")
     assert len(stages) == 1 and "stages=3 lock=1" in stages[0], stages
+    assert len(_launched(COMFUSE_FEW_ROWS="0")) == 2
     assert len(_launched(COMFUSE_SOFTMAX_CLUSTER="1")) == 1 and len(_launched(COMFUSE_SPLIT_BLOCK="0")) == 1
