@@ -1,5 +1,6 @@
 """GELU + LayerNorm MLP of few rows (the hidden layer side by side in a cluster), at the edges of its cuts: one row, full and partial
-row groups, hidden widths that end inside, at and behind a CTA's 128 units, one to sixteen CTAs, row slices that end empty; without
+row groups, hidden widths that end inside, at and behind a CTA's 128 units, one to sixteen CTAs, row slices that end empty, both sides of the lines
+for narrow hidden layers; without
 biases and affine parameters.  Against the fp64 oracle with the bounds of the row-tiled form."""
 import pytest
 import torch
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("affine", [False, True])
-@pytest.mark.parametrize("M,N1", [(1, 8), (3, 1000), (16, 128), (17, 136), (32, 512), (33, 2048), (64, 1920), (65, 384), (300, 520), (900, 256)])
+@pytest.mark.parametrize("M,N1", [(1, 8), (3, 1000), (16, 128), (17, 136), (32, 512), (33, 2048), (64, 1920), (65, 384), (300, 520), (900, 256),
+                                  (2368, 8), (2369, 8), (4736, 40), (4737, 40)])
 def test_few_rows_mlp(M, N1, affine, cuda_device):
     w = wl.b2b_mlp(M=M, K=128, N1=N1, N2=128, seed=M + N1, affine=affine)
     P.check_outputs(w, P.run_gpu(w, P.dev_tensors(w), fused=True), P.run_oracle(w), label=w.name)
