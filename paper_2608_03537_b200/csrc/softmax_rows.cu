@@ -13,10 +13,14 @@ bool softmax_rows_supported(const FusedParams& p) { return p.K <= 256 && p.N >= 
 cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_t stream) {
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
-  const bool resident = p.mask && p.N <= 2 * Cfg::CHUNK;
-  auto kern = resident ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true, true> : softmax_rows_kernel<NSTAGES, YBOXES, false, true, true>)
-              : p.mask ? (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, true, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, true, false>)
-                       : (p.b_nk ? softmax_rows_kernel<NSTAGES, YBOXES, true, false, false> : softmax_rows_kernel<NSTAGES, YBOXES, false, false, false>);
+  const RowMask mask = !p.mask ? kNoMask : p.N <= 2 * Cfg::CHUNK ? kMaskResident : p.M <= 8 ? kMaskThreads : kMaskBoxes;
+  using Kernel = decltype(&softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>);
+  static constexpr Kernel kKernels[4][2] = {
+      {softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>, softmax_rows_kernel<NSTAGES, YBOXES, true, kNoMask>},
+      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskThreads>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskThreads>},
+      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskBoxes>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskBoxes>},
+      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskResident>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskResident>}};
+  const Kernel kern = kKernels[mask][p.b_nk ? 1 : 0];
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
   constexpr int kMaxDev = 64;
@@ -44,12 +48,11 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
   int ncl = max_clusters[di].load(std::memory_order_acquire);
   if (ncl == 0) {
     cudaError_t e = cudaSuccess;
-    for (auto k : {softmax_rows_kernel<NSTAGES, YBOXES, false, false, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, false, false>,
-                   softmax_rows_kernel<NSTAGES, YBOXES, false, true, false>, softmax_rows_kernel<NSTAGES, YBOXES, true, true, false>,
-                   softmax_rows_kernel<NSTAGES, YBOXES, false, true, true>, softmax_rows_kernel<NSTAGES, YBOXES, true, true, true>}) {
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
-      if (e != cudaSuccess) return e;
-    }
+    for (const auto& pair : kKernels)
+      for (const Kernel k : pair) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+      }
     int n = 0;
     cfg.gridDim = dim3(2 * dev->sm_count, 1, 1);
     e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);

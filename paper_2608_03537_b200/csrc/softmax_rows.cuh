@@ -59,21 +59,26 @@ struct RowSoftmaxCfg {
 
 // BKM: the B operand is stored [N, K] (one box of this CTA's 128 columns x 64 contraction elements per stage, K-major for the
 // UMMA, like A) instead of [K, N] (two boxes of 64 contraction rows x 64 columns, MN-major).
-// ADD: an additive mask tensor [M, N].  A thread owns a row of the chunk, so reading the mask straight from global memory
-// touches 32 rows per load instruction (32 sectors for 512 bytes, in both passes): 96 batches of 504 x 504 scores took 47.0 us
-// that way, 36.3 with the boxes below (33.5 with RES).  Every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
+// MASK: an additive mask tensor [M, N].
+// kMaskThreads: a thread owns a row of the chunk and reads its mask values straight from global memory, which touches a sector per row
+// and load instruction, in both passes: 96 batches of 504 x 504 scores took 47.0 us that way, 36.3 with the boxes below (33.5 with
+// kMaskResident).  For a handful of rows in each batch that is less than a box: 134 x 1 x 720 29.7 / 31.2, 198 x 2 x 520 36.0 / 38.7,
+// 42 x 7 x 1072 23.4 / 24.1; but 127 x 9 x 1408 56.5 / 55.2.
+// kMaskBoxes (ADD): every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
 // take the result: read the box, overwrite it with the probabilities, store it.  The warp's elected lane asks for the box
 // of the unit after next as soon as a box is free, and issues the store itself (no barrier round trip through other warps).
-// RES (with ADD): rows of at most 512 columns.  Both chunks of the row stay in their accumulator slots: pass 0 writes the finished
-// scores (capped, scaled, masked, log2 domain, fp32) back over the accumulators and pass 1 only exponentiates them -- one UMMA, one
-// mask box and one soft-cap per chunk instead of two.  Device time without / with: 96 x 504 x 504 35.7 / 33.5 us, 40 x 512 x 512
-// 23.5 / 21.6, 8 x 1379 x 424 14.4 / 13.0.  What is left is the exponentials of both passes and the 4 KB stores.
-template <int NSTAGES, int YBOXES, bool BKM, bool ADD, bool RES>
+// kMaskResident (ADD, RES): rows of at most 512 columns.  Both chunks of the row stay in their accumulator slots: pass 0 writes the
+// finished scores (capped, scaled, masked, log2 domain, fp32) back over the accumulators and pass 1 only exponentiates them -- one
+// UMMA, one mask box and one soft-cap per chunk instead of two.  Device time without / with: 96 x 504 x 504 35.7 / 33.5 us, 40 x 512
+// x 512 23.5 / 21.6, 8 x 1379 x 424 14.4 / 13.0.  What is left is the exponentials of both passes and the 4 KB stores.
+enum RowMask { kNoMask, kMaskThreads, kMaskBoxes, kMaskResident };
+template <int NSTAGES, int YBOXES, bool BKM, RowMask MASK>
 __global__ void __launch_bounds__(32 * 20, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
   constexpr int CHUNK = Cfg::CHUNK;
+  constexpr bool ADD = MASK == kMaskBoxes || MASK == kMaskResident, RES = MASK == kMaskResident;
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
@@ -242,6 +247,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       for (int r = 0; r < rounds && ok; ++r) {
         int b, mpair0, L;
         if (!tile_at(r, b, mpair0, L)) continue;
+        if (MASK == kMaskThreads && mpair0 + static_cast<int>(pm) * 128 + q * 32 >= p.M) continue;  // (that warp passes the tile over)
         for (int c = 0; c < L; ++c) {
         const int col = c * CHUNK + h * 64;
         if (col >= p.N) break;
@@ -307,7 +313,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const bool capped = p.softcap > 0.f;
     const SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
     const float sc = capped ? 1.f : p.alpha * 1.4426950408889634f;
-    constexpr bool additive = ADD;  // additive mask tensor, applied behind the scale / soft-cap
+    constexpr bool additive = MASK != kNoMask;  // additive mask tensor, applied behind the scale / soft-cap
     constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
 
 #ifdef COMFUSE_TRACE
@@ -396,9 +402,9 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     for (int r = 0; r < rounds; ++r) {
       int b, mpair0, L;
       if (!tile_at(r, b, mpair0, L)) continue;
-      if (ADD && mpair0 + static_cast<int>(pm) * 128 + q * 32 >= p.M) {
-        // none of this warp's rows exists (nor of the three it merges with): the accumulators are handed back as they come.  134 batches
-        // of 1 x 720 scores took 29.8 us with masks read by the threads whose rows exist, 34.4 with boxes for all of them
+      if (additive && mpair0 + static_cast<int>(pm) * 128 + q * 32 >= p.M) {
+        // none of this warp's rows exists (nor of the three it merges with): the accumulators are handed back as they come.
+        // With boxes for all warps 134 x 1 x 720 took 35.0 us instead of 31.2, 64 x 16 x 1176 27.9 instead of 24.9.
         for (int u = 0; u < (RES ? 1 : 2) * L; ++u, ++unit) {
           wait_slot(static_cast<int>(unit & 1u));
           release_slot(static_cast<int>(unit & 1u));
@@ -455,7 +461,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
               float2 tv[16];
               if (additive) {  // a full-tensor operand of the epilogue (Sec. 5.2)
                 float2 m2[16];
-                box_mask(mbox, half, m2);
+                if constexpr (ADD) box_mask(mbox, half, m2);
+                else load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) tv[j] = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
               } else {
@@ -531,7 +538,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                   }
                 } else if constexpr (additive) {
                   float2 m2[16];
-                  box_mask(mbox, half, m2);
+                  if constexpr (ADD) box_mask(mbox, half, m2);
+                  else load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
 #pragma unroll
                   for (int j = 0; j < 16; ++j) {  // (a masked score is -inf, and so is -inf - off: its probability is an exact zero)
                     const float2 t01 = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), add2(m2[j], splat2(-off)));
