@@ -497,7 +497,7 @@ comfuse_status_t gemm_epilogue_rows(const comfuse_gemm_desc_t* desc, const void*
   static const bool softmax_forced = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr || std::getenv("COMFUSE_SOFTMAX_STAGES") != nullptr;
   if (desc->fused && few_rows_enabled() && (epi == EPI_SOFTMAX ? !softmax_forced : forced_split_block() < 0)) {
     const int wide_block = need > 0 ? wide_row_block(epi, desc->N, desc->K, form_row_pairs(desc, form_rows)) : 0;
-    const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, *dev);
+    const FewRowsPlan few = few_rows_plan(epi, desc->batch, form_rows, desc->N, desc->K, wide_block, desc->lda, desc->ldb, b_nk, *dev);
     if (few.mt) return run_few_rows(few, epi, *desc, a, A, B, Y, static_cast<float2*>(workspace), *dev, st, form_rows);
   }
   GemmMaps maps;

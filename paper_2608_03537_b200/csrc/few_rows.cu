@@ -647,7 +647,7 @@ int resident_clusters(int size, const DeviceInfo& dev) {
 
 }  // namespace
 
-FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_block, const DeviceInfo& dev) {
+FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_block, long long ld_rows, long long ld_weights, bool b_nk, const DeviceInfo& dev) {
   FewRowsPlan none, c;
   if (epi != EPI_LN && epi != EPI_RMS_MAX && epi != EPI_SOFTMAX) return none;
   if (N > kWideRowBlock && (wide_block != 256 || epi == EPI_SOFTMAX)) return none;
@@ -665,15 +665,33 @@ FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_bloc
   // or the tile kernel is ahead (1024 x 1024 x 64 10.8 / 9.3, 2048 x 768 x 64 8.9 / 9.4, 2048 x 1024 x 1024 19.4 / 20.9).
   // Softmax kind, one round (row or cluster kernel / this one, K = 64): 8 x 64 x 512 11.0 / 4.4, 2 x 1024 x 1024 12.7 / 6.7,
   // 140 x 64 x 128 11.6 / 5.4; two rounds: 16 x 512 x 512 causal 10.6 / 12.8, 2 x 1171 x 1176 masked 11.4 / 12.5.
-  // Two tiles per CTA halve the CTAs where one does not fit: 3000 x 512 x 768 16.3 / 10.1, 2000 x 768 x 1536 18.7 / 14.1, level from
-  // K = 3072 on.  Not for normalised rows of up to 256 columns, which the tile kernel holds in one CTA pair (5923 x 256 x 256
+  // Two tiles per CTA halve the CTAs where one does not fit: 3000 x 512 x 768 16.3 / 10.1, 2000 x 768 x 1536 18.7 / 14.1, 2306 x 512 x
+  // 4096 28.7 / 23.4 (where such calls end: l2_bound).  Not for normalised rows of up to 256 columns, which the tile kernel holds in one CTA pair (5923 x 256 x 256
   // 7.9 / 7.8, x 1536 14.1 / 15.7).
+  // Every row group reads the weights anew, twice as often as the tile kernel's 256-row pairs, and with most of the machine at it the
+  // L2 is what bounds the call (8.5 - 9.5 TB/s).  A box row of 128 bytes that does not start on a 128-byte line touches two of them.
+  // Measured (tile kernel / this one, us; LayerNorm):
+  //   two tiles per CTA, weight rows off their lines, the tile kernel's two-kernel form available: 3520 x 512 x 1032 level, x 2056
+  //   21.9 / 24.0, x 3592 31.1 / 41.7, 2368 x 512 x 2056 21.4 / 22.0; rows of 513 .. 768 columns, which the tile kernel is best at, on
+  //   more than three quarters of the SMs: 2880 x 768 x 520 level, x 1032 17.1 / 17.7, x 4088 40.3 / 41.4, 2880 x 520 x 1032 16.5 /
+  //   17.7, but 2112 x 768 x 1032 16.8 / 15.1, x 4088 39.4 / 37.0;
+  //   weight rows on their lines: 3520 x 512 x 4096 27.9 / 27.5, x 5128 32.7 / 34.7; with the activations' rows on theirs too 2306 x
+  //   512 x 6144 38.1 / 33.2, 2800 x 512 x 8192 47.9 / 52.2; one kernel: 1500 x 768 x 8192 64.2 / 42.9.
+  //   one tile, weights [K, 24] on more than half of the SMs: 7104 rows, K = 3080 27.5 / 28.6, 8184 56.5 / 69.1.
+  auto l2_bound = [&](const FewRowsPlan& q, long long n) {
+    const long long ctas = n * q.ct;
+    if (q.nt == 1) return !q.wide && N < 64 && !b_nk && K > 2560 && ctas > dev.sm_count / 2;
+    const bool weights_on_lines = ld_weights % 64 == 0, rows_on_lines = ld_rows % 64 == 0;
+    if (!weights_on_lines && N > 512 && N <= 768 && K > 768 && ctas > 3 * dev.sm_count / 4) return true;
+    return wide_block == 256 && K > (!weights_on_lines ? 1536 : rows_on_lines ? 6144 : 4096);
+  };
   for (c.nt = 1; c.nt <= (N <= 256 && epi != EPI_SOFTMAX ? 1 : 2); ++c.nt) {
     c.ct = c.wide ? 2 : (N + 128 * c.nt - 1) / (128 * c.nt);
     if (c.ct > 16 || clusters > resident_clusters(c.ct, dev)) {
       if (c.wide) return none;
       continue;
     }
+    if (epi != EPI_SOFTMAX && l2_bound(c, clusters)) return none;
     // Splitting the contraction pays from 12 K blocks on (one exchange costs about as much as four blocks): 128 x 512 x 1024
     // 6.3 / 5.8 / 6.2 us with 1 / 2 / 4 shares, x 2048 8.4 / 6.9 / 6.9, x 256 4.7 / 4.8 / 5.7.  A third of the SMs is left
     // to the next call's set-up (2048 x 256 x 1024: 6.5 us with 64 CTAs, 7.2 with 128).

@@ -42,7 +42,8 @@ struct FewRowsParams {
 };
 
 // `wide_block`: column block width of the two-kernel form the call would take otherwise (0: the row stays on chip).
-FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_block, const DeviceInfo& dev);
+// `ld_rows`, `ld_weights`: leading dimensions of the activations and of the weights; `b_nk`: weights stored [N, K].
+FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_block, long long ld_rows, long long ld_weights, bool b_nk, const DeviceInfo& dev);
 // tmW: the weights in boxes of 64 x 64 elements (either storage order); tmX: the rows in boxes of 64 elements x mt rows.
 cudaError_t launch_few_rows(int epi, const FewRowsPlan& plan, const CUtensorMap& tmW, const CUtensorMap& tmX, FewRowsParams p,
                             cudaStream_t stream);

@@ -1,7 +1,7 @@
 """Fused kinds behind a GEMM of few rows (weights as the tensor core's 128-row operand, contraction split over a
 cluster), at the edges of its cuts: one row, full and partial row groups of 16 / 32 / 64, full and partial 128-column tiles,
 one and two tiles per CTA, 1 to 8 shares of the contraction, row slices that end empty, the two-kernel form with a partial last
-block, both storage orders of the weights.  Against the fp64 oracle with the bounds of the other fused forms."""
+block, both sides of the lines that follow what the L2 delivers, both storage orders of the weights.  Against the fp64 oracle with the bounds of the other fused forms."""
 import pytest
 import torch
 
@@ -12,7 +12,8 @@ from tests import parity as P
 pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 8, 8), (16, 128, 64), (17, 136, 768), (32, 256, 72), (33, 2056, 200), (63, 1000, 2056), (64, 1024, 1792), (65, 4096, 64),
-          (2, 264, 4104), (40, 4096, 4096), (5, 2048, 1024), (70, 2824, 1032), (300, 768, 768), (900, 520, 320)]
+          (2, 264, 4104), (40, 4096, 4096), (5, 2048, 1024), (70, 2824, 1032), (300, 768, 768), (900, 520, 320), (2112, 520, 1032), (2369, 520, 1032), (1100, 512, 1544),
+          (7110, 24, 2568)]
 
 
 @pytest.mark.parametrize("nk", [False, True])
