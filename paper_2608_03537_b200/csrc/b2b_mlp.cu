@@ -602,8 +602,8 @@ b2b_mlp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
+    if (lane == 0) linger_behind_expired_wait(w);
   }
-  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 #ifdef COMFUSE_TRACE
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 64) { p.trace[252] = globaltimer_ns(); p.trace[249] = clock64(); }  // kernel exit
 #endif

@@ -428,8 +428,8 @@ b2b_stream_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
+    if (lane == 0) linger_behind_expired_wait(w);
   }
-  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 }
 
 }  // namespace

@@ -1447,8 +1447,8 @@ COMFUSE_PROGRAM_LOOP
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, Cfg::TMEM_COLS);
+    if (lane == 0) linger_behind_expired_wait(w);
   }
-  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 #ifdef COMFUSE_TRACE
   if (p.trace && blockIdx.x == 0 && threadIdx.x == 64) p.trace[63] = globaltimer_ns();  // kernel exit
 #endif

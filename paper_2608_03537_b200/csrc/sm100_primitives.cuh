@@ -178,7 +178,8 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, const 
 // The last thing that one thread of a kernel does whose copies in flight are not counted one by one, behind the cluster's last
 // barrier (by then everything has been issued, and the issuers have drained their UMMAs): where a wait has expired in this CTA,
 // stay for a millisecond.  Loads and peers' stores that are under way take microseconds; a CTA that nothing is missing in
-// has none left.
+// has none left.  (In the warp that frees tensor memory, which is the last to leave anyway: 32 x 4096 queries of 256 keys 25.7 us with
+// it there, 26.0 in a warp of its own.)
 __device__ __forceinline__ void linger_behind_expired_wait(const WaitCtx& w) {
   if (!*w.abort_flag) return;
   const uint64_t t0 = globaltimer_ns();

@@ -629,8 +629,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncwarp();
     tcgen05_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 2 * CHUNK);
+    if (lane == 0) linger_behind_expired_wait(w);
   }
-  if (threadIdx.x == 0) linger_behind_expired_wait(w);
 }
 
 }  // namespace comfuse
