@@ -677,10 +677,11 @@ FewRowsPlan few_rows_plan(int epi, int batch, int M, int N, int K, int wide_bloc
   //   17.7, but 2112 x 768 x 1032 16.8 / 15.1, x 4088 39.4 / 37.0;
   //   weight rows on their lines: 3520 x 512 x 4096 27.9 / 27.5, x 5128 32.7 / 34.7; with the activations' rows on theirs too 2306 x
   //   512 x 6144 38.1 / 33.2, 2800 x 512 x 8192 47.9 / 52.2; one kernel: 1500 x 768 x 8192 64.2 / 42.9.
-  //   one tile, weights [K, 24] on more than half of the SMs: 7104 rows, K = 3080 27.5 / 28.6, 8184 56.5 / 69.1.
+  //   one tile, narrow weights [K, N] on more than half of the SMs: 7104 x 24 x 3080 27.5 / 28.6, x 8184 56.5 / 69.1; 5200 x 8 x 1024 14.9 /
+  //   17.0, x 2048 19.4 / 20.0.
   auto l2_bound = [&](const FewRowsPlan& q, long long n) {
     const long long ctas = n * q.ct;
-    if (q.nt == 1) return !q.wide && N < 64 && !b_nk && K > 2560 && ctas > dev.sm_count / 2;
+    if (q.nt == 1) return !q.wide && N < 64 && !b_nk && K > (N < 16 ? 768 : 2560) && ctas > dev.sm_count / 2;
     const bool weights_on_lines = ld_weights % 64 == 0, rows_on_lines = ld_rows % 64 == 0;
     if (!weights_on_lines && N > 512 && N <= 768 && K > 768 && ctas > 3 * dev.sm_count / 4) return true;
     return wide_block == 256 && K > (!weights_on_lines ? 1536 : rows_on_lines ? 6144 : 4096);
