@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 8, 8), (16, 128, 64), (17, 136, 768), (32, 256, 72), (33, 2056, 200), (63, 1000, 2056), (64, 1024, 1792), (65, 4096, 64),
           (2, 264, 4104), (40, 4096, 4096), (5, 2048, 1024), (70, 2824, 1032), (300, 768, 768), (900, 520, 320), (2112, 520, 1032), (2369, 520, 1032), (1100, 512, 1544),
-          (7110, 24, 2568)]
+          (7110, 24, 2568), (4740, 8, 776)]
 
 
 @pytest.mark.parametrize("nk", [False, True])
