@@ -13,7 +13,7 @@ bool softmax_rows_supported(const FusedParams& p) { return p.K <= 256 && p.N >= 
 cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_t stream) {
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
-  const RowMask mask = !p.mask ? kNoMask : p.N <= 2 * Cfg::CHUNK ? kMaskResident : p.M <= 8 ? kMaskThreads : kMaskBoxes;
+  const RowMask mask = !p.mask ? kNoMask : p.N <= 2 * Cfg::CHUNK ? kMaskResident : p.M <= 32 ? kMaskThreads : kMaskBoxes;
   using Kernel = decltype(&softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>);
   static constexpr Kernel kKernels[4][2] = {
       {softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>, softmax_rows_kernel<NSTAGES, YBOXES, true, kNoMask>},

@@ -62,8 +62,8 @@ struct RowSoftmaxCfg {
 // MASK: an additive mask tensor [M, N].
 // kMaskThreads: a thread owns a row of the chunk and reads its mask values straight from global memory, which touches a sector per row
 // and load instruction, in both passes: 96 batches of 504 x 504 scores took 47.0 us that way, 36.3 with the boxes below (33.5 with
-// kMaskResident).  For a handful of rows in each batch that is less than a box: 134 x 1 x 720 29.7 / 31.2, 198 x 2 x 520 36.0 / 38.7,
-// 42 x 7 x 1072 23.4 / 24.1; but 127 x 9 x 1408 56.5 / 55.2.
+// kMaskResident).  Where a batch has no more rows than one warp, that is less than a box (threads / boxes): 150 x 9 x 600 34.5 / 39.1,
+// 150 x 20 x 2048 97.3 / 103.4, 40 x 32 x 6576 107.3 / 110.4; but 40 x 43 x 2048 38.1 / 37.3, 150 x 64 x 2048 113.4 / 103.5.
 // kMaskBoxes (ADD): every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
 // take the result: read the box, overwrite it with the probabilities, store it.  The warp's elected lane asks for the box
 // of the unit after next as soon as a box is free, and issues the store itself (no barrier round trip through other warps).
