@@ -478,7 +478,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
 #pragma unroll
         for (int d = LPR / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) sq_l += o[k].x == -INFINITY ? 0.f : o[k].y * ex2_approx(o[k].x - m);
+        for (int k = 0; k < CPL; ++k) sq_l += o[k].y * (o[k].x == -INFINITY ? 0.f : ex2_approx(o[k].x - m));  // (a NaN stays one)
         const float own = r < rv ? s_stat[r * 16 + ct].x : -INFINITY;  // this CTA's exponentials are relative to its own maximum
         mu_l = own == -INFINITY ? 0.f : ex2_approx(own - m);
       } else {
@@ -492,8 +492,8 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         p.wide_partials[(static_cast<long long>(b) * p.M + grow) * p.nblocks + nb] = make_float2(EPI == EPI_LN ? mu_l : sq_l, EPI == EPI_LN ? sq_l : 0.f);
     }
     // factor of the row: 1 / standard deviation, or what turns this CTA's exponentials into probabilities (a row without a live
-    // column is all zero)
-    const float rstd_l = EPI == EPI_SOFTMAX ? (sq_l > 0.f ? mu_l / sq_l : 0.f) : rsqrtf(sq_l * inv_n_all + eps);
+    // column is all zero, a row with a NaN all NaN)
+    const float rstd_l = EPI == EPI_SOFTMAX ? (sq_l == 0.f ? 0.f : mu_l / sq_l) : rsqrtf(sq_l * inv_n_all + eps);
     const float shift_l = -mu_l * rstd_l;
     float rstd[RC], shift[RC], best[RC], best_col[RC];
 #pragma unroll

@@ -68,3 +68,22 @@ def test_few_rows_softmax(batch, M, N, K, softcap, mask, cuda_device):
     P.check_outputs(w, got, P.run_oracle(w), label=f"{w.name} {mask}", softmax_tol=P.TOL_SOFTMAX_MAX)
     if mask == "additive":
         assert (got["Y"][:, M // 2, :] == 0).all()
+
+
+@pytest.mark.parametrize("batch,M,N,K", [(3, 64, 1000, 320), (2, 5, 72, 776), (1, 40, 2056, 64), (4, 17, 512, 64)])
+def test_softmax_rows_with_a_nan_are_nan(batch, M, N, K, cuda_device):
+    bf = torch.bfloat16
+    g = torch.Generator(device=cuda_device).manual_seed(N)
+    A, B = (torch.empty(s, device=cuda_device).normal_(generator=g).to(bf) for s in ((batch, M, K), (batch, K, N)))
+    A[:, 1, 3] = float("nan")                            # every score of row 1
+    mask = torch.zeros(M, N, dtype=bf, device=cuda_device)
+    mask[2, N - 1] = float("nan")                        # one score of row 2
+    mask[3, : N - 8] = float("-inf")
+    mask[3, N - 3] = float("nan")                        # ... of row 3, whose other column ranges have no live column
+    mask[4, 0] = float("inf")
+    for m in (None, mask):
+        Y = torch.zeros(batch, M, N, dtype=bf, device=cuda_device)
+        cf.gemm_epilogue(A, B, Y, cf.EPI_SCALE_MASK_SOFTMAX, alpha=K ** -0.5, mask=cf.MASK_NONE if m is None else cf.MASK_ADDITIVE, mask_tensor=m)
+        want = torch.zeros(M, dtype=torch.bool, device=cuda_device)
+        want[1 : 2 if m is None else 5] = True
+        assert torch.equal(Y.isnan(), want[None, :, None].expand_as(Y))
