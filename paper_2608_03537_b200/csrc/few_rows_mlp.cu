@@ -380,14 +380,14 @@ int rows_per_item(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : 64; }
 // Taken where all its clusters are resident at once.  Measured there (device time, row-tiled form / this one, us): 8 rows x 440 hidden
 // units 8.2 / 3.8, 4 x 952 11.1 / 3.9, 43 x 976 11.1 / 6.2, 679 x 512 8.6 / 5.9, 1227 x 248 7.0 / 5.8, 2473 x 160 7.0 / 5.7.
 // Hidden layers of fewer than 64 units: every CTA asks for the same few sectors of W1 and W2, and many CTAs at once wait for one another
-// there.  8 units: 2000 rows 6.2 / 5.8, 2500 6.3 / 6.1, 3000 6.2 / 6.4, 8000 7.0 / 10.1; 32 units: 4000 6.2 / 5.7, 5000 6.3 / 6.2,
-// 6000 6.3 / 6.8; 64 units: 9000 6.3 / 5.6.
+// there.  8 units: 2000 rows 6.2 / 5.8, 2500 6.3 / 6.1, 3000 6.2 / 6.4, 8000 7.0 / 10.1; 24 units: 3000 6.2 / 5.8, 4000 6.3 / 6.4,
+// 5000 6.5 / 7.6; 40 units: 4000 6.3 / 6.1, 5000 6.6 / 7.3; 64 units: 9000 6.3 / 5.6.
 bool few_rows_mlp_fits(int M, int N1, int N2) {
   const DeviceInfo* dev = current_device_info();
   const int cluster = (N1 + 127) / 128;
   if (!dev || dev->cc_major != 10 || N2 != 128 || cluster > 16) return false;
   const int groups = (M + rows_per_item(M) - 1) / rows_per_item(M);
-  if (N1 < 64 && groups > dev->sm_count / (N1 < 32 ? 4 : 2)) return false;
+  if (N1 < 64 && groups > dev->sm_count / (N1 < 16 ? 4 : N1 < 32 ? 3 : 2)) return false;
   return groups <= resident_clusters(cluster, *dev);
 }
 

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("affine", [False, True])
 @pytest.mark.parametrize("M,N1", [(1, 8), (3, 1000), (16, 128), (17, 136), (32, 512), (33, 2048), (64, 1920), (65, 384), (300, 520), (900, 256),
-                                  (2368, 8), (2369, 8), (4736, 40), (4737, 40)])
+                                  (2368, 8), (2369, 8), (3136, 24), (3137, 24), (4736, 40), (4737, 40)])
 def test_few_rows_mlp(M, N1, affine, cuda_device):
     w = wl.b2b_mlp(M=M, K=128, N1=N1, N2=128, seed=M + N1, affine=affine)
     P.check_outputs(w, P.run_gpu(w, P.dev_tensors(w), fused=True), P.run_oracle(w), label=w.name)
