@@ -74,20 +74,6 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
       : "memory");
 }
 
-template <int N>
-__device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-template <int N>
-__device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
-
-// registers -> 16 consecutive fp32 columns of this thread's lane
-__device__ __forceinline__ void tmem_st_16cols(uint32_t taddr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-
 // KM: the keys (W1) are stored [batch, N1, K], one key per row (a K-major operand), else [batch, K, N1] (MN-major).
 template <bool KM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -382,7 +368,7 @@ b2b_attention_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
             else sum = add2(sum, ex);
             pk[e] = pack_bf16x2_rn(ex);
           }
-          tmem_st_16cols(t_score + c * 16, pk);
+          tmem_st_16(t_score + c * 16, pk);
           if (c & 1) {
             tmem_st_wait();
             tcgen05_fence_before_sync();

@@ -13,13 +13,12 @@ bool softmax_rows_supported(const FusedParams& p) { return p.K <= 256 && p.N >= 
 cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_t stream) {
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
-  const RowMask mask = !p.mask ? kNoMask : p.N <= 2 * Cfg::CHUNK ? kMaskResident : p.M <= 32 ? kMaskThreads : kMaskBoxes;
+  const RowMask mask = !p.mask ? kNoMask : p.M <= 32 ? kMaskThreads : kMaskBoxes;
   using Kernel = decltype(&softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>);
-  static constexpr Kernel kKernels[4][2] = {
+  static constexpr Kernel kKernels[3][2] = {
       {softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>, softmax_rows_kernel<NSTAGES, YBOXES, true, kNoMask>},
       {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskThreads>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskThreads>},
-      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskBoxes>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskBoxes>},
-      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskResident>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskResident>}};
+      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskBoxes>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskBoxes>}};
   const Kernel kern = kKernels[mask][p.b_nk ? 1 : 0];
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
@@ -52,6 +51,10 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
       for (const Kernel k : pair) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
         if (e != cudaSuccess) return e;
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+        if (fa.numRegs < Cfg::kRegsLaunch) return cudaErrorLaunchOutOfResources;  // the warps' shares would wait for ever
       }
     int n = 0;
     cfg.gridDim = dim3(2 * dev->sm_count, 1, 1);

@@ -7,19 +7,30 @@
 // the other side of the same trade: one CTA pair owns 256 complete rows, streams the row through tensor memory in
 // 256-column chunks TWICE (MainLoop re-run instead of on-chip residency), and needs no cross-CTA exchange at all:
 //
-//   pass 0   for every live chunk:  S = A.B_chunk (UMMA, cta_group::2)  ->  online (max, sum) per thread
+//   pass 0   for every live chunk:  S = A.B_chunk (UMMA, cta_group::2)  ->  online (max, sum) per thread; the exponentials of the
+//            last chunk stay in registers, those of the chunk before it in the chunk's accumulator slot (fp32 both)
 //   merge    the four threads that share a row combine their partials through shared memory
-//   pass 1   for every live chunk:  S again  ->  P = 2^(S*alpha*log2e - (max + log2 sum))  ->  bf16 box -> TMA store
+//   result   the two kept chunks: exponential * 2^(m_thread - (max + log2 sum))  ->  bf16 box -> TMA store
+//   pass 1   for every other live chunk:  S again  ->  P = 2^(S*alpha*log2e - (max + log2 sum))  ->  bf16 box -> TMA store
 //
 // Clusters are pairs, so all SMs are used (wider clusters leave SMs idle), any N fits, and the accumulator slots
-// alternate so that the UMMAs of chunk u+1 run under the epilogue of chunk u.  Under a causal mask, chunks above the
-// diagonal are neither computed nor staged: the epilogue warps write their zeros with plain stores, a few rows after
-// every chunk pass, from a cursor that runs through the cluster's tiles on its own.
+// alternate so that the UMMAs of chunk u+1 run under the epilogue of chunk u.  Rows of up to 512 columns are computed and
+// exponentiated once.  Under a causal mask, chunks above the diagonal are neither computed nor staged: a warp of its own
+// writes them with TMA stores of a constant zero box, with a cursor of its own through the cluster's tiles.
 //
-// Warp roles as in the general kernel: warp 0 TMA producer, warp 1 TMEM allocation + UMMA issue (even CTA),
-// 16 epilogue warps (thread = row; warp e takes lane quarter e % 4 and 64-column group e / 4 of each chunk), last warp
-// issues the TMA stores of the staged boxes.  Every wait is bounded.
+// What bounds it: the exponentials (MUFU: 16 results per clock and SM; a pass over 64 x 32 scores of all sixteen warps takes
+// 1640 clocks in a loop of its own) and, where the output outgrows the L2, the writes.  64 x 2048 x 2048 causal, K = 64 (537 MB
+// written, 85 us at the best rate of any store pattern measured here): 122.5 -> 116.2 us, without its stores 99 -> 76.  A thread
+// holds all its 64 columns of a chunk, so the accumulator is handed back before the arithmetic, which needs the registers that
+// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 33.4 -> 29.1 us; thirty shapes drawn from
+// 16 .. 2048 rows and 64 .. 2048 columns 0.995 .. 1.46 times as fast (geometric mean 1.13).
+//
+// Warp roles: warp 0 TMA producer, warp 1 TMEM allocation + UMMA issue (even CTA), warp 2 zero boxes, warp 3 idle (register
+// shares are given to groups of four warps); then 16 epilogue warps (thread = row; warp e takes lane quarter e % 4 and
+// 64-column group e / 4 of each chunk), which stage their boxes and issue the stores themselves.  Every wait is bounded.
 #pragma once
+
+#include <type_traits>
 
 #include "epilogue_common.cuh"
 #include "fused_params.h"
@@ -30,15 +41,21 @@ namespace comfuse {
 template <int NSTAGES, int YBOXES>
 struct RowSoftmaxCfg {
   static constexpr int kEpiWarps = 16;
-  static constexpr int kStoreWarp = 2 + kEpiWarps;
-  static constexpr int kZeroWarp = kStoreWarp + 1;
-  static constexpr int kThreads = 32 * (kZeroWarp + 1);
-  static constexpr int ZERO_TMA_LANES = 4;                   // zero boxes in flight per SM
+  static constexpr int kZeroWarp = 2;                        // (a fourth warp fills up the control warps' group)
+  static constexpr int kFirstEpiWarp = 4;
+  static constexpr int kThreads = 32 * (kFirstEpiWarp + kEpiWarps);
+  // registers a thread: the launch gives every thread 96; the control warps' group hands on what the epilogue warps take
+  static constexpr int kRegsLaunch = 96, kRegsControl = 32, kRegsEpi = 112;
+  static_assert(4 * kRegsControl + 16 * kRegsEpi <= 20 * kRegsLaunch, "the warps' shares have to fit what the launch holds");
+  // zero boxes in flight per SM (2, 4 and 8 level in the kernel; in a kernel that writes nothing else 4 KB boxes reach 6.3 TB/s with 4 in
+  // flight and 5.7 with 16 or more)
+  static constexpr int ZERO_TMA_LANES = 4;
   static constexpr int CHUNK = 256;                          // columns per UMMA and per accumulator slot
   // Which of a 32-column fragment's 16 column pairs take 2^x from the FMA-pipe polynomial instead of the MUFU unit
   // (bit j = pair j).  The MUFU unit delivers 16 results per clock per SM and is this kernel's busiest pipe; the
   // polynomial costs about six issue slots per value.  Measured on the attention-score workload: none 126.2 us,
-  // 2 of 16 pairs 123.7, 3: 123.1, 4: 122.7, 5: 123.9, 6: 124.8, 8: 128.8.
+  // 4 of 16 pairs 122.7, 8: 128.8, when both passes exponentiated every score.  Now, with the writes in the way, 116.6 / 116.3 / 117.6
+  // for none / 4 / 6; without them 81.9 / 76.2 / 81.8 for none / 4 / 8.
   static constexpr uint32_t POLY_PAIRS = 0x1248u;            // pairs 3, 6, 9, 12
   static constexpr int A_BYTES = 128 * 64 * 2;
   static constexpr int STAGE_BYTES = A_BYTES + (CHUNK / 2) * 64 * 2;  // A block + this CTA's half of the B chunk
@@ -49,7 +66,7 @@ struct RowSoftmaxCfg {
   static constexpr int OFF_PRE = OFF_ZERO + WARP_BOX_BYTES;  // per-row partials of the 4 column groups, two tile parities
   static constexpr int PRE_BYTES = 2 * 4 * 128 * 8;
   static constexpr int OFF_BAR = OFF_PRE + PRE_BYTES;
-  static constexpr int NUM_BARS = 2 * NSTAGES + 4 + 1 + 2 * kEpiWarps * YBOXES;
+  static constexpr int NUM_BARS = 2 * NSTAGES + 4 + 1 + kEpiWarps * YBOXES;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
   static constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
@@ -61,24 +78,20 @@ struct RowSoftmaxCfg {
 // UMMA, like A) instead of [K, N] (two boxes of 64 contraction rows x 64 columns, MN-major).
 // MASK: an additive mask tensor [M, N].
 // kMaskThreads: a thread owns a row of the chunk and reads its mask values straight from global memory, which touches a sector per row
-// and load instruction, in both passes: 96 batches of 504 x 504 scores took 47.0 us that way, 36.3 with the boxes below (33.5 with
-// kMaskResident).  Where a batch has no more rows than one warp, that is less than a box (threads / boxes): 150 x 9 x 600 34.5 / 39.1,
-// 150 x 20 x 2048 97.3 / 103.4, 40 x 32 x 6576 107.3 / 110.4; but 40 x 43 x 2048 38.1 / 37.3, 150 x 64 x 2048 113.4 / 103.5.
-// kMaskBoxes (ADD): every epilogue warp's 32 x 64 mask box arrives by TMA in the warp's own staging boxes, which in pass 1 also
-// take the result: read the box, overwrite it with the probabilities, store it.  The warp's elected lane asks for the box
-// of the unit after next as soon as a box is free, and issues the store itself (no barrier round trip through other warps).
-// kMaskResident (ADD, RES): rows of at most 512 columns.  Both chunks of the row stay in their accumulator slots: pass 0 writes the
-// finished scores (capped, scaled, masked, log2 domain, fp32) back over the accumulators and pass 1 only exponentiates them -- one
-// UMMA, one mask box and one soft-cap per chunk instead of two.  Device time without / with: 96 x 504 x 504 35.7 / 33.5 us, 40 x 512
-// x 512 23.5 / 21.6, 8 x 1379 x 424 14.4 / 13.0.  What is left is the exponentials of both passes and the 4 KB stores.
-enum RowMask { kNoMask, kMaskThreads, kMaskBoxes, kMaskResident };
+// and load instruction: 96 batches of 504 x 504 scores took 47.0 us that way when 36.3 with the boxes below.
+// Where a batch has no more rows than one warp, that is less than a box (threads / boxes, measured with both passes over every chunk):
+// 150 x 9 x 600 34.5 / 39.1, 150 x 20 x 2048 97.3 / 103.4, 40 x 32 x 6576 107.3 / 110.4; but 40 x 43 x 2048 38.1 / 37.3, 150 x 64 x
+// 2048 113.4 / 103.5.
+// kMaskBoxes (ADD): every epilogue warp's 32 x 64 mask box arrives by TMA in one of the warp's staging boxes, which also
+// take the result: read the box, overwrite it with the probabilities, store it.
+enum RowMask { kNoMask, kMaskThreads, kMaskBoxes };
 template <int NSTAGES, int YBOXES, bool BKM, RowMask MASK>
 __global__ void __launch_bounds__(32 * 20, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
   constexpr int CHUNK = Cfg::CHUNK;
-  constexpr bool ADD = MASK == kMaskBoxes || MASK == kMaskResident, RES = MASK == kMaskResident;
+  constexpr bool ADD = MASK == kMaskBoxes;
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
@@ -92,8 +105,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   auto bar_tfull = [&](int a) { return bar_base + 8u * (2 * NSTAGES + a); };    // accumulator slot complete
   auto bar_tempty = [&](int a) { return bar_base + 8u * (2 * NSTAGES + 2 + a); };  // slot drained by both CTAs (even CTA)
   const uint32_t bar_drain = bar_base + 8u * (2 * NSTAGES + 4);
-  auto bar_yfull = [&](int e, int k) { return bar_drain + 8u + 8u * (e * YBOXES + k); };
-  auto bar_yfree = [&](int e, int k) { return bar_drain + 8u + 8u * (Cfg::kEpiWarps * YBOXES + e * YBOXES + k); };
+  auto bar_mask = [&](int e, int k) { return bar_drain + 8u + 8u * (e * YBOXES + k); };
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(smem + Cfg::OFF_MISC);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + Cfg::OFF_MISC + 4);
 
@@ -121,8 +133,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     mbar_init(bar_drain, 1);
     for (int e = 0; e < Cfg::kEpiWarps; ++e)
       for (int k = 0; k < YBOXES; ++k) {
-        mbar_init(bar_yfull(e, k), 1);
-        mbar_init(bar_yfree(e, k), 1);
+        mbar_init(bar_mask(e, k), 1);
       }
     *s_abort = 0;
     fence_mbar_init();
@@ -156,469 +167,510 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     return true;
   };
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------------------------------ TMA producer
-    if (elect_one()) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      // every operand chunk is read twice per tile and the K matrix by every tile of its batch, while 16 times as many
-      // output bytes stream through the L2: ask it to keep the operands
-      const uint64_t keep = l2_policy_evict_last();
-      for (int r = 0; r < rounds && ok; ++r) {
-        int b, mpair0, L;
-        if (!tile_at(r, b, mpair0, L)) continue;
-        const int m0 = mpair0 + static_cast<int>(pm) * 128;
-        for (int u = 0; u < (RES ? 1 : 2) * L && ok; ++u) {
-        const int c = u < L ? u : u - L;  // pass 0 over the live chunks, then pass 1
-        for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) { ok = false; break; }  // passes on a fresh barrier
-          const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
-          const uint32_t full = map_to_cta(bar_full(stage), 0);
-          mbar_arrive_expect_tx_cluster(full, Cfg::STAGE_BYTES);
-          tma_load_3d_pair_hint(sa, &tmA, full, kb * 64, m0, b, keep);
-          // this CTA's half of the UMMA's B tile: two boxes of 64 columns, 8 KB apart
-          const int col = c * CHUNK + static_cast<int>(pm) * (CHUNK / 2);
-          if constexpr (BKM) {  // two boxes of 64 rows of B (columns of the product) x 64 contraction elements
-            tma_load_3d_pair_hint(sa + Cfg::A_BYTES, &tmB, full, kb * 64, col, b, keep);
-            tma_load_3d_pair_hint(sa + Cfg::A_BYTES + 8192, &tmB, full, kb * 64, col + 64, b, keep);
-          } else {
-            tma_load_3d_pair_hint(sa + Cfg::A_BYTES, &tmB, full, col, kb * 64, b, keep);
-            tma_load_3d_pair_hint(sa + Cfg::A_BYTES + 8192, &tmB, full, col + 64, kb * 64, b, keep);
+  // Units (accumulators) of a tile: pass 0 takes every chunk; the exponentials of the last two stay on the chip (see the
+  // epilogue), so pass 1 takes the others.  Slots alternate, except that the unit behind pass 0 takes the slot of the last
+  // chunk, which is handed back as soon as it has been loaded; the one before it stays in its slot until it has been written.
+  auto tile_units = [](int L) { return L < 2 ? L : 2 * L - 2; };
+  auto next_slot = [](int slot, int u, int L) { return u == L - 1 && L >= 2 ? slot : slot ^ 1; };
+
+  if (warp < Cfg::kFirstEpiWarp) {
+    setmaxnreg_dec<Cfg::kRegsControl>();
+    if (warp == 0) {
+      // ------------------------------------------------------------------------------------------ TMA producer
+      if (elect_one()) {
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        // every operand chunk is read twice per tile and the K matrix by every tile of its batch, while 16 times as many
+        // output bytes stream through the L2: ask it to keep the operands
+        const uint64_t keep = l2_policy_evict_last();
+        for (int r = 0; r < rounds && ok; ++r) {
+          int b, mpair0, L;
+          if (!tile_at(r, b, mpair0, L)) continue;
+          const int m0 = mpair0 + static_cast<int>(pm) * 128;
+          for (int u = 0; u < tile_units(L) && ok; ++u) {
+            const int c = u < L ? u : u - L;  // pass 0 over the live chunks, then pass 1 over those whose exponentials were not kept
+            for (int kb = 0; kb < KB; ++kb) {
+              if (!mbar_wait<false>(bar_empty(stage), phase ^ 1u, w)) { ok = false; break; }  // passes on a fresh barrier
+              const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
+              const uint32_t full = map_to_cta(bar_full(stage), 0);
+              mbar_arrive_expect_tx_cluster(full, Cfg::STAGE_BYTES);
+              tma_load_3d_pair_hint(sa, &tmA, full, kb * 64, m0, b, keep);
+              // this CTA's half of the UMMA's B tile: two boxes of 64 columns, 8 KB apart
+              const int col = c * CHUNK + static_cast<int>(pm) * (CHUNK / 2);
+              if constexpr (BKM) {  // two boxes of 64 rows of B (columns of the product) x 64 contraction elements
+                tma_load_3d_pair_hint(sa + Cfg::A_BYTES, &tmB, full, kb * 64, col, b, keep);
+                tma_load_3d_pair_hint(sa + Cfg::A_BYTES + 8192, &tmB, full, kb * 64, col + 64, b, keep);
+              } else {
+                tma_load_3d_pair_hint(sa + Cfg::A_BYTES, &tmB, full, col, kb * 64, b, keep);
+                tma_load_3d_pair_hint(sa + Cfg::A_BYTES + 8192, &tmB, full, col + 64, kb * 64, b, keep);
+              }
+              if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
+            }
           }
-          if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
-        }
         }
       }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------------------------------ UMMA issuer (even CTA)
-    if (pm == 0 && elect_one()) {
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t slot_uses[2] = {0, 0};
-      uint32_t unit = 0;
-      constexpr uint32_t idesc = make_idesc_bf16(256, CHUNK, false, !BKM);
-      bool ok = true;
-      uint32_t total_units = 0;
-      for (int r = 0; r < rounds; ++r) {
-        int b, mpair0, L;
-        if (tile_at(r, b, mpair0, L)) total_units += (RES ? 1u : 2u) * L;
-      }
-      while (ok && unit < total_units) {
-        const int slot = static_cast<int>(unit & 1u);
-        ++unit;
-        if (!mbar_wait<false>(bar_tempty(slot), (slot_uses[slot] & 1u) ^ 1u, w)) break;
-        ++slot_uses[slot];
-        tcgen05_fence_after_sync();
-        const uint32_t d_tmem = tmem_base + slot * CHUNK;
-        for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait<false>(bar_full(stage), phase, w)) { ok = false; break; }
-          tcgen05_fence_after_sync();
-          const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
-          const uint64_t adesc = make_smem_desc_sw128(sa, 16, 1024);
-          const uint64_t bdesc = BKM ? make_smem_desc_sw128(sa + Cfg::A_BYTES, 16, 1024)
-                                     : make_smem_desc_sw128(sa + Cfg::A_BYTES, /*next 64-column block*/ 8192, /*next 8 K rows*/ 1024);
+    } else if (warp == 1) {
+      // ------------------------------------------------------------------------------------------ UMMA issuer (even CTA)
+      if (pm == 0 && elect_one()) {
+        int stage = 0;
+        uint32_t phase = 0;
+        uint32_t slot_uses[2] = {0, 0};
+        int slot = 0;
+        constexpr uint32_t idesc = make_idesc_bf16(256, CHUNK, false, !BKM);
+        bool ok = true;
+        for (int r = 0; r < rounds && ok; ++r) {
+          int b, mpair0, L;
+          if (!tile_at(r, b, mpair0, L)) continue;
+          for (int u = 0; u < tile_units(L) && ok; ++u, slot = next_slot(slot, u - 1, L)) {
+            if (!mbar_wait<false>(bar_tempty(slot), (slot_uses[slot] & 1u) ^ 1u, w)) { ok = false; break; }
+            ++slot_uses[slot];
+            tcgen05_fence_after_sync();
+            const uint32_t d_tmem = tmem_base + slot * CHUNK;
+            for (int kb = 0; kb < KB; ++kb) {
+              if (!mbar_wait<false>(bar_full(stage), phase, w)) { ok = false; break; }
+              tcgen05_fence_after_sync();
+              const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
+              const uint64_t adesc = make_smem_desc_sw128(sa, 16, 1024);
+              const uint64_t bdesc = BKM ? make_smem_desc_sw128(sa + Cfg::A_BYTES, 16, 1024)
+                                         : make_smem_desc_sw128(sa + Cfg::A_BYTES, /*next 64-column block*/ 8192, /*next 8 K rows*/ 1024);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)  // K advances by 16 elements: 32 bytes inside a K-major operand's swizzled row, 2048 bytes in an MN-major B
-            umma_bf16_ss_pair(d_tmem, adesc + static_cast<uint64_t>(k * 2), bdesc + static_cast<uint64_t>(BKM ? k * 2 : k * 128), idesc,
-                              (kb | k) != 0 ? 1u : 0u);
-          umma_commit_pair_both(bar_empty(stage));
-          if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
-        }
-        if (!ok) break;
-        umma_commit_pair_both(bar_tfull(slot));
-      }
-      umma_commit_pair(bar_drain);  // nothing may still be writing either CTA's TMEM when it is freed
-      mbar_drain(bar_drain, 0, w);
-    }
-  } else if (warp == Cfg::kStoreWarp) {
-    // ------------------------------------------------------------------------------------------ store warp
-    // Lane e mirrors epilogue warp e: per live chunk, wait until the box is staged, store it, hand the staging box back.
-    if (!ADD && lane < Cfg::kEpiWarps) {  // (with a mask the epilogue warps store their boxes themselves)
-      const int e = lane;
-      const int q = (e + 2) & 3;
-      const int h = e >> 2;
-      constexpr int D = YBOXES - 1;
-      const uint32_t ybox0 = smem_base + Cfg::OFF_YBUF + e * YBOXES * Cfg::WARP_BOX_BYTES;
-      const uint64_t stream_out = l2_policy_evict_first();  // the output is never read again
-      uint32_t n = 0;
-      bool ok = true;
-      for (int r = 0; r < rounds && ok; ++r) {
-        int b, mpair0, L;
-        if (!tile_at(r, b, mpair0, L)) continue;
-        if (MASK == kMaskThreads && mpair0 + static_cast<int>(pm) * 128 + q * 32 >= p.M) continue;  // (that warp passes the tile over)
-        for (int c = 0; c < L; ++c) {
-        const int col = c * CHUNK + h * 64;
-        if (col >= p.N) break;
-        const uint32_t sel = n % YBOXES;
-        if (!mbar_wait<false>(bar_yfull(e, sel), (n / YBOXES) & 1u, w)) { ok = false; break; }
-#ifdef COMFUSE_TRACE
-        if (!(p.trace_flags & 1))
-#endif
-        if (COMFUSE_IN_BOUNDS(col >= 0 && col < p.N && (col & 7) == 0 && mpair0 >= 0 && b >= 0 && b < p.batch, p.status))
-        tma_store_3d_hint(&tmY, ybox0 + sel * Cfg::WARP_BOX_BYTES, col, mpair0 + static_cast<int>(pm) * 128 + q * 32, b, stream_out);
-        tma_store_commit();
-        if (n >= static_cast<uint32_t>(D)) {
-          tma_store_wait_read<D>();
-          mbar_arrive(bar_yfree(e, (n - D) % YBOXES));
-        }
-        ++n;
-        }
-      }
-      tma_store_wait_read<0>();  // shared memory must outlive the last stores' reads (the stores complete at kernel end)
-    }
-  } else if (warp == Cfg::kZeroWarp) {
-    // ------------------------------------------------------------------------------------------ zero-box warp
-    // The chunks above the causal diagonal hold zeros and depend on nothing.  A few lanes, each with one TMA store of a
-    // constant zero box in flight, walk them with a cursor of their own, independent of the epilogue (asynchronous
-    // stores: plain stores would share the SM's memory-instruction queue with the epilogue's exponentials and
-    // shared-memory traffic).  Few boxes in flight, so that a staged box never queues far behind zeros.
-    if (!ADD && lane < Cfg::ZERO_TMA_LANES && p.causal) {
-      const uint64_t stream_out = l2_policy_evict_first();
-      uint32_t k = 0;
-      for (int r = 0; r < rounds; ++r) {
-        int b, mpair0, L;
-        if (!tile_at(r, b, mpair0, L)) continue;
-        const int y0 = mpair0 + static_cast<int>(pm) * 128;
-        for (int c = L; c < nch; ++c)
-          for (int i = 0; i < 16; ++i, ++k) {
-            if (k % Cfg::ZERO_TMA_LANES != static_cast<uint32_t>(lane)) continue;
-            const int col = c * CHUNK + (i >> 2) * 64;
-            if (col >= p.N) continue;
-            tma_store_wait_all();
-#ifdef COMFUSE_TRACE
-            if (!(p.trace_flags & 4))
-#endif
-            if (COMFUSE_IN_BOUNDS(col >= 0 && (col & 7) == 0 && y0 >= 0 && b >= 0 && b < p.batch, p.status))
-            tma_store_3d_hint(&tmY, smem_base + Cfg::OFF_ZERO, col, y0 + (i & 3) * 32, b, stream_out);
-            tma_store_commit();
+              for (int k = 0; k < 4; ++k)  // K advances by 16 elements: 32 bytes inside a K-major operand's swizzled row, 2048 bytes in an MN-major B
+                umma_bf16_ss_pair(d_tmem, adesc + static_cast<uint64_t>(k * 2), bdesc + static_cast<uint64_t>(BKM ? k * 2 : k * 128), idesc,
+                                  (kb | k) != 0 ? 1u : 0u);
+              umma_commit_pair_both(bar_empty(stage));
+              if (++stage == NSTAGES) { stage = 0; phase ^= 1u; }
+            }
+            if (!ok) break;
+            umma_commit_pair_both(bar_tfull(slot));
           }
+        }
+        umma_commit_pair(bar_drain);  // nothing may still be writing either CTA's TMEM when it is freed
+        mbar_drain(bar_drain, 0, w);
       }
-      tma_store_wait_read<0>();
+    } else if (warp == Cfg::kZeroWarp) {
+      // ------------------------------------------------------------------------------------------ zero-box warp
+      // The chunks above the causal diagonal hold zeros and depend on nothing.  A few lanes, each with one TMA store of a
+      // constant zero box in flight, walk them with a cursor of their own, independent of the epilogue (asynchronous
+      // stores: plain stores would share the SM's memory-instruction queue with the epilogue's exponentials and
+      // shared-memory traffic).  Few boxes in flight, so that a staged box never queues far behind zeros.
+      if (lane < Cfg::ZERO_TMA_LANES && p.causal) {
+        const uint64_t stream_out = l2_policy_evict_first();
+        uint32_t k = 0;
+        for (int r = 0; r < rounds; ++r) {
+          int b, mpair0, L;
+          if (!tile_at(r, b, mpair0, L)) continue;
+          const int y0 = mpair0 + static_cast<int>(pm) * 128;
+          for (int c = L; c < nch; ++c)
+            for (int i = 0; i < 16; ++i, ++k) {
+              if (k % Cfg::ZERO_TMA_LANES != static_cast<uint32_t>(lane)) continue;
+              const int col = c * CHUNK + (i >> 2) * 64;
+              if (col >= p.N) continue;
+              tma_store_wait_all();
+#ifdef COMFUSE_TRACE
+              if (!(p.trace_flags & 4))
+#endif
+              if (COMFUSE_IN_BOUNDS(col >= 0 && (col & 7) == 0 && y0 >= 0 && b >= 0 && b < p.batch, p.status))
+              tma_store_3d_hint(&tmY, smem_base + Cfg::OFF_ZERO, col, y0 + (i & 3) * 32, b, stream_out);
+              tma_store_commit();
+            }
+        }
+        tma_store_wait_read<0>();
+      }
     }
   } else {
+    setmaxnreg_inc<Cfg::kRegsEpi>();
     // ------------------------------------------------------------------------------------------ epilogue warps
-    const int e = warp - 2;
+    const int e = warp - Cfg::kFirstEpiWarp;
     const int q = warp & 3;  // TMEM lane quarter this warp may touch: rows 32q .. 32q+31 of the CTA's row block
     const int h = e >> 2;    // the 64-column group of every chunk this warp takes
     const int row = q * 32 + lane;
     const uint32_t lane_sel = static_cast<uint32_t>(q * 32) << 16;
     const uint32_t tempty_leader = map_to_cta(bar_tempty(0), 0);
     const uint32_t ybox0 = smem_base + Cfg::OFF_YBUF + e * YBOXES * Cfg::WARP_BOX_BYTES;
-    uint32_t slot_uses[2] = {0, 0};
-    uint32_t unit = 0, nbox = 0, tile_par = 0;
     // log2 domain: t = Acc * (alpha * log2 e), so exp(x - m) = 2^(t - m_t)
-    // with a soft-cap the accumulators are mapped to capped log2-domain scores right after they are loaded, and sc = 1
+    // with a soft-cap the accumulators are mapped to capped log2-domain scores right after they are loaded, and the scale is 1
     const bool capped = p.softcap > 0.f;
     const SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
     const float sc = capped ? 1.f : p.alpha * 1.4426950408889634f;
     constexpr bool additive = MASK != kNoMask;  // additive mask tensor, applied behind the scale / soft-cap
+    // plain: the scale is positive and nothing else happens to a score, so it can be folded into the exponential's argument
+    const bool plain = !additive && !capped && sc > 0.f;
+    const float scale = plain ? sc : 1.f;
     constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
 
-#ifdef COMFUSE_TRACE
-    int trace_ix = 0;
-#define ROWS_TRACE_POINT()                                                                             \
-  do {                                                                                                 \
-    if (p.trace && blockIdx.x == 0 && warp == 2 && lane == 0 && trace_ix < 60) p.trace[trace_ix++] = globaltimer_ns(); \
-  } while (0)
-#else
-#define ROWS_TRACE_POINT() do { } while (0)
-#endif
-    auto wait_slot = [&](int slot) {
-      ROWS_TRACE_POINT();
-      mbar_wait<false>(bar_tfull(slot), slot_uses[slot] & 1u, w);
-      ++slot_uses[slot];
+    int slot = 0;
+    uint32_t slot_uses[2] = {0, 0};
+    uint32_t tile_par = 0;
+    auto wait_slot = [&](int sl) {
+      mbar_wait<false>(bar_tfull(sl), slot_uses[sl] & 1u, w);
+      ++slot_uses[sl];
       __syncwarp();
       tcgen05_fence_after_sync();
-      ROWS_TRACE_POINT();
     };
-    auto release_slot = [&](int slot) {
+    auto release_slot = [&](int sl) {
       tcgen05_fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster_noflush(tempty_leader + 8u * slot);
+      if (lane == 0) mbar_arrive_cluster_noflush(tempty_leader + 8u * sl);
     };
 
-    // ADD: unit n of this warp (passes 0 and 1 of every tile, the chunks in which its columns exist) uses box n % YBOXES; its mask
-    // is requested when unit n - YBOXES has finished with the box.
-    const int my_chunks = ADD ? (p.N - h * 64 + CHUNK - 1) / CHUNK : 0;  // (causal off: every chunk is live)
-    int load_r = -1, load_c = 0, load_row = 0;
-    bool load_pass1 = true;
-    uint32_t load_n = 0, mask_n = 0;
-    bool store_pending = false;
-    const uint64_t keep_mask = ADD ? l2_policy_evict_last() : 0, stream_box = ADD ? l2_policy_evict_first() : 0;
-    // the elected lane; steps through the units in the order in which they run (load_r = rounds: no further unit)
-    load_c = my_chunks;
-    auto request_mask = [&]() {
-      if (load_c >= my_chunks) {
-        load_c = 0;
-        load_pass1 = !RES && !load_pass1;
-        if (!load_pass1 && load_r < rounds) {
+    // Staging boxes: use n of this warp takes box n % YBOXES.  A use holds the chunk's mask (ADD), its result, or first one and
+    // then the other.  The elected lane issues the stores itself; it hands a box on when its store has read it, and asks for the
+    // mask of the box's next use then.
+    const bool elected = elect_one();
+    uint32_t use = 0;
+    const uint64_t stream_out = l2_policy_evict_first();  // the output is never read again
+    const uint64_t keep_mask = ADD ? l2_policy_evict_last() : 0;
+    // ADD: the uses of a tile (causal off: L = nch) are nch - 1 masks, mask and result of the last chunk (if it has columns for
+    // this warp), the result of the one before, masks and results of the others
+    const bool has_last = (nch - 1) * CHUNK + h * 64 < p.N;
+    const int tile_uses = tile_units(nch) + (nch >= 2 ? 1 : 0) - (has_last ? 0 : 1);
+    int req_r = -1, req_i = tile_uses, req_row = 0;
+    uint32_t req_use = 0, mask_phases = 0;
+    auto request_use = [&]() {  // (the elected lane) the mask of the next use not asked for yet, if it has one
+      if (req_i >= tile_uses) {
+        req_i = 0;
+        if (req_r < rounds) {
           do {  // (tiles in which this warp's rows do not exist are passed over)
             int lb, lm = 0, lL;
-            if (++load_r < rounds && !tile_at(load_r, lb, lm, lL)) load_r = rounds;
-            load_row = lm + static_cast<int>(pm) * 128 + q * 32;
-          } while (load_r < rounds && load_row >= p.M);
+            if (++req_r < rounds && !tile_at(req_r, lb, lm, lL)) req_r = rounds;
+            req_row = lm + static_cast<int>(pm) * 128 + q * 32;
+          } while (req_r < rounds && req_row >= p.M);
         }
       }
-      if (my_chunks <= 0 || load_r >= rounds) return;
-      const uint32_t sel = RES ? (my_chunks == 2 ? static_cast<uint32_t>(load_c) : 0u) : load_n % YBOXES;
-      mbar_arrive_expect_tx(bar_yfull(e, sel), Cfg::WARP_BOX_BYTES);
-      tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_yfull(e, sel), load_c * CHUNK + h * 64, load_row, 0, keep_mask);
-      ++load_n;
-      ++load_c;
+      if (tile_uses <= 0 || req_r >= rounds) return;
+      const int first_out = nch - (has_last ? 0 : 1);  // the use without a mask
+      const int c = req_i < first_out ? req_i : req_i - first_out - 1;
+      if (c >= 0) {
+        const uint32_t sel = req_use % YBOXES;
+        mbar_arrive_expect_tx(bar_mask(e, sel), Cfg::WARP_BOX_BYTES);
+        tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_mask(e, sel), c * CHUNK + h * 64, req_row, 0, keep_mask);
+      }
+      ++req_use;
+      ++req_i;
     };
-    bool elected = false;
     if constexpr (ADD) {
-      elected = elect_one();
       if (elected)
-        for (int i = 0; i < (RES && my_chunks < YBOXES ? my_chunks : YBOXES); ++i) request_mask();
+        for (int i = 0; i < YBOXES; ++i) request_use();
       __syncwarp();
     }
-    // the previous unit's box, once its store has read it, takes the mask of the unit after this one
+    bool store_pending = false;
+    // in front of a use: the previous use's box, once its store has read it, takes the mask of the use after this one
     auto reclaim_box = [&]() {
-      if (!store_pending) return;
+      if constexpr (ADD) {
+        if (!store_pending) return;
+        if (elected) {
+          tma_store_wait_read<0>();
+          request_use();
+        }
+        __syncwarp();
+        store_pending = false;
+      }
+    };
+    auto wait_mask = [&]() {
+      const uint32_t sel = use % YBOXES;
+      mbar_wait<false>(bar_mask(e, sel), (mask_phases >> sel) & 1u, w);
+      mask_phases ^= 1u << sel;
+      __syncwarp();
+    };
+    auto end_mask_use = [&]() {  // the use held a mask only and every lane has read its row
+      __syncwarp();
+      if (elected) request_use();
+      __syncwarp();
+      ++use;
+    };
+    // 64 result columns of this thread's row -> the box of this use -> global memory
+    auto emit = [&](const uint32_t (&pk)[32], int colg, int row0, int b) {
+      const uint32_t ybox = ybox0 + (use % YBOXES) * Cfg::WARP_BOX_BYTES;
+      ++use;
+      if constexpr (!ADD) {
+        if (elected) tma_store_wait_read<YBOXES - 1>();
+        __syncwarp();
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t a = ybox + static_cast<uint32_t>(lane * 128 + ((i ^ (lane & 7)) << 4));  // 128-byte swizzle
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(pk[4 * i]), "r"(pk[4 * i + 1]),
+                     "r"(pk[4 * i + 2]), "r"(pk[4 * i + 3])
+                     : "memory");
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
       if (elected) {
-        tma_store_wait_read<0>();
-        if (!RES || my_chunks == 2) request_mask();
+        if (COMFUSE_IN_BOUNDS(colg >= 0 && colg < p.N && (colg & 7) == 0 && row0 >= 0 && b >= 0 && b < p.batch, p.status))
+        tma_store_3d_hint(&tmY, ybox, colg, row0, b, stream_out);
+        tma_store_commit();
       }
       __syncwarp();
-      store_pending = false;
+      store_pending = true;
     };
-    // 32 mask values of half `half` of this thread's row of the box, as log2-domain addends
-    auto box_mask = [&](uint32_t box, int half, float2 (&m2)[16]) {
+    // scores of 32 columns in the log2 domain, in place (not in the plain case): soft-cap or scale, mask
+    auto transform = [&](uint32_t (&v)[32], int half, int grow, int col0) {
+      if (capped) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint32_t w4[4];
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(w4[0]), "=r"(w4[1]), "=r"(w4[2]), "=r"(w4[3])
-                     : "r"(box + static_cast<uint32_t>(lane * 128 + (((half * 4 + i) ^ (lane & 7)) << 4)))
-                     : "memory");
+        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
+      }
+      if constexpr (ADD) {
+        const uint32_t box = ybox0 + (use % YBOXES) * Cfg::WARP_BOX_BYTES;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) m2[4 * i + k] = mul2(bf16x2_to_f2(w4[k]), splat2(1.4426950408889634f));
+        for (int i = 0; i < 4; ++i) {
+          uint32_t w4[4];
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(w4[0]), "=r"(w4[1]), "=r"(w4[2]), "=r"(w4[3])
+                       : "r"(box + static_cast<uint32_t>(lane * 128 + (((half * 4 + i) ^ (lane & 7)) << 4)))
+                       : "memory");
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float2 m2 = mul2(bf16x2_to_f2(w4[k]), splat2(1.4426950408889634f));
+            const float2 t = fma2(f2_from_bits(v[8 * i + 2 * k], v[8 * i + 2 * k + 1]), splat2(sc), m2);
+            v[8 * i + 2 * k] = __float_as_uint(t.x);
+            v[8 * i + 2 * k + 1] = __float_as_uint(t.y);
+          }
+        }
+      } else if constexpr (additive) {
+        float2 m2[16];
+        load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float2 t = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
+          v[2 * j] = __float_as_uint(t.x);
+          v[2 * j + 1] = __float_as_uint(t.y);
+        }
+      } else if (!capped) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
+      }
+    };
+    auto scores = [&](uint32_t (&va)[32], uint32_t (&vb)[32], int c, int grow) {
+      if constexpr (ADD) {
+        reclaim_box();
+        wait_mask();
+      }
+      if (!plain) {
+        transform(va, 0, grow, c * CHUNK + h * 64);
+        transform(vb, 1, grow, c * CHUNK + h * 64 + 32);
+      }
+    };
+    // this thread's running maximum of the row and sum of 2^(t - max)
+    float m_run, s_run;
+    // takes 64 scores into (m_run, s_run) and leaves 2^(t - m_run) in their place (kKeep), or nothing.  A masked score's kept
+    // exponential has to be an exact zero, which the polynomial's is not: with a mask tensor it takes no part.
+    auto accumulate = [&](uint32_t (&va)[32], uint32_t (&vb)[32], auto keep) {
+      constexpr bool kKeep = decltype(keep)::value;
+      constexpr uint32_t poly = kKeep && additive ? 0u : poly_pairs;
+      float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        mx0 = max3(mx0, __uint_as_float(va[j]), __uint_as_float(va[j + 1]));
+        mx1 = max3(mx1, __uint_as_float(va[j + 2]), __uint_as_float(va[j + 3]));
+      }
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        mx0 = max3(mx0, __uint_as_float(vb[j]), __uint_as_float(vb[j + 1]));
+        mx1 = max3(mx1, __uint_as_float(vb[j + 2]), __uint_as_float(vb[j + 3]));
+      }
+      const float m_new = fmaxf(m_run, scale * fmaxf(mx0, mx1));
+      const float ref = m_new == -INFINITY ? 0.f : m_new;  // (nothing but masked columns so far)
+      float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 d = fma2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(scale), splat2(-ref));
+        const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
+        acc0 = add2(acc0, x);
+        if constexpr (kKeep) {
+          va[2 * j] = __float_as_uint(x.x);
+          va[2 * j + 1] = __float_as_uint(x.y);
+        }
+      }
+      {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float2 d = fma2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(scale), splat2(-ref));
+          const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
+          acc1 = add2(acc1, x);
+          if constexpr (kKeep) {
+            vb[2 * j] = __float_as_uint(x.x);
+            vb[2 * j + 1] = __float_as_uint(x.y);
+          }
+        }
+      }
+      const float2 acc = add2(acc0, acc1);
+      const float sum = m_new == -INFINITY ? 0.f : acc.x + acc.y;
+      s_run = fmaf(s_run, ex2_approx(m_run - ref), sum);
+      m_run = m_new;
+    };
+    auto load_slot = [&](uint32_t taddr, uint32_t (&va)[32], uint32_t (&vb)[32]) {
+#pragma unroll
+      for (int i = 0; i < 32; i += 16) {
+        tmem_ld_issue_16(taddr + i, va + i);
+        tmem_ld_issue_16(taddr + 32 + i, vb + i);
+      }
+#pragma unroll
+      for (int i = 0; i < 32; i += 16) {
+        tmem_ld_wait_16(va + i);
+        tmem_ld_wait_16(vb + i);
       }
     };
 
     for (int r = 0; r < rounds; ++r) {
       int b, mpair0, L;
       if (!tile_at(r, b, mpair0, L)) continue;
-      if (additive && mpair0 + static_cast<int>(pm) * 128 + q * 32 >= p.M) {
+      const int row0 = mpair0 + static_cast<int>(pm) * 128 + q * 32;  // the warp's first row
+      const int grow = row0 + lane;
+      if (additive && row0 >= p.M) {
         // none of this warp's rows exists (nor of the three it merges with): the accumulators are handed back as they come.
         // With boxes for all warps 134 x 1 x 720 took 35.0 us instead of 31.2, 64 x 16 x 1176 27.9 instead of 24.9.
-        for (int u = 0; u < (RES ? 1 : 2) * L; ++u, ++unit) {
-          wait_slot(static_cast<int>(unit & 1u));
-          release_slot(static_cast<int>(unit & 1u));
+        for (int u = 0; u < tile_units(L); ++u) {
+          wait_slot(slot);
+          release_slot(slot);
+          slot = next_slot(slot, u, L);
         }
         continue;
       }
-      float m_run = -INFINITY, s_run = 0.f;  // pass 0: this thread's running maximum and sum of 2^(t - max)
-      float off = INFINITY;                  // pass 1: P = 2^(t - off)
-      for (int u = 0; u < 2 * L; ++u) {
-        {
-          const int pass = u < L ? 0 : 1, c = u < L ? u : u - L;
-          const int m0 = mpair0 + static_cast<int>(pm) * 128;
-          const int grow = m0 + row;
-          // last live column of this thread's row, and of the warp's first / last row (fragment classification must be
-          // uniform over the warp so that the warp-wide TMEM loads stay convergent)
-          const int lim = p.causal ? (grow < p.N - 1 ? grow : p.N - 1) : p.N - 1;
-          const int wrow0 = m0 + q * 32;
-          const int lim_lo = p.causal ? (wrow0 < p.N - 1 ? wrow0 : p.N - 1) : p.N - 1;
-          const int lim_hi = p.causal ? (wrow0 + 31 < p.N - 1 ? wrow0 + 31 : p.N - 1) : p.N - 1;
-          // 2 = all 32 columns live for all 32 rows, 0 = none live for any row, 1 = mixed
-          auto frag_state = [&](int col0) { return col0 + 31 <= lim_lo ? 2 : (col0 > lim_hi ? 0 : 1); };
-
-          const int slot = static_cast<int>((RES && pass == 1 ? unit - static_cast<uint32_t>(L - c) : unit) & 1u);
-          if (!RES || pass == 0) {
-            ++unit;
-            wait_slot(slot);
+      m_run = -INFINITY;
+      s_run = 0.f;
+      float m_kept = -INFINITY;  // what the kept exponentials of the last chunk but one are relative to
+      // ---------------- pass 0: online (max, sum of 2^(t - max)) over this thread's columns of each chunk.  All columns of all
+      // chunks but the last are live.
+      for (int c = 0; c < L - 2; ++c) {
+        uint32_t va[32], vb[32];
+        wait_slot(slot);
+        load_slot(tmem_base + lane_sel + slot * CHUNK + h * 64, va, vb);
+        release_slot(slot);
+        slot ^= 1;
+        scores(va, vb, c, grow);
+        if constexpr (ADD) end_mask_use();
+        accumulate(va, vb, std::false_type{});
+      }
+      if (L >= 2) {  // the exponentials of the last chunk but one stay in its accumulator slot
+        uint32_t va[32], vb[32];
+        wait_slot(slot);
+        const uint32_t taddr = tmem_base + lane_sel + slot * CHUNK + h * 64;
+        load_slot(taddr, va, vb);
+        slot ^= 1;
+        scores(va, vb, L - 2, grow);
+        if constexpr (ADD) end_mask_use();
+        accumulate(va, vb, std::true_type{});
+        m_kept = m_run;
+#pragma unroll
+        for (int i = 0; i < 32; i += 16) {
+          tmem_st_16(taddr + i, va + i);
+          tmem_st_16(taddr + 32 + i, vb + i);
+        }
+        tmem_st_wait();
+      }
+      // the four column groups of the row (they live in the four warps of this lane quarter) meet: P = 2^(t - off)
+      auto meet = [&]() {
+        float2* pre = s_pre + tile_par * 512;
+        tile_par ^= 1u;
+        pre[h * 128 + row] = make_float2(m_run, s_run);
+        named_barrier_sync(1 + q, 128);
+        float m_row = -INFINITY, s_row = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 o = pre[i * 128 + row];
+          const float m_new = fmaxf(m_row, o.x);
+          if (m_new != -INFINITY) {
+            s_row = s_row * ex2_approx(m_row - m_new) + o.y * ex2_approx(o.x - m_new);
+            m_row = m_new;
           }
-          const uint32_t taddr = tmem_base + lane_sel + slot * CHUNK + h * 64;
-          const int colg = c * CHUNK + h * 64;
-          // RES: the masks of a row of two chunks take a box each, which pass 1 then fills; of one chunk box 0, pass 1 fills box 1
-          const uint32_t msel = !RES ? mask_n % YBOXES : my_chunks == 2 ? static_cast<uint32_t>(c) : (pass == 0 ? 0u : 1u);
-          const uint32_t mbox = ybox0 + msel * Cfg::WARP_BOX_BYTES;
-          if constexpr (ADD) {
-            if (!RES || pass == 0) reclaim_box();
-            if (colg < p.N && (!RES || pass == 0)) {
-              mbar_wait<false>(bar_yfull(e, msel), (RES && my_chunks < 2 ? mask_n : mask_n / YBOXES) & 1u, w);
-              __syncwarp();
-              ++mask_n;
+        }
+        // a row without a live column (cannot happen under the causal mask) is all zero: 2^(-inf)
+        return s_row > 0.f ? m_row + __log2f(s_row) : INFINITY;
+      };
+      // the factor of exponentials relative to m; a row without a sum is all zero (its NaN elements stay NaN)
+      auto factor = [&](float m, float off) { return off == INFINITY ? 0.f : ex2_approx(m - off); };
+      float off;
+      {
+        // ---------------- the last chunk: its exponentials stay in registers
+        const int colg = (L - 1) * CHUNK + h * 64;
+        const int lim = p.causal && grow < p.N - 1 ? grow : p.N - 1;  // last live column of this thread's row
+        const int lim_lo = p.causal && row0 < p.N - 1 ? row0 : p.N - 1;
+        const int lim_hi = p.causal && row0 + 31 < p.N - 1 ? row0 + 31 : p.N - 1;
+        wait_slot(slot);
+        if (colg <= lim_hi) {  // uniform over the warp
+          uint32_t va[32], vb[32];
+          load_slot(tmem_base + lane_sel + slot * CHUNK + h * 64, va, vb);
+          release_slot(slot);
+          scores(va, vb, L - 1, grow);
+          if constexpr (ADD) __syncwarp();
+          const bool whole = colg + 63 <= lim_lo;  // else it crosses the diagonal or the end of the row
+          if (!whole) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              if (colg + j > lim) va[j] = __float_as_uint(-INFINITY);
+              if (colg + 32 + j > lim) vb[j] = __float_as_uint(-INFINITY);
             }
           }
-          if (pass == 0) {
-            // ---------------- pass 0: online (max, sum of 2^(t - max)) over this thread's columns of the chunk
+          accumulate(va, vb, std::true_type{});
+          const float m_last = m_run;
+          off = meet();
+          const float f = factor(m_last, off);
+          uint32_t pk[32];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const int col0 = colg + half * 32;
-              const int st = frag_state(col0);
-              if (st == 0) continue;
-              uint32_t v[32];
-              tmem_ld_32cols(taddr + half * 32, v);
-              if (capped) {
+          for (int j = 0; j < 16; ++j) {
+            pk[j] = pack_bf16x2_rn(mul2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(f)));
+            pk[16 + j] = pack_bf16x2_rn(mul2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(f)));
+          }
+          if (!additive && !whole) {  // (the polynomial's exponential of a masked score is not zero)
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
-              }
-              float2 tv[16];
-              if (additive) {  // a full-tensor operand of the epilogue (Sec. 5.2)
-                float2 m2[16];
-                if constexpr (ADD) box_mask(mbox, half, m2);
-                else load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) tv[j] = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
-              } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) tv[j] = mul2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc));
-              }
-              if (st != 2) {  // the fragment crosses the diagonal (or the end of the row): rare, kept out of the main path
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  if (col0 + 2 * j > lim) tv[j].x = -INFINITY;
-                  if (col0 + 2 * j + 1 > lim) tv[j].y = -INFINITY;
-                }
-              }
-              if constexpr (RES) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  v[2 * j] = __float_as_uint(tv[j].x);
-                  v[2 * j + 1] = __float_as_uint(tv[j].y);
-                }
-                tmem_st_32cols(taddr + half * 32, v);
-              }
-              float mx0 = m_run, mx1 = -INFINITY;
-#pragma unroll
-              for (int j = 0; j < 16; j += 2) {
-                mx0 = max3(mx0, tv[j].x, tv[j].y);
-                mx1 = max3(mx1, tv[j + 1].x, tv[j + 1].y);
-              }
-              const float m_new = fmaxf(mx0, mx1);
-              if ((st == 2 && !additive) || m_new != -INFINITY) {  // else every column seen so far is masked for this row
-                float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
-                const float2 neg_m = splat2(-m_new);
-#pragma unroll
-                for (int j = 0; j < 16; j += 2) {
-                  const float2 d0 = add2(tv[j], neg_m), d1 = add2(tv[j + 1], neg_m);
-                  acc0 = add2(acc0, ((poly_pairs >> j) & 1u) ? ex2_poly2(d0) : make_float2(ex2_approx(d0.x), ex2_approx(d0.y)));
-                  acc1 = add2(acc1, ((poly_pairs >> (j + 1)) & 1u) ? ex2_poly2(d1) : make_float2(ex2_approx(d1.x), ex2_approx(d1.y)));
-                }
-                const float2 acc = add2(acc0, acc1);
-                s_run = fmaf(s_run, ex2_approx(m_run - m_new), acc.x + acc.y);
-                m_run = m_new;
-              }
+            for (int j = 0; j < 32; ++j) {
+              if (colg + 2 * j > lim) pk[j] = 0u;
+              else if (colg + 2 * j + 1 > lim) pk[j] &= 0xffffu;
             }
-            if constexpr (RES) tmem_st_wait();
-            else release_slot(slot);
-            if (ADD && colg < p.N) {
-              __syncwarp();  // every lane has read its row of the box
-              if (elected && (!RES || my_chunks < 2)) request_mask();
-              __syncwarp();
-            }
-          } else {
-            // ---------------- pass 1: the scores again, normalised, rounded once, staged and stored
+          }
+          emit(pk, colg, row0, b);
+        } else {
+          release_slot(slot);
+          if constexpr (ADD) reclaim_box();
+          off = meet();
+          if (colg < p.N) {  // above the diagonal
             uint32_t pk[32];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const int col0 = colg + half * 32;
-              const int st = frag_state(col0);
-              if (st == 0) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) pk[half * 16 + j] = 0u;
-              } else {
-                uint32_t v[32];
-                tmem_ld_32cols(taddr + half * 32, v);
-                if (!RES && capped) {
-#pragma unroll
-                  for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
-                }
-                float2 ev[16];
-                if constexpr (RES) {
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) {  // (a masked score is -inf, and so is -inf - off: its probability is an exact zero)
-                    const float2 t01 = add2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(-off));
-                    ev[j] = make_float2(ex2_approx(t01.x), ex2_approx(t01.y));
-                  }
-                } else if constexpr (additive) {
-                  float2 m2[16];
-                  if constexpr (ADD) box_mask(mbox, half, m2);
-                  else load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) {  // (a masked score is -inf, and so is -inf - off: its probability is an exact zero)
-                    const float2 t01 = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), add2(m2[j], splat2(-off)));
-                    ev[j] = make_float2(ex2_approx(t01.x), ex2_approx(t01.y));
-                  }
-                } else {
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) {
-                    const float2 t01 = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), splat2(-off));
-                    ev[j] = ((poly_pairs >> j) & 1u) ? ex2_poly2(t01) : make_float2(ex2_approx(t01.x), ex2_approx(t01.y));
-                  }
-                }
-                if (st != 2) {  // crosses the diagonal (or the end of the row)
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) {
-                    if (col0 + 2 * j > lim) ev[j].x = 0.f;
-                    if (col0 + 2 * j + 1 > lim) ev[j].y = 0.f;
-                  }
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) pk[half * 16 + j] = pack_bf16x2_rn(ev[j]);
-              }
-            }
-            release_slot(slot);
-            if (RES) reclaim_box();  // (no accumulator wait in front of this unit: the store has had the arithmetic's time instead)
-            if (colg < p.N) {
-              const uint32_t sel = ADD ? msel : nbox % YBOXES;
-              const uint32_t ybox = ybox0 + sel * Cfg::WARP_BOX_BYTES;
-              // the store of the box's previous contents has read it out (ADD: the box holds this unit's mask, every lane has
-              // read its own row of it and now overwrites that row)
-              if (!ADD) mbar_wait<false>(bar_yfree(e, sel), ((nbox / YBOXES) & 1u) ^ 1u, w);
-              ++nbox;
-              __syncwarp();
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const uint32_t a = ybox + static_cast<uint32_t>(lane * 128 + ((i ^ (lane & 7)) << 4));  // 128-byte swizzle
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(pk[4 * i]), "r"(pk[4 * i + 1]),
-                             "r"(pk[4 * i + 2]), "r"(pk[4 * i + 3])
-                             : "memory");
-              }
-              fence_proxy_async_smem();
-              __syncwarp();
-              if constexpr (ADD) {
-                if (elected) {
-                  if (COMFUSE_IN_BOUNDS(colg >= 0 && colg < p.N && (colg & 7) == 0 && mpair0 >= 0 && b >= 0 && b < p.batch, p.status))
-                  tma_store_3d_hint(&tmY, ybox, colg, m0 + q * 32, b, stream_box);
-                  tma_store_commit();
-                }
-                __syncwarp();
-                store_pending = true;
-              } else {
-                if (lane == 0) mbar_arrive(bar_yfull(e, sel));
-              }
-            }
+            for (int j = 0; j < 32; ++j) pk[j] = 0u;
+            emit(pk, colg, row0, b);
           }
         }
-        if (u == L - 1) {
-          // ---------------- pass 0 of the tile is complete: merge the four column groups of the row (they live in the
-          // four warps of this lane quarter); the result serves the tile's pass 1, which starts with the next unit
-          float2* pre = s_pre + tile_par * 512;
-          tile_par ^= 1u;
-          pre[h * 128 + row] = make_float2(m_run, s_run);
-          named_barrier_sync(1 + q, 128);
-          float m_row = -INFINITY, s_row = 0.f;
+        slot = next_slot(slot, L - 1, L);
+      }
+      if (L >= 2) {
+        // ---------------- the chunk before it: its exponentials are in its accumulator slot
+        const int kslot = slot ^ 1;
+        uint32_t va[32], vb[32];
+        load_slot(tmem_base + lane_sel + kslot * CHUNK + h * 64, va, vb);
+        release_slot(kslot);
+        const float f = factor(m_kept, off);
+        uint32_t pk[32];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 o = pre[i * 128 + row];
-            const float m_new = fmaxf(m_row, o.x);
-            if (m_new != -INFINITY) {
-              s_row = s_row * ex2_approx(m_row - m_new) + o.y * ex2_approx(o.x - m_new);
-              m_row = m_new;
-            }
-          }
-          // a row without a live column (cannot happen under the causal mask) is all zero: 2^(-inf)
-          off = s_row > 0.f ? m_row + __log2f(s_row) : INFINITY;
+        for (int j = 0; j < 16; ++j) {
+          pk[j] = pack_bf16x2_rn(mul2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(f)));
+          pk[16 + j] = pack_bf16x2_rn(mul2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(f)));
         }
+        reclaim_box();
+        emit(pk, (L - 2) * CHUNK + h * 64, row0, b);
+      }
+      // ---------------- pass 1: the other chunks' scores again, normalised, rounded once, staged and stored
+      for (int c = 0; c < L - 2; ++c) {
+        wait_slot(slot);
+        uint32_t va[32], vb[32];
+        load_slot(tmem_base + lane_sel + slot * CHUNK + h * 64, va, vb);
+        release_slot(slot);
+        scores(va, vb, c, grow);
+        if constexpr (ADD) __syncwarp();  // every lane has read its row of the mask
+        constexpr uint32_t poly = additive ? 0u : poly_pairs;
+        uint32_t pk[32];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float2 d0 = fma2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(scale), splat2(-off));
+          const float2 d1 = fma2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(scale), splat2(-off));
+          pk[j] = pack_bf16x2_rn(((poly >> j) & 1u) ? ex2_poly2(d0) : make_float2(ex2_approx(d0.x), ex2_approx(d0.y)));
+          pk[16 + j] = pack_bf16x2_rn(((poly >> j) & 1u) ? ex2_poly2(d1) : make_float2(ex2_approx(d1.x), ex2_approx(d1.y)));
+        }
+        emit(pk, c * CHUNK + h * 64, row0, b);
+        slot ^= 1;
       }
     }
-    if (ADD && elected) tma_store_wait_read<0>();  // the boxes must outlive the last store's read
+    if (elected) tma_store_wait_read<0>();  // the boxes must outlive the last store's read
   }
 
   // -------------------------------------------------------------------------------------------- teardown
