@@ -35,6 +35,7 @@ struct FewRowsCfg {
   static constexpr int W_BYTES = NT * 128 * 64 * 2;         // weights of one K block
   static constexpr int X_BYTES = MT * 64 * 2;               // rows of one K block
   static constexpr int STAGE_BYTES = W_BYTES + X_BYTES;
+  static constexpr int PREFETCH_BLOCKS = 384 * 1024 / W_BYTES;  // 148 CTAs ask for less than half of the L2
   static constexpr int ROW_BYTES = NT * 128 * 4;            // one row of the CTA's columns, fp32
   static constexpr int RECV_BYTES = (MT + 7) * ROW_BYTES;   // partial sums of the CTA's row slice from up to 8 shares (8 * ceil(MT / 8) rows)
   static constexpr int STAT_BYTES = MT * 16 * 8;            // one exchange: up to 16 partials per row
@@ -151,6 +152,18 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     mbar_arrive_expect_tx(bar_max, static_cast<uint32_t>(ct == 0 ? p.ct * rv * 8 : 0));
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmX);
+  }
+  // The weights are asked of the L2 while the previous kernel still runs: a prefetch returns nothing, so it may stand in front of the
+  // wait whoever writes the weights (writes meet in the L2 too).  40 x 4096 x 4096, weights from memory: 13.1 -> 12.1 us, the
+  // finishing kernel of the call before now covers 33 MB of reads; in the L2 already: 10.7 both ways.  One row group asks.  Not where
+  // one kernel does it all: its successor's CTAs come too late for it to pay (48 x 960 x 3664 10.1 / 10.2, 69 x 3880 x 336 9.06 / 9.13
+  // with weights from memory, 10.2 / 10.4 and 9.0 / 9.1 from the L2).
+  if (p.wide && warp == 2 && grp == 0 && elect_one()) {
+    const int last = kb1 - kb0 < Cfg::PREFETCH_BLOCKS ? kb1 : kb0 + Cfg::PREFETCH_BLOCKS;
+    for (int kb = kb0; kb < last; ++kb)
+#pragma unroll
+      for (int j = 0; j < 2 * NT; ++j)
+        tma_prefetch_l2_3d(&tmW, p.b_nk ? kb * 64 : n0 + j * 64, p.b_nk ? n0 + j * 64 : kb * 64, b);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(s_tmem_base), Cfg::TMEM_COLS);

@@ -201,6 +201,10 @@ __device__ __forceinline__ void tell_cluster(volatile int* told, uint32_t cluste
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
+// Asks the L2 for a box; nothing waits for it.
+__device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap* tm, int x, int y, int z) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(x), "r"(y), "r"(z) : "memory");
+}
 // Tiled 3-D load global -> this CTA's shared memory, completing `bar` with the box's byte count.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int x, int y, int z) {
   asm volatile(
