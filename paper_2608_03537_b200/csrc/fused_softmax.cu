@@ -8,10 +8,8 @@ cudaError_t launch_fused_softmax(const GemmMaps& maps, const FusedParams& p, cud
   // Short K: recomputing a score chunk is cheaper than keeping the row block on-chip across a cluster.
   // COMFUSE_SOFTMAX_CLUSTER=1 forces the cluster kernel where it has an instantiation (for comparisons).
   static const bool force_cluster = std::getenv("COMFUSE_SOFTMAX_CLUSTER") != nullptr;
-  // ... unless the problem is so small that the row kernel's CTA pairs do not fill the machine: up to 32 pairs of row blocks
-  // (8192 rows) of 768 columns or more run faster on clusters, which put 4 to 16 CTAs on every pair.  Measured at 8192 rows,
-  // K = 64 (row kernel / cluster kernel, us): N = 768: 22.3 / 15.2, 1024: 19.1 / 15.7, 2048 causal: 31.8 / 26.5, 4096: 59.1 / 50.7;
-  // at 16384 rows the row kernel is ahead again (N = 2048 causal: 32.5 / 41.4), and far ahead once the output outgrows L2.
+  // ... unless the problem is so small that the row kernel's CTA pairs do not fill the machine: then clusters, which put 4 to 16 CTAs on
+  // every pair of row blocks, are faster.
   // A row length between two instantiations runs on the next wider one: the columns from N on read as zeros and are
   // masked like the ones above the diagonal of a causal mask.
   static const int kForms[] = {256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2560, 3072, 3584, 4096};
@@ -19,7 +17,14 @@ cudaError_t launch_fused_softmax(const GemmMaps& maps, const FusedParams& p, cud
   for (int f : kForms)
     if (form == 0 && p.N <= f) form = f;
   const long long row_pairs = static_cast<long long>(p.batch) * ((p.M + 255) / 256);
-  const bool small = row_pairs <= 32 && form >= 768 && p.N > form / 2;
+  // Few row blocks: the cluster kernel, up to where its clusters need a third round (of the narrower forms' a second or third is still
+  // level).  Measured, cluster / row kernel, us, K = 64: 1280 columns 20 / 24 pairs of row blocks 14.6 / 15.8, 19.4 / 15.8; 1536
+  // 13.6 / 18.7, 23.1 / 18.7; 1792 20.3 / 21.2, 25.2 / 21.3; 2048 28 / 32 pairs 21.9 / 23.8, 29.9 / 23.8 (causal 25.2 / 23.1);
+  // 2560 20 / 24 pairs 25.7 / 28.6, 36.1 / 28.6; 3072 12 / 16 / 24 25.6 / 33.4, 36.2 / 33.5, 47.3 / 33.5; 3584 37.2 / 38.7, 47.9 / 38.7; 4096
+  // 28 / 32 pairs 41.4 / 44.0, 50.0 / 43.8; 1024 32 pairs 13.8 / 13.5, causal, K = 128, 13.5 / 14.5.
+  // A soft-cap (two MUFU operations a score, which the row kernel pays in both passes): up to 32 pairs (4 x 1864 x 1864 causal 40.8 / 49.5).
+  const int most = form <= 1024 || p.softcap > 0.f ? 32 : form == 2048 ? 30 : form == 4096 ? 28 : form == 3072 ? 14 : 22;
+  const bool small = row_pairs <= most && form >= 768 && p.N > form / 2;
   if (softmax_rows_supported(p) && !force_cluster && !small) return supported_only ? cudaSuccess : launch_softmax_rows(maps, p, st);
 #define COMFUSE_CASE(n, b0, b1, cn, nst, epw) \
   case n:                                     \

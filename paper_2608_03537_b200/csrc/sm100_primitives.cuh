@@ -526,11 +526,12 @@ __device__ __forceinline__ float2 f2_from_bits(uint32_t a, uint32_t b) { return 
 // the two bf16 halves of a packed word, widened exactly
 // 2^x for two values on the FMA pipe, without the MUFU unit (which the ex2 instruction shares with shared-memory and
 // global stores through the SM's memory-instruction queue): x = n + f with n = round(x), |f| <= 0.5; 2^f by a degree-4
-// minimax polynomial (relative error 4.2e-6); the exponent is added to the float's bit pattern.  x is clamped at -126
-// (results below 2^-126 come out as 2^-126); meant for x <= 0.
+// minimax polynomial (relative error 4.2e-6); the exponent is added to the float's bit pattern.  x is clamped at -127, whose
+// bit pattern comes out as an exact zero (a masked score is -inf); what lies between 2^-127 and 2^-126 is some value
+// below 2^-126.  Meant for x <= 0.
 __device__ __forceinline__ float2 ex2_poly2(float2 x) {
-  x.x = fmaxf(x.x, -126.f);
-  x.y = fmaxf(x.y, -126.f);
+  x.x = fmaxf(x.x, -127.f);
+  x.y = fmaxf(x.y, -127.f);
   const float2 r = add2(x, splat2(12582912.f));  // 1.5 * 2^23: the low mantissa bits of r hold n in two's complement
   const float2 n = add2(r, splat2(-12582912.f));
   const float2 f = fma2(n, splat2(-1.f), x);

@@ -14,12 +14,12 @@ cudaError_t launch_softmax_rows(const GemmMaps& maps, FusedParams p, cudaStream_
   constexpr int NSTAGES = 2, YBOXES = 2;
   using Cfg = RowSoftmaxCfg<NSTAGES, YBOXES>;
   const RowMask mask = !p.mask ? kNoMask : p.M <= 32 ? kMaskThreads : kMaskBoxes;
-  using Kernel = decltype(&softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>);
-  static constexpr Kernel kKernels[3][2] = {
-      {softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask>, softmax_rows_kernel<NSTAGES, YBOXES, true, kNoMask>},
-      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskThreads>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskThreads>},
-      {softmax_rows_kernel<NSTAGES, YBOXES, false, kMaskBoxes>, softmax_rows_kernel<NSTAGES, YBOXES, true, kMaskBoxes>}};
-  const Kernel kern = kKernels[mask][p.b_nk ? 1 : 0];
+  using Kernel = decltype(&softmax_rows_kernel<NSTAGES, YBOXES, false, kNoMask, false>);
+#define COMFUSE_FORMS(mask, cap) {softmax_rows_kernel<NSTAGES, YBOXES, false, mask, cap>, softmax_rows_kernel<NSTAGES, YBOXES, true, mask, cap>}
+  static constexpr Kernel kKernels[6][2] = {COMFUSE_FORMS(kNoMask, false), COMFUSE_FORMS(kMaskThreads, false), COMFUSE_FORMS(kMaskBoxes, false),
+                                            COMFUSE_FORMS(kNoMask, true), COMFUSE_FORMS(kMaskThreads, true), COMFUSE_FORMS(kMaskBoxes, true)};
+#undef COMFUSE_FORMS
+  const Kernel kern = kKernels[mask + (p.softcap > 0.f ? 3 : 0)][p.b_nk ? 1 : 0];
   const DeviceInfo* dev = current_device_info();
   if (!dev) return cudaErrorInvalidDevice;
   constexpr int kMaxDev = 64;

@@ -20,10 +20,11 @@
 //
 // What bounds it: the exponentials (MUFU: 16 results per clock and SM; a pass over 64 x 32 scores of all sixteen warps takes
 // 1640 clocks in a loop of its own) and, where the output outgrows the L2, the writes.  64 x 2048 x 2048 causal, K = 64 (537 MB
-// written, 85 us at the best rate of any store pattern measured here): 122.5 -> 116.2 us, without its stores 99 -> 76.  A thread
+// written, 85 us at the best rate of any store pattern measured here): 122.5 -> 115.2 us, without its stores 99 -> 76.  A thread
 // holds all its 64 columns of a chunk, so the accumulator is handed back before the arithmetic, which needs the registers that
-// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 33.4 -> 29.1 us; thirty shapes drawn from
-// 16 .. 2048 rows and 64 .. 2048 columns 0.995 .. 1.46 times as fast (geometric mean 1.13).
+// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 33.4 -> 27.7 us; thirty shapes drawn from
+// 16 .. 2048 rows and 64 .. 2048 columns 0.995 .. 1.49 times as fast (geometric mean 1.16).  A kernel without a soft-cap carries no code for one:
+// a CTA runs through a few tiles only, and the first one waits for every line of code it is the first to reach (96 x 504 x 504 29.1 / 28.2).
 //
 // Warp roles: warp 0 TMA producer, warp 1 TMEM allocation + UMMA issue (even CTA), warp 2 zero boxes, warp 3 idle (register
 // shares are given to groups of four warps); then 16 epilogue warps (thread = row; warp e takes lane quarter e % 4 and
@@ -85,7 +86,7 @@ struct RowSoftmaxCfg {
 // kMaskBoxes (ADD): every epilogue warp's 32 x 64 mask box arrives by TMA in one of the warp's staging boxes, which also
 // take the result: read the box, overwrite it with the probabilities, store it.
 enum RowMask { kNoMask, kMaskThreads, kMaskBoxes };
-template <int NSTAGES, int YBOXES, bool BKM, RowMask MASK>
+template <int NSTAGES, int YBOXES, bool BKM, RowMask MASK, bool CAP>
 __global__ void __launch_bounds__(32 * 20, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmY, const FusedParams p) {
@@ -288,15 +289,16 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const uint32_t lane_sel = static_cast<uint32_t>(q * 32) << 16;
     const uint32_t tempty_leader = map_to_cta(bar_tempty(0), 0);
     const uint32_t ybox0 = smem_base + Cfg::OFF_YBUF + e * YBOXES * Cfg::WARP_BOX_BYTES;
-    // log2 domain: t = Acc * (alpha * log2 e), so exp(x - m) = 2^(t - m_t)
-    // with a soft-cap the accumulators are mapped to capped log2-domain scores right after they are loaded, and the scale is 1
-    const bool capped = p.softcap > 0.f;
-    const SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
-    const float sc = capped ? 1.f : p.alpha * 1.4426950408889634f;
+    // Exponentials are 2^(scale * t - ..), t a score.  plain: t is the accumulator and the scale alpha * log2 e (a positive one);
+    // mask boxes: t = alpha * Acc + mask and the scale log2 e, one fused multiply-add a pair instead of a multiplication more;
+    // otherwise t is transformed to the log2 domain first.
+    constexpr float kLog2e = 1.4426950408889634f;
     constexpr bool additive = MASK != kNoMask;  // additive mask tensor, applied behind the scale / soft-cap
-    // plain: the scale is positive and nothing else happens to a score, so it can be folded into the exponential's argument
-    const bool plain = !additive && !capped && sc > 0.f;
-    const float scale = plain ? sc : 1.f;
+    SoftcapLog2 cap_fn(p.alpha, CAP ? p.softcap : 1.f);
+    if (ADD) cap_fn.c1 = p.softcap;
+    const float sc = CAP ? 1.f : ADD ? p.alpha : p.alpha * kLog2e;
+    const bool plain = !additive && !CAP && sc > 0.f;
+    const float scale = plain ? sc : ADD ? kLog2e : 1.f;
     constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
 
     int slot = 0;
@@ -404,9 +406,9 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       __syncwarp();
       store_pending = true;
     };
-    // scores of 32 columns in the log2 domain, in place (not in the plain case): soft-cap or scale, mask
+    // scores of 32 columns, in place (not in the plain case): soft-cap or scale, mask
     auto transform = [&](uint32_t (&v)[32], int half, int grow, int col0) {
-      if (capped) {
+      if constexpr (CAP) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
       }
@@ -421,8 +423,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                        : "memory");
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const float2 m2 = mul2(bf16x2_to_f2(w4[k]), splat2(1.4426950408889634f));
-            const float2 t = fma2(f2_from_bits(v[8 * i + 2 * k], v[8 * i + 2 * k + 1]), splat2(sc), m2);
+            const float2 t = fma2(f2_from_bits(v[8 * i + 2 * k], v[8 * i + 2 * k + 1]), splat2(sc), bf16x2_to_f2(w4[k]));
             v[8 * i + 2 * k] = __float_as_uint(t.x);
             v[8 * i + 2 * k + 1] = __float_as_uint(t.y);
           }
@@ -436,7 +437,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           v[2 * j] = __float_as_uint(t.x);
           v[2 * j + 1] = __float_as_uint(t.y);
         }
-      } else if (!capped) {
+      } else if constexpr (!CAP) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
       }
@@ -457,7 +458,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // exponential has to be an exact zero, which the polynomial's is not: with a mask tensor it takes no part.
     auto accumulate = [&](uint32_t (&va)[32], uint32_t (&vb)[32], auto keep) {
       constexpr bool kKeep = decltype(keep)::value;
-      constexpr uint32_t poly = kKeep && additive ? 0u : poly_pairs;
+      constexpr uint32_t poly = poly_pairs;
       float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
@@ -612,13 +613,6 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             pk[j] = pack_bf16x2_rn(mul2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(f)));
             pk[16 + j] = pack_bf16x2_rn(mul2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(f)));
           }
-          if (!additive && !whole) {  // (the polynomial's exponential of a masked score is not zero)
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              if (colg + 2 * j > lim) pk[j] = 0u;
-              else if (colg + 2 * j + 1 > lim) pk[j] &= 0xffffu;
-            }
-          }
           emit(pk, colg, row0, b);
         } else {
           release_slot(slot);
@@ -657,7 +651,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         release_slot(slot);
         scores(va, vb, c, grow);
         if constexpr (ADD) __syncwarp();  // every lane has read its row of the mask
-        constexpr uint32_t poly = additive ? 0u : poly_pairs;
+        constexpr uint32_t poly = poly_pairs;
         uint32_t pk[32];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
