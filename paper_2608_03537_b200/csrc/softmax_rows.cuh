@@ -39,6 +39,18 @@
 
 namespace comfuse {
 
+// Maxima that are NaN if an argument is: a row with a NaN score (or one of +inf) comes out as NaN, whichever column it stands in.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
 template <int NSTAGES, int YBOXES>
 struct RowSoftmaxCfg {
   static constexpr int kEpiWarps = 16;
@@ -454,23 +466,22 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     };
     // this thread's running maximum of the row and sum of 2^(t - max)
     float m_run, s_run;
-    // takes 64 scores into (m_run, s_run) and leaves 2^(t - m_run) in their place (kKeep), or nothing.  A masked score's kept
-    // exponential has to be an exact zero, which the polynomial's is not: with a mask tensor it takes no part.
+    // takes 64 scores into (m_run, s_run) and leaves 2^(t - m_run) in their place (kKeep), or nothing
     auto accumulate = [&](uint32_t (&va)[32], uint32_t (&vb)[32], auto keep) {
       constexpr bool kKeep = decltype(keep)::value;
       constexpr uint32_t poly = poly_pairs;
       float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
-        mx0 = max3(mx0, __uint_as_float(va[j]), __uint_as_float(va[j + 1]));
-        mx1 = max3(mx1, __uint_as_float(va[j + 2]), __uint_as_float(va[j + 3]));
+        mx0 = max3_nan(mx0, __uint_as_float(va[j]), __uint_as_float(va[j + 1]));
+        mx1 = max3_nan(mx1, __uint_as_float(va[j + 2]), __uint_as_float(va[j + 3]));
       }
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
-        mx0 = max3(mx0, __uint_as_float(vb[j]), __uint_as_float(vb[j + 1]));
-        mx1 = max3(mx1, __uint_as_float(vb[j + 2]), __uint_as_float(vb[j + 3]));
+        mx0 = max3_nan(mx0, __uint_as_float(vb[j]), __uint_as_float(vb[j + 1]));
+        mx1 = max3_nan(mx1, __uint_as_float(vb[j + 2]), __uint_as_float(vb[j + 3]));
       }
-      const float m_new = fmaxf(m_run, scale * fmaxf(mx0, mx1));
+      const float m_new = max_nan(m_run, scale * max_nan(mx0, mx1));
       const float ref = m_new == -INFINITY ? 0.f : m_new;  // (nothing but masked columns so far)
       float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -570,16 +581,16 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 o = pre[i * 128 + row];
-          const float m_new = fmaxf(m_row, o.x);
+          const float m_new = max_nan(m_row, o.x);
           if (m_new != -INFINITY) {
             s_row = s_row * ex2_approx(m_row - m_new) + o.y * ex2_approx(o.x - m_new);
             m_row = m_new;
           }
         }
         // a row without a live column (cannot happen under the causal mask) is all zero: 2^(-inf)
-        return s_row > 0.f ? m_row + __log2f(s_row) : INFINITY;
+        return m_row == -INFINITY ? INFINITY : m_row + __log2f(s_row);
       };
-      // the factor of exponentials relative to m; a row without a sum is all zero (its NaN elements stay NaN)
+      // the factor of exponentials relative to m; a row without a live column is all zero
       auto factor = [&](float m, float off) { return off == INFINITY ? 0.f : ex2_approx(m - off); };
       float off;
       {
@@ -659,6 +670,10 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           const float2 d1 = fma2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(scale), splat2(-off));
           pk[j] = pack_bf16x2_rn(((poly >> j) & 1u) ? ex2_poly2(d0) : make_float2(ex2_approx(d0.x), ex2_approx(d0.y)));
           pk[16 + j] = pack_bf16x2_rn(((poly >> j) & 1u) ? ex2_poly2(d1) : make_float2(ex2_approx(d1.x), ex2_approx(d1.y)));
+        }
+        if (off != off) {  // a row with a NaN (the polynomial's clamp takes one for a masked score)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) pk[j] = 0x7FFF7FFFu;
         }
         emit(pk, c * CHUNK + h * 64, row0, b);
         slot ^= 1;
