@@ -22,7 +22,7 @@
 // 1640 clocks in a loop of its own) and, where the output outgrows the L2, the writes.  64 x 2048 x 2048 causal, K = 64 (537 MB
 // written, 85 us at the best rate of any store pattern measured here): 122.5 -> 115.2 us, without its stores 99 -> 76.  A thread
 // holds all its 64 columns of a chunk, so the accumulator is handed back before the arithmetic, which needs the registers that
-// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 33.4 -> 27.7 us; thirty shapes drawn from
+// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 34.3 -> 28.4 us a call; thirty shapes drawn from
 // 16 .. 2048 rows and 64 .. 2048 columns 0.995 .. 1.49 times as fast (geometric mean 1.16).  A kernel without a soft-cap carries no code for one:
 // a CTA runs through a few tiles only, and the first one waits for every line of code it is the first to reach (96 x 504 x 504 29.1 / 28.2).
 //
@@ -314,11 +314,10 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
 
     int slot = 0;
-    uint32_t slot_uses[2] = {0, 0};
-    uint32_t tile_par = 0;
+    uint32_t slot_phases = 0, tile_par = 0;
     auto wait_slot = [&](int sl) {
-      mbar_wait<false>(bar_tfull(sl), slot_uses[sl] & 1u, w);
-      ++slot_uses[sl];
+      mbar_wait<false>(bar_tfull(sl), (slot_phases >> sl) & 1u, w);
+      slot_phases ^= 1u << sl;
       __syncwarp();
       tcgen05_fence_after_sync();
     };
@@ -330,11 +329,9 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     // Staging boxes: use n of this warp takes box n % YBOXES.  A use holds the chunk's mask (ADD), its result, or first one and
     // then the other.  The elected lane issues the stores itself; it hands a box on when its store has read it, and asks for the
-    // mask of the box's next use then.
+    // mask of the box's next use then.  (The L2 policies are made where they are used: the 64 columns leave few registers.)
     const bool elected = elect_one();
     uint32_t use = 0;
-    const uint64_t stream_out = l2_policy_evict_first();  // the output is never read again
-    const uint64_t keep_mask = ADD ? l2_policy_evict_last() : 0;
     // ADD: the uses of a tile (causal off: L = nch) are nch - 1 masks, mask and result of the last chunk (if it has columns for
     // this warp), the result of the one before, masks and results of the others
     const bool has_last = (nch - 1) * CHUNK + h * 64 < p.N;
@@ -358,7 +355,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       if (c >= 0) {
         const uint32_t sel = req_use % YBOXES;
         mbar_arrive_expect_tx(bar_mask(e, sel), Cfg::WARP_BOX_BYTES);
-        tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_mask(e, sel), c * CHUNK + h * 64, req_row, 0, keep_mask);
+        tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_mask(e, sel), c * CHUNK + h * 64, req_row, 0, l2_policy_evict_last());
       }
       ++req_use;
       ++req_i;
@@ -412,7 +409,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       __syncwarp();
       if (elected) {
         if (COMFUSE_IN_BOUNDS(colg >= 0 && colg < p.N && (colg & 7) == 0 && row0 >= 0 && b >= 0 && b < p.batch, p.status))
-        tma_store_3d_hint(&tmY, ybox, colg, row0, b, stream_out);
+        tma_store_3d_hint(&tmY, ybox, colg, row0, b, l2_policy_evict_first());  // the output is never read again
         tma_store_commit();
       }
       __syncwarp();
@@ -483,12 +480,12 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
       const float m_new = max_nan(m_run, scale * max_nan(mx0, mx1));
       const float ref = m_new == -INFINITY ? 0.f : m_new;  // (nothing but masked columns so far)
-      float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+      float2 acc = make_float2(0.f, 0.f);  // (one pair of sums and no more: with two, mask boxes spill; 96 x 504 x 504 28.4 / 29.3 us)
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const float2 d = fma2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(scale), splat2(-ref));
         const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
-        acc0 = add2(acc0, x);
+        acc = add2(acc, x);
         if constexpr (kKeep) {
           va[2 * j] = __float_as_uint(x.x);
           va[2 * j + 1] = __float_as_uint(x.y);
@@ -499,14 +496,13 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         for (int j = 0; j < 16; ++j) {
           const float2 d = fma2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(scale), splat2(-ref));
           const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
-          acc1 = add2(acc1, x);
+          acc = add2(acc, x);
           if constexpr (kKeep) {
             vb[2 * j] = __float_as_uint(x.x);
             vb[2 * j + 1] = __float_as_uint(x.y);
           }
         }
       }
-      const float2 acc = add2(acc0, acc1);
       const float sum = m_new == -INFINITY ? 0.f : acc.x + acc.y;
       s_run = fmaf(s_run, ex2_approx(m_run - ref), sum);
       m_run = m_new;
