@@ -81,7 +81,8 @@ struct RowSoftmaxCfg {
   static constexpr int OFF_BAR = OFF_PRE + PRE_BYTES;
   static constexpr int NUM_BARS = 2 * NSTAGES + 4 + 1 + kEpiWarps * YBOXES;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
-  static constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;
+  static constexpr int OFF_REQ = OFF_MISC + 16;              // per epilogue warp: where its mask requests stand
+  static constexpr int SMEM_BYTES = OFF_REQ + kEpiWarps * 16 + 1024;
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
   static_assert(SMEM_BYTES > 116 * 1024, "one CTA per SM is assumed (TMEM allocation never waits for a co-resident CTA)");
   static_assert(NSTAGES >= 2 && NSTAGES <= 8 && YBOXES >= 1 && YBOXES <= 4, "ring and staging depths");
@@ -301,23 +302,37 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const uint32_t lane_sel = static_cast<uint32_t>(q * 32) << 16;
     const uint32_t tempty_leader = map_to_cta(bar_tempty(0), 0);
     const uint32_t ybox0 = smem_base + Cfg::OFF_YBUF + e * YBOXES * Cfg::WARP_BOX_BYTES;
-    // Exponentials are 2^(scale * t - ..), t a score.  plain: t is the accumulator and the scale alpha * log2 e (a positive one);
-    // mask boxes: t = alpha * Acc + mask and the scale log2 e, one fused multiply-add a pair instead of a multiplication more;
-    // otherwise t is transformed to the log2 domain first.
+    // Exponentials are 2^(scale * (t - maximum)), t a score.  plain: t is the accumulator and the scale alpha * log2 e (a positive one);
+    // with a mask: t = alpha * Acc + mask and the scale log2 e; otherwise t is transformed to the log2 domain first and the scale 1.
+    // With a mask the difference comes first, which is an exact zero for the maximum whatever its size: with the scaled maximum taken
+    // off in a fused multiply-add it is that product's rounding, hundreds for a column masked with -1e10.  Without one it is that
+    // multiply-add, and the other order where a maximum is beyond kFar (64 x 2048 x 2048 causal 114.4 us, with the difference first 115.0).
     constexpr float kLog2e = 1.4426950408889634f;
     constexpr bool additive = MASK != kNoMask;  // additive mask tensor, applied behind the scale / soft-cap
     SoftcapLog2 cap_fn(p.alpha, CAP ? p.softcap : 1.f);
-    if (ADD) cap_fn.c1 = p.softcap;
-    const float sc = CAP ? 1.f : ADD ? p.alpha : p.alpha * kLog2e;
+    if (additive) cap_fn.c1 = p.softcap;
+    const float sc = CAP ? 1.f : additive ? p.alpha : p.alpha * kLog2e;
     const bool plain = !additive && !CAP && sc > 0.f;
-    const float scale = plain ? sc : ADD ? kLog2e : 1.f;
-    constexpr uint32_t poly_pairs = Cfg::POLY_PAIRS;
+    const float scale = plain ? sc : additive ? kLog2e : 1.f;
+    constexpr float kFar = 1024.f;
+    auto any_far = [&](float scaled) { return !additive && !CAP && __any_sync(0xFFFFFFFFu, fabsf(scaled) > kFar); };  // (with a soft-cap the scale is 1)
+    auto take_off = [&](uint32_t (&va)[32], uint32_t (&vb)[32], float ref) {
+#pragma unroll
+      for (int j = 0; j < 32; j += 2) {
+        const float2 a = add2(f2_from_bits(va[j], va[j + 1]), splat2(-ref)), b = add2(f2_from_bits(vb[j], vb[j + 1]), splat2(-ref));
+        va[j] = __float_as_uint(a.x);
+        va[j + 1] = __float_as_uint(a.y);
+        vb[j] = __float_as_uint(b.x);
+        vb[j + 1] = __float_as_uint(b.y);
+      }
+    };
 
     int slot = 0;
-    uint32_t slot_phases = 0, tile_par = 0;
+    // phase bits: 0, 1 of the slots, 2 .. of the mask boxes, 31 which half of s_pre
+    uint32_t phases = 0;
     auto wait_slot = [&](int sl) {
-      mbar_wait<false>(bar_tfull(sl), (slot_phases >> sl) & 1u, w);
-      slot_phases ^= 1u << sl;
+      mbar_wait<false>(bar_tfull(sl), (phases >> sl) & 1u, w);
+      phases ^= 1u << sl;
       __syncwarp();
       tcgen05_fence_after_sync();
     };
@@ -336,9 +351,10 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // this warp), the result of the one before, masks and results of the others
     const bool has_last = (nch - 1) * CHUNK + h * 64 < p.N;
     const int tile_uses = tile_units(nch) + (nch >= 2 ? 1 : 0) - (has_last ? 0 : 1);
-    int req_r = -1, req_i = tile_uses, req_row = 0;
-    uint32_t req_use = 0, mask_phases = 0;
-    auto request_use = [&]() {  // (the elected lane) the mask of the next use not asked for yet, if it has one
+    // round, use and first row of the next request: in shared memory, read and written by the elected lane alone
+    volatile int* req = reinterpret_cast<volatile int*>(smem + Cfg::OFF_REQ) + 4 * e;
+    auto request_use = [&](uint32_t sel) {  // (the elected lane) the mask of the next use not asked for yet, if it has one, into its box
+      int req_r = req[0], req_i = req[1], req_row = req[2];
       if (req_i >= tile_uses) {
         req_i = 0;
         if (req_r < rounds) {
@@ -348,21 +364,24 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             req_row = lm + static_cast<int>(pm) * 128 + q * 32;
           } while (req_r < rounds && req_row >= p.M);
         }
+        req[0] = req_r;
+        req[2] = req_row;
       }
       if (tile_uses <= 0 || req_r >= rounds) return;
       const int first_out = nch - (has_last ? 0 : 1);  // the use without a mask
       const int c = req_i < first_out ? req_i : req_i - first_out - 1;
       if (c >= 0) {
-        const uint32_t sel = req_use % YBOXES;
         mbar_arrive_expect_tx(bar_mask(e, sel), Cfg::WARP_BOX_BYTES);
         tma_load_3d_hint(ybox0 + sel * Cfg::WARP_BOX_BYTES, &tmM, bar_mask(e, sel), c * CHUNK + h * 64, req_row, 0, l2_policy_evict_last());
       }
-      ++req_use;
-      ++req_i;
+      req[1] = req_i + 1;
     };
     if constexpr (ADD) {
-      if (elected)
-        for (int i = 0; i < YBOXES; ++i) request_use();
+      if (elected) {
+        req[0] = -1;
+        req[1] = tile_uses;
+        for (int i = 0; i < YBOXES; ++i) request_use(i);
+      }
       __syncwarp();
     }
     bool store_pending = false;
@@ -372,7 +391,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (!store_pending) return;
         if (elected) {
           tma_store_wait_read<0>();
-          request_use();
+          request_use((use + YBOXES - 1) % YBOXES);
         }
         __syncwarp();
         store_pending = false;
@@ -380,13 +399,13 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     };
     auto wait_mask = [&]() {
       const uint32_t sel = use % YBOXES;
-      mbar_wait<false>(bar_mask(e, sel), (mask_phases >> sel) & 1u, w);
-      mask_phases ^= 1u << sel;
+      mbar_wait<false>(bar_mask(e, sel), (phases >> (2 + sel)) & 1u, w);
+      phases ^= 4u << sel;
       __syncwarp();
     };
     auto end_mask_use = [&]() {  // the use held a mask only and every lane has read its row
       __syncwarp();
-      if (elected) request_use();
+      if (elected) request_use(use % YBOXES);
       __syncwarp();
       ++use;
     };
@@ -439,7 +458,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       } else if constexpr (additive) {
         float2 m2[16];
-        load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
+        load_mask_32(p.mask + static_cast<long long>(grow) * p.N + col0, grow < p.M ? p.N - col0 : 0, m2);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const float2 t = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
@@ -461,12 +480,12 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         transform(vb, 1, grow, c * CHUNK + h * 64 + 32);
       }
     };
-    // this thread's running maximum of the row and sum of 2^(t - max)
+    // this thread's running maximum of the row and sum of 2^(scale * (t - max))
     float m_run, s_run;
-    // takes 64 scores into (m_run, s_run) and leaves 2^(t - m_run) in their place (kKeep), or nothing
+    // takes 64 scores into (m_run, s_run) and leaves 2^(scale * (t - m_run)) in their place (kKeep), or nothing
     auto accumulate = [&](uint32_t (&va)[32], uint32_t (&vb)[32], auto keep) {
       constexpr bool kKeep = decltype(keep)::value;
-      constexpr uint32_t poly = poly_pairs;
+      constexpr uint32_t poly = Cfg::POLY_PAIRS;
       float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
@@ -478,33 +497,31 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         mx0 = max3_nan(mx0, __uint_as_float(vb[j]), __uint_as_float(vb[j + 1]));
         mx1 = max3_nan(mx1, __uint_as_float(vb[j + 2]), __uint_as_float(vb[j + 3]));
       }
-      const float m_new = max_nan(m_run, scale * max_nan(mx0, mx1));
+      const float m_new = max_nan(m_run, max_nan(mx0, mx1));
       const float ref = m_new == -INFINITY ? 0.f : m_new;  // (nothing but masked columns so far)
-      float2 acc = make_float2(0.f, 0.f);  // (one pair of sums and no more: with two, mask boxes spill; 96 x 504 x 504 28.4 / 29.3 us)
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float2 d = fma2(f2_from_bits(va[2 * j], va[2 * j + 1]), splat2(scale), splat2(-ref));
-        const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
-        acc = add2(acc, x);
-        if constexpr (kKeep) {
-          va[2 * j] = __float_as_uint(x.x);
-          va[2 * j + 1] = __float_as_uint(x.y);
-        }
+      float r = scale * ref;  // (not with a mask)
+      if (any_far(r)) {
+        take_off(va, vb, ref);
+        r = 0.f;
       }
-      {
+      float2 acc = make_float2(0.f, 0.f);  // (one pair of sums and no more: with two, mask boxes spill)
+      auto exponentials = [&](uint32_t (&v)[32]) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const float2 d = fma2(f2_from_bits(vb[2 * j], vb[2 * j + 1]), splat2(scale), splat2(-ref));
+          const float2 t = f2_from_bits(v[2 * j], v[2 * j + 1]);
+          const float2 d = additive ? mul2(add2(t, splat2(-ref)), splat2(scale)) : fma2(t, splat2(scale), splat2(-r));
           const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
           acc = add2(acc, x);
           if constexpr (kKeep) {
-            vb[2 * j] = __float_as_uint(x.x);
-            vb[2 * j + 1] = __float_as_uint(x.y);
+            v[2 * j] = __float_as_uint(x.x);
+            v[2 * j + 1] = __float_as_uint(x.y);
           }
         }
-      }
+      };
+      exponentials(va);
+      exponentials(vb);
       const float sum = m_new == -INFINITY ? 0.f : acc.x + acc.y;
-      s_run = fmaf(s_run, ex2_approx(m_run - ref), sum);
+      s_run = fmaf(s_run, ex2_approx(scale * (m_run - ref)), sum);
       m_run = m_new;
     };
     auto load_slot = [&](uint32_t taddr, uint32_t (&va)[32], uint32_t (&vb)[32]) {
@@ -567,34 +584,36 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
         tmem_st_wait();
       }
-      // the four column groups of the row (they live in the four warps of this lane quarter) meet: P = 2^(t - off)
+      // The four column groups of the row (they live in the four warps of this lane quarter) meet: P = 2^(scale * (t - m_row) - off), off
+      // the sum's logarithm.  A row without a live column (which cannot happen under the causal mask) is all zero: m_row 0 and off +inf.
+      float m_row, off;
       auto meet = [&]() {
-        float2* pre = s_pre + tile_par * 512;
-        tile_par ^= 1u;
+        float2* pre = s_pre + (phases >> 31) * 512;
+        phases ^= 1u << 31;
         pre[h * 128 + row] = make_float2(m_run, s_run);
         named_barrier_sync(1 + q, 128);
-        float m_row = -INFINITY, s_row = 0.f;
+        float m_all = -INFINITY, s_all = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 o = pre[i * 128 + row];
-          const float m_new = max_nan(m_row, o.x);
+          const float m_new = max_nan(m_all, o.x);
           if (m_new != -INFINITY) {
-            s_row = s_row * ex2_approx(m_row - m_new) + o.y * ex2_approx(o.x - m_new);
-            m_row = m_new;
+            s_all = s_all * ex2_approx(scale * (m_all - m_new)) + o.y * ex2_approx(scale * (o.x - m_new));
+            m_all = m_new;
           }
         }
-        // a row without a live column (cannot happen under the causal mask) is all zero: 2^(-inf)
-        return m_row == -INFINITY ? INFINITY : m_row + __log2f(s_row);
+        m_row = m_all == -INFINITY ? 0.f : m_all;
+        off = m_all == -INFINITY ? INFINITY : m_all < INFINITY ? __log2f(s_all) : NAN;
       };
-      // the factor of exponentials relative to m; a row without a live column is all zero
-      auto factor = [&](float m, float off) { return off == INFINITY ? 0.f : ex2_approx(m - off); };
-      float off;
+      // what turns exponentials relative to m into probabilities
+      auto factor = [&](float m) { return ex2_approx(fmaf(scale, m - m_row, -off)); };
       {
         // ---------------- the last chunk: its exponentials stay in registers
         const int colg = (L - 1) * CHUNK + h * 64;
-        const int lim = p.causal && grow < p.N - 1 ? grow : p.N - 1;  // last live column of this thread's row
-        const int lim_lo = p.causal && row0 < p.N - 1 ? row0 : p.N - 1;
-        const int lim_hi = p.causal && row0 + 31 < p.N - 1 ? row0 + 31 : p.N - 1;
+        const bool causal = !additive && p.causal;  // (one mask or the other)
+        const int lim = causal && grow < p.N - 1 ? grow : p.N - 1;  // last live column of this thread's row
+        const int lim_lo = causal && row0 < p.N - 1 ? row0 : p.N - 1;
+        const int lim_hi = causal && row0 + 31 < p.N - 1 ? row0 + 31 : p.N - 1;
         wait_slot(slot);
         if (colg <= lim_hi) {  // uniform over the warp
           uint32_t va[32], vb[32];
@@ -612,8 +631,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           }
           accumulate(va, vb, std::true_type{});
           const float m_last = m_run;
-          off = meet();
-          const float f = factor(m_last, off);
+          meet();
+          const float f = factor(m_last);
           uint32_t pk[32];
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -624,7 +643,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         } else {
           release_slot(slot);
           if constexpr (ADD) reclaim_box();
-          off = meet();
+          meet();
           if (colg < p.N) {  // above the diagonal
             uint32_t pk[32];
 #pragma unroll
@@ -640,7 +659,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t va[32], vb[32];
         load_slot(tmem_base + lane_sel + kslot * CHUNK + h * 64, va, vb);
         release_slot(kslot);
-        const float f = factor(m_kept, off);
+        const float f = factor(m_kept);
         uint32_t pk[32];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
@@ -651,6 +670,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         emit(pk, (L - 2) * CHUNK + h * 64, row0, b);
       }
       // ---------------- pass 1: the other chunks' scores again, normalised, rounded once, staged and stored
+      const bool far = any_far(scale * m_row);
+      if (!additive && !far) off = fmaf(scale, m_row, off);
       for (int c = 0; c < L - 2; ++c) {
         wait_slot(slot);
         uint32_t va[32], vb[32];
@@ -658,7 +679,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         release_slot(slot);
         scores(va, vb, c, grow);
         if constexpr (ADD) __syncwarp();  // every lane has read its row of the mask
-        constexpr uint32_t poly = poly_pairs;
+        if (additive || far) take_off(va, vb, m_row);
+        constexpr uint32_t poly = Cfg::POLY_PAIRS;
         uint32_t pk[32];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
