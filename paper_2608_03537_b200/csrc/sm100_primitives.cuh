@@ -523,25 +523,47 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 #endif
 __device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 f2_from_bits(uint32_t a, uint32_t b) { return make_float2(__uint_as_float(a), __uint_as_float(b)); }
-// the two bf16 halves of a packed word, widened exactly
 // 2^x for two values on the FMA pipe, without the MUFU unit (which the ex2 instruction shares with shared-memory and
 // global stores through the SM's memory-instruction queue): x = n + f with n = round(x), |f| <= 0.5; 2^f by a degree-4
 // minimax polynomial (relative error 4.2e-6); the exponent is added to the float's bit pattern.  x is clamped at -127, whose
 // bit pattern comes out as an exact zero (a masked score is -inf); what lies between 2^-127 and 2^-126 is some value
 // below 2^-126.  Meant for x <= 0.
+constexpr float kPoly2Round = 12582912.f;  // 1.5 * 2^23: behind its addition the low mantissa bits hold n in two's complement
+__device__ __forceinline__ float2 poly2_scale(float2 q, float2 r) {
+  return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(r.x) << 23)),
+                     __int_as_float(__float_as_int(q.y) + (__float_as_int(r.y) << 23)));
+}
 __device__ __forceinline__ float2 ex2_poly2(float2 x) {
   x.x = fmaxf(x.x, -127.f);
   x.y = fmaxf(x.y, -127.f);
-  const float2 r = add2(x, splat2(12582912.f));  // 1.5 * 2^23: the low mantissa bits of r hold n in two's complement
-  const float2 n = add2(r, splat2(-12582912.f));
+  const float2 r = add2(x, splat2(kPoly2Round));
+  const float2 n = add2(r, splat2(-kPoly2Round));
   const float2 f = fma2(n, splat2(-1.f), x);
   float2 q = fma2(splat2(0.009689519181847572f), f, splat2(0.055905185639858246f));
   q = fma2(q, f, splat2(0.24021807312965393f));
   q = fma2(q, f, splat2(0.6931246519088745f));
   q = fma2(q, f, splat2(1.f));
-  return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(r.x) << 23)),
-                     __int_as_float(__float_as_int(q.y) + (__float_as_int(r.y) << 23)));
+  return poly2_scale(q, r);
 }
+// e^x in the same way, to the accuracy of the ex2 instruction (2.4e-7): a degree-5 minimax polynomial (coefficients from a linear program
+// over the relative error; 1.7e-7 with its fp32 roundings).  The multiplication by log2 e goes into the rounding and the remainder.  Below
+// -88.029 (just above -127 in the log2 domain, so that f is not negative there, which would borrow from the exponent) it is some
+// value below 2^-136, which bf16 rounds to zero.
+__device__ __forceinline__ float2 exp_poly2(float2 x) {
+  constexpr float kLog2e = 1.4426950408889634f;
+  x.x = fmaxf(x.x, -88.029f);
+  x.y = fmaxf(x.y, -88.029f);
+  const float2 r = fma2(x, splat2(kLog2e), splat2(kPoly2Round));
+  const float2 n = add2(r, splat2(-kPoly2Round));
+  const float2 f = fma2(x, splat2(kLog2e), make_float2(-n.x, -n.y));
+  float2 q = fma2(splat2(0.001326472032815218f), f, splat2(0.009671512991189957f));
+  q = fma2(q, f, splat2(0.05550733953714371f));
+  q = fma2(q, f, splat2(0.24022242426872253f));
+  q = fma2(q, f, splat2(0.6931470036506653f));
+  q = fma2(q, f, splat2(1.f));
+  return poly2_scale(q, r);
+}
+// the two bf16 halves of a packed word, widened exactly
 __device__ __forceinline__ float2 bf16x2_to_f2(uint32_t u) { return make_float2(bf16_lo(u), bf16_hi(u)); }
 __device__ __forceinline__ uint32_t pack_bf16x2_rn(float2 v) { return pack_bf16x2_rn(v.x, v.y); }
 // GELU, tanh form, on a pair: six packed instructions and two MUFU.TANH

@@ -69,6 +69,8 @@ struct RowSoftmaxCfg {
   // polynomial costs about six issue slots per value.  Measured on the attention-score workload: none 126.2 us,
   // 4 of 16 pairs 122.7, 8: 128.8, when both passes exponentiated every score.  Now, with the writes in the way, 116.6 / 116.3 / 117.6
   // for none / 4 / 6; without them 81.9 / 76.2 / 81.8 for none / 4 / 8.
+  // With a mask: a polynomial as accurate as the instruction, and in the statistics pass and the kept chunks only
+  // (16 x 2048 x 2048 64.2 us, with it in the second pass too 64.4; 96 x 504 x 504 27.9, with the instruction alone 28.2).
   static constexpr uint32_t POLY_PAIRS = 0x1248u;            // pairs 3, 6, 9, 12
   static constexpr int A_BYTES = 128 * 64 * 2;
   static constexpr int STAGE_BYTES = A_BYTES + (CHUNK / 2) * 64 * 2;  // A block + this CTA's half of the B chunk
@@ -504,14 +506,29 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         take_off(va, vb, ref);
         r = 0.f;
       }
-      float2 acc = make_float2(0.f, 0.f);  // (one pair of sums and no more: with two, mask boxes spill)
+      // Sums of a few pairs at a time: one chain of 32 rounds more often.  (Two are what costs nothing without a mask: 96 x 512 x 512
+      // 17.9 us, four 18.5, four chains of eight 18.5.)
+      constexpr int kGroup = additive ? 4 : 2;
+      float2 acc = make_float2(0.f, 0.f), part = acc;
       auto exponentials = [&](uint32_t (&v)[32]) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const float2 t = f2_from_bits(v[2 * j], v[2 * j + 1]);
-          const float2 d = additive ? mul2(add2(t, splat2(-ref)), splat2(scale)) : fma2(t, splat2(scale), splat2(-r));
-          const float2 x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
-          acc = add2(acc, x);
+          float2 x;
+          if constexpr (additive) {
+            const float2 d = add2(t, splat2(-ref));
+            if ((poly >> j) & 1u) {
+              x = exp_poly2(d);
+            } else {
+              const float2 d2 = mul2(d, splat2(kLog2e));
+              x = make_float2(ex2_approx(d2.x), ex2_approx(d2.y));
+            }
+          } else {
+            const float2 d = fma2(t, splat2(scale), splat2(-r));
+            x = ((poly >> j) & 1u) ? ex2_poly2(d) : make_float2(ex2_approx(d.x), ex2_approx(d.y));
+          }
+          part = j % kGroup == 0 ? x : add2(part, x);
+          if (j % kGroup == kGroup - 1) acc = add2(acc, part);
           if constexpr (kKeep) {
             v[2 * j] = __float_as_uint(x.x);
             v[2 * j + 1] = __float_as_uint(x.y);
@@ -680,7 +697,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         scores(va, vb, c, grow);
         if constexpr (ADD) __syncwarp();  // every lane has read its row of the mask
         if (additive || far) take_off(va, vb, m_row);
-        constexpr uint32_t poly = Cfg::POLY_PAIRS;
+        constexpr uint32_t poly = additive ? 0u : Cfg::POLY_PAIRS;
         uint32_t pk[32];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
