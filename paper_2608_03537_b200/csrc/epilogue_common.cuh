@@ -19,11 +19,12 @@ struct MergeWelford {  // (mean, M2); pairwise update of Chan et al.
 struct MergeSum {  // (sum, unused)
   __device__ __forceinline__ float2 operator()(float2 a, float, float2 b, float) const { return make_float2(a.x + b.x, 0.f); }
 };
-struct MergeMaxSumExp2 {  // (max, sum of 2^(t - max)); a partial with max = -inf carries nothing
+struct MergeMaxSumExp2 {  // (max, sum of 2^(scale * (t - max))); a partial with max = -inf carries nothing
+  float scale;
   __device__ __forceinline__ float2 operator()(float2 a, float, float2 b, float) const {
     const float m = fmaxf(a.x, b.x);
-    const float fa = (a.x == -INFINITY) ? 0.f : ex2_approx(a.x - m);
-    const float fb = (b.x == -INFINITY) ? 0.f : ex2_approx(b.x - m);
+    const float fa = (a.x == -INFINITY) ? 0.f : ex2_approx(scale * (a.x - m));
+    const float fb = (b.x == -INFINITY) ? 0.f : ex2_approx(scale * (b.x - m));
     return make_float2(m, a.y * fa + b.y * fb);
   }
 };
@@ -147,13 +148,6 @@ __device__ __forceinline__ void load_mask_32(const uint16_t* seg, int valid, flo
 #pragma unroll
     for (int k = 0; k < 4; ++k) m2[4 * i + k] = bf16x2_to_f2(w4[k]);
   }
-}
-
-// The same as log2-domain addends, m * log2(e); -inf stays -inf.
-__device__ __forceinline__ void load_mask_log2_32(const uint16_t* seg, int valid, float2 (&m2)[16]) {
-  load_mask_32(seg, valid, m2);
-#pragma unroll
-  for (int i = 0; i < 16; ++i) m2[i] = mul2(m2[i], splat2(1.4426950408889634f));
 }
 
 __device__ __forceinline__ void store_chunk_bf16(uint16_t* dst, const uint32_t (&pk)[16]) {

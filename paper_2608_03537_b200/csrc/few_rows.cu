@@ -360,12 +360,14 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             for (int j = 0; j < 4; ++j) x[i][t][j] += o[j];
           }
       }
+    constexpr float kLog2e = 1.4426950408889634f;
     float pa[RC], pb[RC];  // (mean, M2), (sum of squares, unused) or (maximum, sum of exponentials) of this lane's columns
     if constexpr (EPI == EPI_SOFTMAX) {
-      // scores in the log2 domain; masked ones and the columns from N on are -inf
+      // masked scores and the columns from N on are -inf; log2 e comes behind the difference from the maximum, so that no mask
+      // value leaves the range of fp32
       const bool capped = p.softcap > 0.f;
-      const SoftcapLog2 cap_fn(alpha, capped ? p.softcap : 1.f);
-      const float sc = alpha * 1.4426950408889634f;
+      SoftcapLog2 cap_fn(alpha, capped ? p.softcap : 1.f);
+      cap_fn.c1 = p.softcap;
 #pragma unroll
       for (int i = 0; i < RC; ++i) {
         const int last = p.causal ? row0 + e + i * Cfg::kEpiWarps : p.N - 1;  // last live column of the row
@@ -373,11 +375,11 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
           float(&xx)[4] = x[i][t];
-          const float2 m01 = mul2(bf16x2_to_f2(res[i][t].x), splat2(1.4426950408889634f)), m23 = mul2(bf16x2_to_f2(res[i][t].y), splat2(1.4426950408889634f));
+          const float2 m01 = bf16x2_to_f2(res[i][t].x), m23 = bf16x2_to_f2(res[i][t].y);
           const float mk[4] = {m01.x, m01.y, m23.x, m23.y};
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            xx[j] = capped ? cap_fn(xx[j]) + mk[j] : fmaf(xx[j], sc, mk[j]);
+            xx[j] = capped ? cap_fn(xx[j]) + mk[j] : fmaf(xx[j], alpha, mk[j]);
             if (!in[t] || col[t] + j > last) xx[j] = -INFINITY;
             pa[i] = fmaxf(pa[i], xx[j]);
           }
@@ -393,7 +395,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         for (int t = 0; t < NT; ++t)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            x[i][t][j] = ex2_approx(x[i][t][j] - m);
+            x[i][t][j] = ex2_approx(kLog2e * (x[i][t][j] - m));
             pb[i] += x[i][t][j];
           }
       }
@@ -491,9 +493,9 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
 #pragma unroll
         for (int d = LPR / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) sq_l += o[k].y * (o[k].x == -INFINITY ? 0.f : ex2_approx(o[k].x - m));  // (a NaN stays one)
+        for (int k = 0; k < CPL; ++k) sq_l += o[k].y * (o[k].x == -INFINITY ? 0.f : ex2_approx(kLog2e * (o[k].x - m)));  // (a NaN stays one)
         const float own = r < rv ? s_stat[r * 16 + ct].x : -INFINITY;  // this CTA's exponentials are relative to its own maximum
-        mu_l = own == -INFINITY ? 0.f : ex2_approx(own - m);
+        mu_l = own == -INFINITY ? 0.f : ex2_approx(kLog2e * (own - m));
       } else {
 #pragma unroll
         for (int k = 0; k < CPL; ++k) sq_l += o[k].x;

@@ -1294,12 +1294,16 @@ COMFUSE_PROGRAM_LOOP
         }
 #undef COMFUSE_PROGRAM_LOOP
       } else {  // EPI_SOFTMAX
-        // log2 domain: t = Acc * (alpha * log2 e), so exp(x - m) = 2^(t - m_t)
-        // with a soft-cap the accumulators are mapped to capped log2-domain scores right after they are loaded, and sc = 1
+        // Exponentials are 2^(scale * (t - maximum)), t a score: the accumulator, or minus it where alpha is negative, and the scale
+        // |alpha| * log2 e; with a soft-cap the capped score in the log2 domain and 1; with a mask alpha * Acc (or the capped score) + mask
+        // and log2 e.  The difference comes first: it is an exact zero for the maximum whatever its size, and no mask value
+        // leaves the range of fp32.
         const bool capped = p.softcap > 0.f;
-        const SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
-        const float sc = capped ? 1.f : p.alpha * 1.4426950408889634f;
         const bool additive = p.mask != nullptr;  // additive mask tensor, applied behind the scale / soft-cap
+        SoftcapLog2 cap_fn(p.alpha, capped ? p.softcap : 1.f);
+        if (additive) cap_fn.c1 = p.softcap;
+        const float sc = capped ? 1.f : additive ? p.alpha : p.alpha >= 0.f ? 1.f : -1.f;
+        const float scale = additive ? 1.4426950408889634f : capped ? 1.f : fabsf(p.alpha) * 1.4426950408889634f;
         // The last live column of a row: the diagonal under the causal mask, and never beyond the row's end -- the
         // instantiation may be wider than the row (N = 1000 on the 1024-column form), columns from N on are masked.
         // Fragment classification, uniform over the warp's 32 rows so that the warp-wide TMEM loads stay convergent:
@@ -1311,9 +1315,11 @@ COMFUSE_PROGRAM_LOOP
         const int wlim_hi = p.causal ? (wrow0 + 31 < nlast ? wrow0 + 31 : nlast) : nlast;
         auto frag_state = [&](int col0) { return col0 + 31 <= wlim_lo ? 2 : (col0 > wlim_hi ? 0 : 1); };
         COMFUSE_TRACE_POINT();
+        // (The sub-tiles of the form without a cluster stay a loop: unrolled, both passes' values of both spill hundreds of registers, 64 x
+        // 512 x 512 behind K = 320 36.9 us instead of 29.5.)
         // ---------------- pass A: thread-local row max
         float mloc = -INFINITY;
-#pragma unroll
+#pragma unroll (CN == 1 ? 1 : ESUB)
         for (int sub = 0; sub < ESUB; ++sub) {
           wait_accumulator(sub);
           if (!live[sub]) continue;
@@ -1336,7 +1342,7 @@ COMFUSE_PROGRAM_LOOP
                 // a full-tensor operand of the epilogue (Sec. 5.2): t = score + mask, written back over the accumulator so
                 // that pass B finds it there
                 float2 m2[16];
-                load_mask_log2_32(p.mask + static_cast<long long>(grow) * p.N + col0, valid ? (p.N - col0 < 32 ? p.N - col0 : 32) : 0, m2);
+                load_mask_32(p.mask + static_cast<long long>(grow) * p.N + col0, valid ? (p.N - col0 < 32 ? p.N - col0 : 32) : 0, m2);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                   const float2 t01 = fma2(f2_from_bits(v[2 * j], v[2 * j + 1]), splat2(sc), m2[j]);
@@ -1347,11 +1353,17 @@ COMFUSE_PROGRAM_LOOP
                 }
                 tmem_st_32cols(tmem_of(sub) + g * 64 + half * 32, v);
               } else {
+                if (st == 2) {
 #pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                  const float t0 = __uint_as_float(v[j]) * sc, t1 = __uint_as_float(v[j + 1]) * sc;
-                  if (st == 2 || col0 + j <= rlim) m0v = fmaxf(m0v, t0);
-                  if (st == 2 || col0 + j + 1 <= rlim) m1v = fmaxf(m1v, t1);
+                  for (int j = 0; j < 32; j += 4) {
+                    const float2 t01 = mul2(f2_from_bits(v[j], v[j + 1]), splat2(sc)), t23 = mul2(f2_from_bits(v[j + 2], v[j + 3]), splat2(sc));
+                    m0v = max3(m0v, t01.x, t01.y);
+                    m1v = max3(m1v, t23.x, t23.y);
+                  }
+                } else {
+#pragma unroll
+                  for (int j = 0; j < 32; ++j)
+                    if (col0 + j <= rlim) m0v = fmaxf(m0v, __uint_as_float(v[j]) * sc);
                 }
               }
               mloc = fmaxf(mloc, fmaxf(m0v, m1v));
@@ -1360,10 +1372,10 @@ COMFUSE_PROGRAM_LOOP
         }
         if (additive) tmem_st_wait();
         COMFUSE_TRACE_POINT();
-        // ---------------- pass B: e = 2^(t - mloc), thread-local sum, e written back over the scores
+        // ---------------- pass B: e = 2^(scale * (t - mloc)), thread-local sum, e written back over the scores
         float lloc = 0.f;
         const float msub = (mloc == -INFINITY) ? 0.f : mloc;
-#pragma unroll
+#pragma unroll (CN == 1 ? 1 : ESUB)
         for (int sub = 0; sub < ESUB; ++sub) {
           if (!live[sub]) continue;
           const int W = unit_width(sub);
@@ -1381,10 +1393,10 @@ COMFUSE_PROGRAM_LOOP
                 for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(cap_fn(__uint_as_float(v[j])));
               }
               float s0 = 0.f, s1 = 0.f;
-              const float scb = additive ? 1.f : sc;  // with a mask tensor pass A has left t itself in the accumulator
+              const float scb = additive ? 1.f : sc;  // with a mask tensor pass A has left t itself in the accumulator; +-1
 #pragma unroll
               for (int j = 0; j < 32; j += 2) {
-                const float2 t01 = fma2(f2_from_bits(v[j], v[j + 1]), splat2(scb), splat2(-msub));
+                const float2 t01 = mul2(fma2(f2_from_bits(v[j], v[j + 1]), splat2(scb), splat2(-msub)), splat2(scale));
                 float e0 = ex2_approx(t01.x);
                 float e1 = ex2_approx(t01.y);
                 if (st != 2) {
@@ -1403,9 +1415,9 @@ COMFUSE_PROGRAM_LOOP
         }
         tmem_st_wait();
         COMFUSE_TRACE_POINT();
-        const float2 tot = cluster_row_reduce<CN, MergeMaxSumExp2, EPW>(make_float2(mloc, lloc), kThreadCount, MergeMaxSumExp2(), s_pre, s_stats,
+        const float2 tot = cluster_row_reduce<CN, MergeMaxSumExp2, EPW>(make_float2(mloc, lloc), kThreadCount, MergeMaxSumExp2{scale}, s_pre, s_stats,
                                                   bar_stats, row, h, crank, xpar, xphase, w, 2u, pm, p.leader_reduce != 0);
-        const float f = (mloc == -INFINITY || tot.y == 0.f) ? 0.f : ex2_approx(mloc - tot.x) / tot.y;
+        const float f = (mloc == -INFINITY || tot.y == 0.f) ? 0.f : ex2_approx(scale * (mloc - tot.x)) / tot.y;
         COMFUSE_TRACE_POINT();
         // ---------------- pass C: scale, round once, store (zeros where masked)
 #pragma unroll

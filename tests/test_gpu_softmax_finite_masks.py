@@ -1,6 +1,6 @@
-"""Additive masks whose masked entries are finite, from -1e4 to the lowest bf16, in the row softmax: masks that leave no live column to whole
-64-column groups (a causal mask, a window and a padding mask given as data) and to whole rows; and a window of scores far
-below the others without a mask.
+"""Additive masks whose masked entries are finite, from -1e4 to the lowest bf16, in each kernel that takes a mask: masks that leave no live column
+to whole 64-column groups (a causal mask, a window and a padding mask given as data) and to whole rows; and a window of scores
+far below the others without a mask.
 
 The reference adds score and mask in fp32, as every kernel does, and goes on in 64 bits: a row in which every score is masked with
 -1e9 or less has equal sums and so the probabilities 1/N, in 64 bits throughout it would have those of the unmasked scores."""
@@ -44,6 +44,23 @@ def test_row_kernel(batch, M, N, K, softcap, fill, cuda_device):
     check(batch, M, N, K, softcap, fill)
 
 
+# short and long contraction, rows that end inside the kernel's width
+CLUSTER = [(20, 130, 1000, 64), (12, 130, 2048, 320), (8, 300, 776, 320), (30, 130, 512, 768)]
+FEW = [(1, 40, 200, 64), (4, 64, 1000, 64), (2, 16, 512, 1024), (60, 20, 304, 64)]
+
+
+@pytest.mark.parametrize("fill", [-1e9, -1e30, LOWEST])
+@pytest.mark.parametrize("softcap", [0.0, 3.0])
+@pytest.mark.parametrize("batch,M,N,K", CLUSTER + FEW + [(8, 40, 4104, 320)])
+def test_other_kernels(batch, M, N, K, softcap, fill, cuda_device):
+    check(batch, M, N, K, softcap, fill)
+
+
+@pytest.mark.parametrize("fill", [-1e9, LOWEST])
+def test_unfused(fill, cuda_device):
+    check(3, 70, 504, 64, 0.0, fill, fused=False, tol=P.TOL_SOFTMAX_UNFUSED)
+
+
 def check(batch, M, N, K, softcap, fill, fused=True, tol=P.TOL_SOFTMAX_MAX):
     w = wl.scaled_masked_softmax(batch, M, N, K, seed=M + N, causal=False, softcap=softcap)
     w.tensors["mask"] = finite_mask(M, N, fill)
@@ -57,7 +74,8 @@ def check(batch, M, N, K, softcap, fill, fused=True, tol=P.TOL_SOFTMAX_MAX):
     assert (np.abs(dead - want) <= want * (2.0 ** -8 + (2.0 ** -9 if fill == -1e4 else 0.0))).all()
 
 
-@pytest.mark.parametrize("batch,M,N,causal,sign", [(40, 200, 504, False, 1), (36, 100, 1032, False, 1), (60, 504, 504, True, 1), (40, 200, 504, False, -1)])
+@pytest.mark.parametrize("batch,M,N,causal,sign", [(40, 200, 504, False, 1), (36, 100, 1032, False, 1), (60, 504, 504, True, 1), (40, 200, 504, False, -1),
+                                                   (20, 130, 1000, False, 1), (20, 1000, 1000, True, 1), (20, 130, 1000, False, -1), (2, 64, 504, False, 1)])
 @pytest.mark.parametrize("fill", [-1e4, -1e9, -1e10, -1e20, -1e30])
 def test_scores_far_below_the_others(batch, M, N, causal, sign, fill, cuda_device):
     # the mask folded into the contraction: its last element is 1 in A and, in B, the fill of the columns that are masked
@@ -65,7 +83,7 @@ def test_scores_far_below_the_others(batch, M, N, causal, sign, fill, cuda_devic
     w.scalars["alpha"] *= sign
     w.tensors["A"][:, :, 63] = wl.f32_to_bf16_bits(np.ones(1, np.float32))
     last = np.zeros(N, np.float32)
-    last[64:200] = fill * sign
+    last[64: 200 if N < 1000 else N - 200] = fill * sign  # (whole rows of what a thread holds in the cluster kernel)
     w.tensors["B"][:, 63, :] = wl.f32_to_bf16_bits(last)
     got = P.run_gpu(w, P.dev_tensors(w), fused=True)
     P.check_outputs(w, got, P.run_oracle(w), label=w.name)
