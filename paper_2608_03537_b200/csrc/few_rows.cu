@@ -35,7 +35,8 @@ struct FewRowsCfg {
   static constexpr int W_BYTES = NT * 128 * 64 * 2;         // weights of one K block
   static constexpr int X_BYTES = MT * 64 * 2;               // rows of one K block
   static constexpr int STAGE_BYTES = W_BYTES + X_BYTES;
-  static constexpr int PREFETCH_BLOCKS = 384 * 1024 / W_BYTES;  // 148 CTAs ask for less than half of the L2
+  // K blocks asked of the L2 ahead of the loads: under the set-up, and at most (148 CTAs: less than half of the L2)
+  static constexpr int ASK_FIRST = 128 * 1024 / W_BYTES, ASK_MOST = 384 * 1024 / W_BYTES;
   static constexpr int ROW_BYTES = NT * 128 * 4;            // one row of the CTA's columns, fp32
   static constexpr int RECV_BYTES = (MT + 7) * ROW_BYTES;   // partial sums of the CTA's row slice from up to 8 shares (8 * ceil(MT / 8) rows)
   static constexpr int STAT_BYTES = MT * 16 * 8;            // one exchange: up to 16 partials per row
@@ -47,12 +48,12 @@ struct FewRowsCfg {
   static constexpr int OFF_BAR = OFF_STAT + 2 * STAT_BYTES;
   static constexpr int NUM_BARS = 2 * NSTAGES + 4;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
-  static constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;
+  static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
   static constexpr int TMEM_COLS = NT * MT <= 32 ? 32 : NT * MT <= 64 ? 64 : 128;
   static_assert(MT % 16 == 0 && NT * MT <= 128, "UMMA shape and tensor memory");
   static_assert(STAGE_BYTES % 1024 == 0, "swizzled tiles start on 1024-byte boundaries");
   static_assert(MT * ROW_BYTES <= NSTAGES * STAGE_BYTES, "the accumulators are staged in the idle ring");
-  static_assert(NUM_BARS * 8 + 16 <= 256, "barrier room");
+  static_assert(NUM_BARS * 8 + 32 <= 256, "barrier room");
   static_assert(SMEM_BYTES <= 232448 && SMEM_BYTES > 116 * 1024, "one CTA per SM (tensor-memory allocation never waits)");
 };
 
@@ -111,6 +112,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + Cfg::OFF_MISC + 4);
   volatile int* s_told = s_abort + 1;    // a wait expired in some CTA of the cluster
   volatile int* s_issued = s_abort + 2;  // K blocks whose loads are issued (fewer than all where the producer's wait expires)
+  volatile int* s_begun = s_abort + 3;   // the previous kernel has ended
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -144,6 +146,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     mbar_init(bar_max, 1);
     *s_abort = 0;
     *s_told = 0;
+    *s_begun = 0;
     *s_issued = kb1 - kb0;
     fence_mbar_init();
     // what each exchange will deliver is known now: arm the barriers before any peer can send
@@ -153,18 +156,26 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmX);
   }
-  // The weights are asked of the L2 while the previous kernel still runs: a prefetch returns nothing, so it may stand in front of the
-  // wait whoever writes the weights (writes meet in the L2 too).  40 x 4096 x 4096, weights from memory: 13.1 -> 12.1 us, the
-  // finishing kernel of the call before now covers 33 MB of reads; in the L2 already: 10.7 both ways.  One row group asks.  Not where
-  // one kernel does it all: its successor's CTAs come too late for it to pay (48 x 960 x 3664 10.1 / 10.2, 69 x 3880 x 336 9.06 / 9.13
-  // with weights from memory, 10.2 / 10.4 and 9.0 / 9.1 from the L2).
-  if (p.wide && warp == 2 && grp == 0 && elect_one()) {
-    const int last = kb1 - kb0 < Cfg::PREFETCH_BLOCKS ? kb1 : kb0 + Cfg::PREFETCH_BLOCKS;
-    for (int kb = kb0; kb < last; ++kb)
+  // Two-kernel form: the weights are asked of the L2 while the previous kernel still runs (a prefetch returns nothing, so it may stand in
+  // front of the wait whoever writes the weights: writes meet in the L2 too), by one row group.  First as many blocks as the set-up covers, which
+  // a lone call gains from as well; then, while the previous kernel lasts, the others.  A request takes the time of a load: all of
+  // them under the set-up held back the loads of calls that had nothing to wait for.  Us a call, without / all under the set-up / this; queued
+  // with weights from memory, behind a kernel that lets no successor start early with weights from memory and from the L2:
+  //   40 x 4096 x 4096  13.1 / 12.4 / 12.1, 13.4 / 13.4 / 13.3, 11.3 / 12.2 / 11.3    4 x 4096 x 1024  7.7 / 7.2 / 7.1, 8.4 / 7.2 / 7.2, 7.2 / 7.2 / 7.2
+  //   16 x 2048 x 4096  9.4 / 8.6 / 8.5, 9.9 / 9.2 / 9.2, 9.2 / 9.2 / 9.2             40 x 2560 x 2048  10.1 / 9.5 / 9.7, 10.6 / 9.2 / 9.3, 9.2 / 9.2 / 9.2
+  //   16 x 8192 x 4096  19.7 / 20.5 / 19.5, 19.8 / 20.0 / 19.8, 15.4 / 17.4 / 15.4    33 x 2304 x 3584  10.7 / 10.0 / 10.0, 11.3 / 11.3 / 11.3, 10.1 / 11.3 / 10.4
+  // Queued with weights that are in the L2 already it costs about 1 % (40 x 4096 x 4096 10.7 / 10.8 / 10.9).  Long shares: half as many blocks (16 x
+  // 8192 x 4096, 64 blocks a share, 19.5 instead of 20.6, 16 x 6144 x 6144, 48 blocks, 18.4 / 18.6; 16 x 2048 x 8192, 32 blocks, 11.7 / 11.4).
+  // Not where one kernel does it all: its successor's CTAs come too late for it to pay (48 x 960 x 3664 10.1 / 10.2, 69 x 3880 x 336 9.06 /
+  // 9.13 with weights from memory, 10.2 / 10.4 and 9.0 / 9.1 from the L2).
+  auto ask = [&](int kb) {
 #pragma unroll
-      for (int j = 0; j < 2 * NT; ++j)
-        tma_prefetch_l2_3d(&tmW, p.b_nk ? kb * 64 : n0 + j * 64, p.b_nk ? n0 + j * 64 : kb * 64, b);
-  }
+    for (int j = 0; j < 2 * NT; ++j)
+      tma_prefetch_l2_3d(&tmW, p.b_nk ? kb * 64 : n0 + j * 64, p.b_nk ? n0 + j * 64 : kb * 64, b);
+  };
+  if (warp == 2 && p.wide && grp == 0 && elect_one())
+#pragma unroll 1
+    for (int kb = kb0; kb < kb1 && kb < kb0 + Cfg::ASK_FIRST; ++kb) ask(kb);
   if (warp == 1) {
     tmem_alloc(smem_u32(s_tmem_base), Cfg::TMEM_COLS);
     tmem_relinquish_alloc_permit();
@@ -174,7 +185,15 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   tcgen05_fence_after_sync();
   cluster_sync_after_init();  // every CTA's barriers exist and are armed before any peer signals them
   const uint32_t tmem_base = *s_tmem_base;
-  griddep_wait();  // the set-up above may overlap the previous kernel's tail; global memory is touched only below
+  if (warp == 2) {
+    if (p.wide && grp == 0 && elect_one()) {
+      const int most = kb1 - kb0 <= 32 ? Cfg::ASK_MOST : Cfg::ASK_MOST / 2;
+#pragma unroll 1
+      for (int kb = kb0 + Cfg::ASK_FIRST; kb < kb1 && kb < kb0 + most && !*s_begun; ++kb) ask(kb);
+    }
+    __syncwarp();
+  }
+  griddep_wait();  // what stands above may overlap the previous kernel's tail: nothing there writes global memory or takes a value from it
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
@@ -198,6 +217,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ UMMA issuer
     if (elect_one()) {
+      *s_begun = 1;
       int stage = 0;
       uint32_t phase = 0;
       // weights stored [N, K]: K-major, 16 elements = 32 bytes per step; stored [K, N]: MN-major (64-column blocks 8 KB
