@@ -10,8 +10,8 @@
 //   pass 0   for every live chunk:  S = A.B_chunk (UMMA, cta_group::2)  ->  online (max, sum) per thread; the exponentials of the
 //            last chunk stay in registers, those of the chunk before it in the chunk's accumulator slot (fp32 both)
 //   merge    the four threads that share a row combine their partials through shared memory
-//   result   the two kept chunks: exponential * 2^(m_thread - (max + log2 sum))  ->  bf16 box -> TMA store
-//   pass 1   for every other live chunk:  S again  ->  P = 2^(S*alpha*log2e - (max + log2 sum))  ->  bf16 box -> TMA store
+//   result   the two kept chunks: exponential * 2^((m_thread - max)*log2e - log2 sum)  ->  bf16 box -> TMA store
+//   pass 1   for every other live chunk:  S again  ->  P = 2^((t - max)*log2e - log2 sum), t = alpha*S + mask  ->  bf16 box -> TMA store
 //
 // Clusters are pairs, so all SMs are used (wider clusters leave SMs idle), any N fits, and the accumulator slots
 // alternate so that the UMMAs of chunk u+1 run under the epilogue of chunk u.  Rows of up to 512 columns are computed and
@@ -20,9 +20,9 @@
 //
 // What bounds it: the exponentials (MUFU: 16 results per clock and SM; a pass over 64 x 32 scores of all sixteen warps takes
 // 1640 clocks in a loop of its own) and, where the output outgrows the L2, the writes.  64 x 2048 x 2048 causal, K = 64 (537 MB
-// written, 85 us at the best rate of any store pattern measured here): 122.5 -> 115.2 us, without its stores 99 -> 76.  A thread
+// written, 85 us at the best rate of any store pattern measured here): 122.5 -> 115.2 us, without its stores 99 -> 75.  A thread
 // holds all its 64 columns of a chunk, so the accumulator is handed back before the arithmetic, which needs the registers that
-// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 34.3 -> 28.4 us a call; thirty shapes drawn from
+// the control warps give up (setmaxnreg: 112 instead of 96).  96 x 504 x 504 with a mask 34.3 -> 28.3 us a call; thirty shapes drawn from
 // 16 .. 2048 rows and 64 .. 2048 columns 0.995 .. 1.49 times as fast (geometric mean 1.16).  A kernel without a soft-cap carries no code for one:
 // a CTA runs through a few tiles only, and the first one waits for every line of code it is the first to reach (96 x 504 x 504 29.1 / 28.2).
 //
