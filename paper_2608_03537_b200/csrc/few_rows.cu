@@ -161,10 +161,10 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   // a lone call gains from as well; then, while the previous kernel lasts, the others.  A request takes the time of a load: all of
   // them under the set-up held back the loads of calls that had nothing to wait for.  Us a call, without / all under the set-up / this; queued
   // with weights from memory, behind a kernel that lets no successor start early with weights from memory and from the L2:
-  //   40 x 4096 x 4096  13.1 / 12.4 / 12.1, 13.4 / 13.4 / 13.3, 11.3 / 12.2 / 11.3    4 x 4096 x 1024  7.7 / 7.2 / 7.1, 8.4 / 7.2 / 7.2, 7.2 / 7.2 / 7.2
-  //   16 x 2048 x 4096  9.4 / 8.6 / 8.5, 9.9 / 9.2 / 9.2, 9.2 / 9.2 / 9.2             40 x 2560 x 2048  10.1 / 9.5 / 9.7, 10.6 / 9.2 / 9.3, 9.2 / 9.2 / 9.2
-  //   16 x 8192 x 4096  19.7 / 20.5 / 19.5, 19.8 / 20.0 / 19.8, 15.4 / 17.4 / 15.4    33 x 2304 x 3584  10.7 / 10.0 / 10.0, 11.3 / 11.3 / 11.3, 10.1 / 11.3 / 10.4
-  // Queued with weights that are in the L2 already it costs about 1 % (40 x 4096 x 4096 10.7 / 10.8 / 10.9).  Long shares: half as many blocks (16 x
+  //   40 x 4096 x 4096  13.1 / 12.4 / 12.0, 13.4 / 13.4 / 13.3, 11.3 / 12.2 / 11.3    4 x 4096 x 1024  7.7 / 7.2 / 7.0, 8.4 / 7.2 / 7.2, 7.2 / 7.2 / 7.2
+  //   16 x 2048 x 4096  9.4 / 8.6 / 8.4, 9.9 / 9.2 / 9.2, 9.2 / 9.2 / 9.2             40 x 2560 x 2048  10.1 / 9.5 / 9.6, 10.6 / 9.2 / 9.3, 9.2 / 9.2 / 9.2
+  //   16 x 8192 x 4096  19.7 / 20.5 / 19.5, 19.8 / 20.0 / 19.8, 15.4 / 17.4 / 15.4    33 x 2304 x 3584  10.7 / 10.0 / 9.9, 11.3 / 11.3 / 11.3, 10.1 / 11.3 / 10.3
+  // Queued with weights that are in the L2 already: level (40 x 4096 x 4096 10.7 / 10.8 / 10.7, 40 x 4096 x 1024 9.0 / 9.1 / 9.0).  Long shares: half as many blocks (16 x
   // 8192 x 4096, 64 blocks a share, 19.5 instead of 20.6, 16 x 6144 x 6144, 48 blocks, 18.4 / 18.6; 16 x 2048 x 8192, 32 blocks, 11.7 / 11.4).
   // Not where one kernel does it all: its successor's CTAs come too late for it to pay (48 x 960 x 3664 10.1 / 10.2, 69 x 3880 x 336 9.06 /
   // 9.13 with weights from memory, 10.2 / 10.4 and 9.0 / 9.1 from the L2).
@@ -173,9 +173,10 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     for (int j = 0; j < 2 * NT; ++j)
       tma_prefetch_l2_3d(&tmW, p.b_nk ? kb * 64 : n0 + j * 64, p.b_nk ? n0 + j * 64 : kb * 64, b);
   };
-  if (warp == 2 && p.wide && grp == 0 && elect_one())
+  if (warp == 2 && p.wide && grp == 0 && elect_one()) {
 #pragma unroll 1
     for (int kb = kb0; kb < kb1 && kb < kb0 + Cfg::ASK_FIRST; ++kb) ask(kb);
+  }
   if (warp == 1) {
     tmem_alloc(smem_u32(s_tmem_base), Cfg::TMEM_COLS);
     tmem_relinquish_alloc_permit();
@@ -185,18 +186,12 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
   tcgen05_fence_after_sync();
   cluster_sync_after_init();  // every CTA's barriers exist and are armed before any peer signals them
   const uint32_t tmem_base = *s_tmem_base;
-  if (warp == 2) {
-    if (p.wide && grp == 0 && elect_one()) {
-      const int most = kb1 - kb0 <= 32 ? Cfg::ASK_MOST : Cfg::ASK_MOST / 2;
-#pragma unroll 1
-      for (int kb = kb0 + Cfg::ASK_FIRST; kb < kb1 && kb < kb0 + most && !*s_begun; ++kb) ask(kb);
-    }
-    __syncwarp();
-  }
-  griddep_wait();  // what stands above may overlap the previous kernel's tail: nothing there writes global memory or takes a value from it
+  // What stands above may overlap the previous kernel's tail: nothing there writes global memory or takes a value from it.  Each role waits for
+  // itself (behind one wait for all 40 x 4096 x 1024 9.2 / 9.4 us, 100 x 2048 x 2048 9.3 / 9.5).
 
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
+    griddep_wait();
     if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
@@ -216,6 +211,7 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ UMMA issuer
+    griddep_wait();
     if (elect_one()) {
       *s_begun = 1;
       int stage = 0;
@@ -247,6 +243,15 @@ few_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
     }
   } else {
     // ------------------------------------------------------------------------------------------ epilogue warps
+    if (warp == 2) {
+      if (p.wide && grp == 0 && elect_one()) {
+        const int most = kb1 - kb0 <= 32 ? Cfg::ASK_MOST : Cfg::ASK_MOST / 2;
+#pragma unroll 1
+        for (int kb = kb0 + Cfg::ASK_FIRST; kb < kb1 && kb < kb0 + most && !*s_begun; ++kb) ask(kb);
+      }
+      __syncwarp();
+    }
+    griddep_wait();
     const int e = warp - 2;
     const int q = warp & 3;  // TMEM lane quarter: columns 32q .. 32q+31 of each 128-column tile
     const int h = e >> 2;    // which rows of the tile this warp moves from tensor memory to shared memory
